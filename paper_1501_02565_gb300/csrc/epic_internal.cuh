@@ -95,6 +95,7 @@ __host__ __device__ __forceinline__ int unit_shift_of(unsigned cmax_bits, int re
     const float ext = r * (float)(tw > th ? tw : th) + 0.41421357f * r * (float)(tw < th ? tw : th);
     const float dbound = cmax * ext * 1.001f + 1e-3f;
     int s = 0;
+    if (cmax < 2.f && dbound < 1024.f) return 0;
     while (s < MAX_UNIT_SHIFT && (cmax >= ldexpf(2.f, s) || dbound >= ldexpf(1024.f, s))) ++s;
     return s;
 }
@@ -128,6 +129,7 @@ struct PairDev {
     int sweep;              // relaxation schedule: 0 segmented lines, 1 whole lines
                             // (k_dt.cu); 2 row-closure passes on warp tiles (k_relax.cu)
     int tiles_x, tiles_y;
+    int stack;              // warp tiles: tiles of a column solved as one (1 or 2)
     int hash_cap;           // power of two
     int flow_vec_ok;        // flow pointer is 16-byte aligned
     pkey_t *keys;            // [H*W] packed (D, L)
@@ -172,31 +174,31 @@ struct PairDev {
     int tma_bw_fresh, tma_bw_again;
     CUtensorMap tm_cost_fresh;
     CUtensorMap tm_cost_again;
-    // TMA staging of the warp tiles (k_relax.cu; tma_warp = 0: plain loads):
-    // boxes of the keys (u64, 68 x (tile_h + 2) from x0 - 2) and of the
-    // costs (float32, 72 x (tile_h + 2) from x0 - 4), tile and ring
-    int tma_warp;
     // written on the device by the prepare kernel (zero from the host): the
     // float bits of the pair's largest cost and the tile-step reach of its
     // seeds, from which unit_shift() derives the distance unit
     unsigned cmax_bits;
     int seed_reach;
-    CUtensorMap tm_warp_keys;
-    CUtensorMap tm_warp_cost;
 };
 
 // The distance unit shift of a pair (0 for the sweep schedules of k_dt.cu,
 // which keep the unit 2^-31).
 __device__ __forceinline__ int unit_shift(const PairDev &P) {
     return P.sweep == SWEEP_WARP
-               ? unit_shift_of(*(volatile const unsigned *)&P.cmax_bits,
-                               *(volatile const int *)&P.seed_reach, P.tile_w, P.tile_h)
+               ? unit_shift_of(P.cmax_bits, P.seed_reach, P.tile_w, P.tile_h)
                : 0;
 }
 
 struct GridBarrier {
     unsigned count;
     unsigned gen;
+};
+
+// Requests for tile solves that are not answered yet, and solves done (see
+// own_tiles in relax_tiles.cuh).
+struct TileWork {
+    int open;
+    unsigned solves;
 };
 
 // Counters that live in the arena for the whole handle.
@@ -211,11 +213,8 @@ struct RunState {
     unsigned edge_next;    // boundary-edge tile dispenser
     unsigned wl_count[3];  // worklist lengths of the chunked relaxation passes (rotating)
     unsigned compact_done; // CTAs finished in the pruning compaction
-    // the warp-tile relaxation's work queue (phase 2): tickets taken, items
-    // pushed, items pushed or held but not finished, items taken
-    unsigned q_head, q_tail;
-    int q_busy;
-    unsigned q_items;
+    TileWork tiles[2];     // the warp-tile relaxation's: distances, then labels
+    unsigned fresh_done;   // tiles that phase 1 of the distances has written
     GridBarrier barrier;
 };
 
@@ -228,15 +227,17 @@ struct BatchArgs {
     const int *chunk_base;   // [npairs+1] prefix of write-out chunks
     const int *hash_base;    // [npairs+1] prefix of hash slots
     const int *clear_base;   // [npairs+1] prefix of clear chunks
+    const int *solve_base;   // [npairs+1] prefix of the warp-tile relaxation's solve tiles
+    int total_solve;
     int total_tiles, total_matches, total_chunks, total_hash, total_clear;
     int uniform_tiles;       // > 0: every pair has this many tiles (pair = tile / uniform_tiles)
     int *wl;                 // chunked relaxation only: 3 worklists of total_tiles flat tile indices
     int *wl_queued;          // [total_tiles] last pass + 1 a tile was queued for (0 = never)
     int max_degree;
     int knn_hs, knn_fs, knn_kmax;  // main-pass K-NN table sizes per warp, and K bound
-    int *relax_queue;      // [total_tiles] warp-tile relaxation work queue (-1 = empty slot);
-                           // null for runs of the apron-tile relaxation
-    int *relax_queued;     // [total_tiles] per-tile queue state (see k_relax.cu)
+    unsigned *relax_req;   // [2][total_solve] warp-tile relaxation: requests for a solve of
+                           // each tile (distances, labels); null for runs of the apron-tile
+                           // relaxation
     int *knn_retry_list;   // global match indices to search again; holds every match of
                            // the batch (a match is queued at most once per pass)
     int max_passes;
@@ -288,8 +289,8 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 
 // Sense-free generation barrier over all CTAs of a cooperative launch.  The
-// wait gives up after BARRIER_LIMIT_NS (or as soon as another CTA has given
-// up) and reports EPIC_ERR_TIMEOUT instead of spinning forever.
+// wait gives up after BARRIER_LIMIT_NS (or as soon as the run has recorded an
+// error: other CTAs may have left) and reports EPIC_ERR_TIMEOUT instead of spinning forever.
 static __device__ __noinline__ bool grid_sync(RunState *st, unsigned nblocks,
                           unsigned long long limit_ns = BARRIER_LIMIT_NS) {
     __shared__ int s_ok;
@@ -307,7 +308,7 @@ static __device__ __noinline__ bool grid_sync(RunState *st, unsigned nblocks,
         } else {
             unsigned long long t0 = global_ns();
             while (ld_acquire(&b->gen) == g) {
-                if (get_status(st) == EPIC_ERR_TIMEOUT) { ok = 0; break; }
+                if (get_status(st) != 0) { ok = 0; break; }
                 if (global_ns() - t0 > limit_ns) {
                     set_status(st, EPIC_ERR_TIMEOUT);
                     ok = 0;
@@ -398,10 +399,13 @@ cudaError_t launch_collect_edges(const PairDev *pair_host_copy, int *em,
                                  int *en, float *ew, int cap, int *count,
                                  cudaStream_t stream);
 size_t dt_smem_bytes(int tile_w, int tile_h, int apron);
-// The interpolator's relaxation on warp-owned tiles of 64 x tile_h pixels
-// (k_relax.cu); max_rows = the largest tile_h of the batch (<= 32).
+// The interpolator's relaxation on tiles of 64 x tile_h pixels (k_relax.cu);
+// max_rows = the rows of the batch's largest solve tile (<= 32).
 constexpr int RELAX_TILE_W = 64;
 constexpr int RELAX_MAX_ROWS = 32;
+// Tiles are solved in stacks of two (see solve_stack in epic_interp.cu) from
+// this many on.
+constexpr int RELAX_STACK_TILES = 1400;
 size_t relax_smem_bytes(int max_rows);
 cudaError_t launch_relax(const BatchArgs &a, const BatchArgs *dev, const LaunchCfg &lc,
                          int max_rows, bool fixed_grid, int *grid_used);

@@ -182,6 +182,17 @@ bool uses_warp_tiles(const epic_config_t &c, const std::vector<epic_tile_rule_t>
     return true;
 }
 
+// Relaxation tiles of a column that the warp-tile relaxation solves as one.  A
+// solve costs ~5 us beside its rounds however many pixels it holds (staging,
+// the fences and requests between tiles), so with enough tiles to fill the GPU
+// two 64 x 16 tiles at a time are faster (distances and settling of a
+// 2048 x 1024 pair, 2048 tiles: 249 -> 181 us; of 8 pruned 1024 x 436 pairs,
+// 3584 tiles: 1114 -> 860 us); with fewer, one at a time spreads over more SMs
+// (912 tiles are resident at once).
+int solve_stack(long long tiles, int max_th) {
+    return tiles >= epic::RELAX_STACK_TILES && 2 * max_th <= epic::RELAX_MAX_ROWS ? 2 : 1;
+}
+
 struct Layout {
     size_t keys, tile_start, tile_fill, tile_seeds, tile_stamp, hkeys, hw, deg, wmin, wmin2, wnear,
         row, adj, models,
@@ -249,6 +260,7 @@ PairDev make_pair_desc(const epic_config_t &c, const std::vector<epic_tile_rule_
                  uses_warp_tiles(c, rules));
     P.tiles_x = (d.W + P.tile_w - 1) / P.tile_w;
     P.tiles_y = (d.H + P.tile_h - 1) / P.tile_h;
+    P.stack = 1;
     P.hash_cap = std::max(1024, next_pow2(8LL * d.N));
     P.flow_vec_ok = ((uintptr_t)d.flow_out % 16) == 0;
     return P;
@@ -301,37 +313,6 @@ void encode_cost_maps(PairDev &P) {
     P.tma_bw_fresh = bw_f;
     P.tma_bw_again = bw_a;
     P.tma_cost = 1;
-}
-
-// Tensor maps of the warp-tile relaxation (k_relax.cu): the pair's keys as a
-// W x H array of 8-byte elements with boxes of 68 x (tile_h + 2), and its
-// cost map as float32 with boxes of 72 x (tile_h + 2); both boxes start at
-// an x coordinate that is a multiple of 64 minus 2 (keys) or 4 (costs), so
-// every copy starts on a 16-byte boundary.  Leaves tma_warp = 0 (plain
-// loads) unless both maps can be encoded: 16-byte-aligned bases and row
-// pitches that are multiples of 16 bytes (W even for the keys, W a multiple
-// of 4 for the costs).
-void encode_warp_maps(PairDev &P) {
-    P.tma_warp = 0;
-    if (P.sweep != SWEEP_WARP_TILES) return;
-    EncodeTiledFn fn = encode_tiled();
-    if (!fn || ((uintptr_t)P.C % 16) != 0 || ((uintptr_t)P.keys % 16) != 0 ||
-        ((size_t)P.W * 4) % 16 != 0 || P.tile_h + 2 > 256)
-        return;
-    const cuuint64_t dims[2] = {(cuuint64_t)P.W, (cuuint64_t)P.H};
-    const cuuint64_t kstr[1] = {(cuuint64_t)P.W * 8};
-    const cuuint64_t cstr[1] = {(cuuint64_t)P.W * 4};
-    const cuuint32_t estr[2] = {1, 1};
-    const cuuint32_t kbox[2] = {68u, (cuuint32_t)(P.tile_h + 2)};
-    const cuuint32_t cbox[2] = {72u, (cuuint32_t)(P.tile_h + 2)};
-    if (fn(&P.tm_warp_keys, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, P.keys, dims, kstr, kbox, estr,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
-        fn(&P.tm_warp_cost, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(P.C), dims,
-           cstr, cbox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return;
-    P.tma_warp = 1;
 }
 
 int validate(epic_interp_t *h, const epic_pair_desc_t &d, int i) {
@@ -576,17 +557,17 @@ int epic_interp_run_batch(epic_interp_t *h, const epic_pair_desc_t *descs, int n
     // queued at most once per pass
     const size_t retry_off = align_up(off, 256);
     off = retry_off + sizeof(int) * total_N;
-    // the relaxation's work queue and queued flags: one slot each per tile
+    // the relaxation's requests: two counts per tile (distances, labels)
     size_t total_T = 0;
     for (int i = 0; i < n; ++i) total_T += (size_t)P[i].tiles_x * P[i].tiles_y;
     const size_t rq_off = align_up(off, 256);
-    off = rq_off + 2 * sizeof(int) * total_T;
+    off = rq_off + 2 * sizeof(unsigned) * total_T;
     if (max_K > EPIC_MAX_K)
         return fail(h, EPIC_ERR_INVALID, "K (clamped to N) above EPIC_MAX_K");
     int rc = ensure_arena(h, off);
     if (rc) return rc;
     for (int i = 0; i < n; ++i) {
-        encode_cost_maps(P[i]);
+        if (P[i].sweep != SWEEP_WARP_TILES) encode_cost_maps(P[i]);
         char *b = h->arena;
         P[i].keys = reinterpret_cast<pkey_t *>(b + L[i].keys);
         P[i].tile_start = reinterpret_cast<int *>(b + L[i].tile_start);
@@ -609,44 +590,12 @@ int epic_interp_run_batch(epic_interp_t *h, const epic_pair_desc_t *descs, int n
             P[i].knn_count = reinterpret_cast<int *>(b + L[i].knn_count);
         }
         P[i].info = reinterpret_cast<int *>(b + L[i].info);
-        encode_warp_maps(P[i]);
         if (c.prune) {
             P[i].keep = reinterpret_cast<int *>(b + L[i].keep);
             P[i].pruned = reinterpret_cast<float4 *>(b + L[i].pruned);
             P[i].kept_index = reinterpret_cast<int *>(b + L[i].kept_index);
         }
     }
-    // batch table: BatchArgs, PairDev[n], then 5 prefix arrays of n+1 ints
-    std::vector<int> tile_base(n + 1), match_base(n + 1), chunk_base(n + 1),
-        hash_base(n + 1), clear_base(n + 1);
-    long long tt = 0, tm = 0, tc = 0, th = 0, tcl = 0;
-    for (int i = 0; i < n; ++i) {
-        tile_base[i] = (int)tt;
-        match_base[i] = (int)tm;
-        chunk_base[i] = (int)tc;
-        hash_base[i] = (int)th;
-        clear_base[i] = (int)tcl;
-        tt += (long long)P[i].tiles_x * P[i].tiles_y;
-        tm += P[i].N;
-        tc += ((long long)P[i].H * P[i].W + epic::WRITEOUT_CHUNK - 1) / epic::WRITEOUT_CHUNK;
-        th += P[i].hash_cap;
-        tcl += ((long long)P[i].hash_cap + epic::CLEAR_CHUNK - 1) / epic::CLEAR_CHUNK;
-    }
-    if (tt > INT32_MAX || tm > INT32_MAX || tc > INT32_MAX || th > INT32_MAX || tcl > INT32_MAX)
-        return fail(h, EPIC_ERR_INVALID, "batch too large");
-    tile_base[n] = (int)tt;
-    match_base[n] = (int)tm;
-    chunk_base[n] = (int)tc;
-    hash_base[n] = (int)th;
-    clear_base[n] = (int)tcl;
-    const size_t args_bytes = align_up(sizeof(BatchArgs), 256);
-    const size_t pd_bytes = align_up(sizeof(PairDev) * n, 256);
-    const size_t pre_bytes = sizeof(int) * (n + 1);
-    const size_t pre_stride = align_up(pre_bytes, 256);
-    const size_t table_bytes = args_bytes + pd_bytes + 5 * pre_stride;
-    rc = ensure_table(h, table_bytes);
-    if (rc) return rc;
-
     // graph replay applies when the launch shapes chosen below do not depend
     // on this batch: kernel sizes from the configured maxima
     // graph launches size the relaxation's shared memory for the largest
@@ -675,6 +624,49 @@ int epic_interp_run_batch(epic_interp_t *h, const epic_pair_desc_t *descs, int n
     const int knn_K = graph ? cfg_K : max_K;
     const int dt_tw = graph ? cfg_tw : max_tw, dt_th = graph ? cfg_th : max_th;
     const int dt_ap = graph ? cfg_ap : max_ap;
+    // a captured sequence keeps the choice of the configured batch
+    int stack = 1;
+    if (warp_tiles) {
+        const long long cfg_tiles = (long long)std::max(1, c.max_pairs) *
+                                    ((std::max(1, c.max_W) + epic::RELAX_TILE_W - 1) / epic::RELAX_TILE_W) *
+                                    ((std::max(1, c.max_H) + cfg_th - 1) / cfg_th);
+        stack = graph ? solve_stack(cfg_tiles, cfg_th) : solve_stack((long long)total_T, max_th);
+    }
+
+    // batch table: BatchArgs, PairDev[n], then 6 prefix arrays of n+1 ints
+    std::vector<int> tile_base(n + 1), match_base(n + 1), chunk_base(n + 1),
+        hash_base(n + 1), clear_base(n + 1), solve_base(n + 1);
+    long long tt = 0, tm = 0, tc = 0, th = 0, tcl = 0, ts = 0;
+    for (int i = 0; i < n; ++i) {
+        tile_base[i] = (int)tt;
+        match_base[i] = (int)tm;
+        chunk_base[i] = (int)tc;
+        hash_base[i] = (int)th;
+        clear_base[i] = (int)tcl;
+        solve_base[i] = (int)ts;
+        P[i].stack = stack;
+        ts += (long long)P[i].tiles_x * ((P[i].tiles_y + stack - 1) / stack);
+        tt += (long long)P[i].tiles_x * P[i].tiles_y;
+        tm += P[i].N;
+        tc += ((long long)P[i].H * P[i].W + epic::WRITEOUT_CHUNK - 1) / epic::WRITEOUT_CHUNK;
+        th += P[i].hash_cap;
+        tcl += ((long long)P[i].hash_cap + epic::CLEAR_CHUNK - 1) / epic::CLEAR_CHUNK;
+    }
+    if (tt > INT32_MAX || tm > INT32_MAX || tc > INT32_MAX || th > INT32_MAX || tcl > INT32_MAX)
+        return fail(h, EPIC_ERR_INVALID, "batch too large");
+    tile_base[n] = (int)tt;
+    match_base[n] = (int)tm;
+    chunk_base[n] = (int)tc;
+    hash_base[n] = (int)th;
+    clear_base[n] = (int)tcl;
+    solve_base[n] = (int)ts;
+    const size_t args_bytes = align_up(sizeof(BatchArgs), 256);
+    const size_t pd_bytes = align_up(sizeof(PairDev) * n, 256);
+    const size_t pre_bytes = sizeof(int) * (n + 1);
+    const size_t pre_stride = align_up(pre_bytes, 256);
+    const size_t table_bytes = args_bytes + pd_bytes + 6 * pre_stride;
+    rc = ensure_table(h, table_bytes);
+    if (rc) return rc;
 
     Handle::Slot &sl = h->slot[h->next_slot];
     h->next_slot ^= 1;
@@ -694,6 +686,8 @@ int epic_interp_run_batch(epic_interp_t *h, const epic_pair_desc_t *descs, int n
     a.chunk_base = pre_dev(2);
     a.hash_base = pre_dev(3);
     a.clear_base = pre_dev(4);
+    a.solve_base = pre_dev(5);
+    a.total_solve = (int)ts;
     a.total_tiles = (int)tt;
     a.total_matches = (int)tm;
     a.total_chunks = (int)tc;
@@ -705,8 +699,7 @@ int epic_interp_run_batch(epic_interp_t *h, const epic_pair_desc_t *descs, int n
     epic::knn_table_sizes(knn_K, size_lc, &a.knn_hs, &a.knn_fs);
     a.knn_kmax = knn_K;
     a.knn_retry_list = reinterpret_cast<int *>(h->arena + retry_off);
-    a.relax_queue = reinterpret_cast<int *>(h->arena + rq_off);
-    a.relax_queued = a.relax_queue + total_T;
+    a.relax_req = reinterpret_cast<unsigned *>(h->arena + rq_off);
     a.max_passes = c.max_passes;
     a.weight_squared = c.weight_squared ? 1 : 0;
     a.fallback_eps = c.fallback_eps;
@@ -717,23 +710,23 @@ int epic_interp_run_batch(epic_interp_t *h, const epic_pair_desc_t *descs, int n
     a.state = h->state;
     if (epic::knn_warps_per_cta(knn_K, size_lc) < 1)
         return fail(h, EPIC_ERR_INVALID, "K too large for the per-warp search tables");
-    if ((warp_tiles ? epic::relax_smem_bytes(dt_th) : epic::dt_smem_bytes(dt_tw, dt_th, dt_ap)) >
+    if ((warp_tiles ? epic::relax_smem_bytes(stack * dt_th) : epic::dt_smem_bytes(dt_tw, dt_th, dt_ap)) >
         (size_t)h->smem_optin)
         return fail(h, EPIC_ERR_INVALID, "relaxation tile does not fit in shared memory");
 
     char *hs = sl.host;
     memcpy(hs, &a, sizeof(BatchArgs));
     memcpy(hs + args_bytes, P.data(), sizeof(PairDev) * n);
-    const int *pres[5] = {tile_base.data(), match_base.data(), chunk_base.data(),
-                          hash_base.data(), clear_base.data()};
-    for (int k = 0; k < 5; ++k) memcpy(hs + args_bytes + pd_bytes + k * pre_stride, pres[k], pre_bytes);
+    const int *pres[6] = {tile_base.data(), match_base.data(), chunk_base.data(),
+                          hash_base.data(), clear_base.data(), solve_base.data()};
+    for (int k = 0; k < 6; ++k) memcpy(hs + args_bytes + pd_bytes + k * pre_stride, pres[k], pre_bytes);
     const BatchArgs *dev_a = reinterpret_cast<const BatchArgs *>(sl.dev);
 
     epic::LaunchCfg lc{h->num_sms, h->smem_optin, stream, h->smem_per_sm, h->smem_reserved};
     BatchArgs *dev_rw = reinterpret_cast<BatchArgs *>(sl.dev);
     auto relax = [&]() -> cudaError_t {
-        return warp_tiles ? epic::launch_relax(a, dev_a, lc, dt_th, graph, nullptr)
-                          : epic::launch_dt(a, dev_a, lc, dt_tw, dt_th, dt_ap, graph, nullptr);
+        if (!warp_tiles) return epic::launch_dt(a, dev_a, lc, dt_tw, dt_th, dt_ap, graph, nullptr);
+        return epic::launch_relax(a, dev_a, lc, stack * dt_th, graph, nullptr);
     };
     const bool prune = c.prune != 0;
     // ev (timing only): a start and an end event per stage
@@ -1522,11 +1515,11 @@ int epic_interp_request_bytes(const epic_interp_t *h, const epic_config_t *cfg, 
     const PairDev P = make_pair_desc(c, h ? h->rules : no_rules, d);
     // the pair's arena regions (each 256-byte aligned, so a pair placed after
     // any other needs at most its aligned size), its K-NN retry-list slots
-    // and its tiles' slots in the relaxation's work queue and queued flags
+    // and its tiles' request counts of the relaxation
     const size_t per = layout_pair(0, P, c.max_degree, c.keep_intermediates != 0,
                                    c.prune != 0).end;
     *bytes = (long long)(per + sizeof(int) * (size_t)N +
-                         2 * sizeof(int) * (size_t)P.tiles_x * P.tiles_y);
+                         2 * sizeof(unsigned) * (size_t)P.tiles_x * P.tiles_y);
     return EPIC_OK;
 }
 

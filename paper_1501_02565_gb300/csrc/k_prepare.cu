@@ -171,18 +171,17 @@ __global__ void __launch_bounds__(1024) prepare_kernel(const BatchArgs *__restri
         st->wl_count[0] = st->wl_count[1] = st->wl_count[2] = 0;
         st->barrier.count = 0;
         st->compact_done = 0;
-        st->q_head = st->q_tail = st->q_items = 0;
-        st->q_busy = a.total_tiles;   // the initial sweep's items
+        st->fresh_done = 0;
+        for (TileWork &w : st->tiles) {
+            w.open = a.total_solve;   // the first solve of every tile
+            w.solves = 0;
+        }
     }
-    // the warp-tile relaxation's work queue: empty slots; every tile counts
-    // as queued until the sweep of phase 2 takes it.  Runs of the apron-tile
-    // relaxation (the exact variant's, the no-allocation entry point's) have
-    // no queue.
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; a.relax_queue && i < a.total_tiles;
-         i += gridDim.x * blockDim.x) {
-        a.relax_queue[i] = -1;
-        a.relax_queued[i] = 1;
-    }
+    // the warp-tile relaxation's requests: one for the first solve of every
+    // tile.  Runs of the apron-tile relaxation (the exact variant's) have none.
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; a.relax_req && i < 2 * a.total_solve;
+         i += gridDim.x * blockDim.x)
+        a.relax_req[i] = 1;
     // seed binning: one CTA per pair at a time
     for (int p = blockIdx.x; p < a.npairs; p += gridDim.x) {
         const PairDev &P = a.pairs[p];
