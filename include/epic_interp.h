@@ -131,13 +131,14 @@ typedef struct {
                              every installed rule ask for them; otherwise a
                              frame whose rule says 2 gets 64 x 32 tiles with
                              apron 4 and schedule 0.  The exact variant's
-                             single-source runs always use schedule 0 or 1.
+                             cap map always uses schedule 0 or 1.
                              Every schedule gives the same result. */
     long long exact_chunk_bytes; /* epic_exact_interp with metric 0: device
                              bytes of packed keys its single-source
                              relaxations may hold at once (8 bytes per pixel
-                             per match); the matches run in chunks of
-                             max(1, min(N, exact_chunk_bytes / (8 H W))).
+                             per match); at most
+                             max(1, min(N, exact_chunk_bytes / (8 H W)))
+                             matches run at a time.
                              0 = 1 GiB (default).  Only speed and memory
                              depend on it, never the results. */
 } epic_config_t;
@@ -318,9 +319,11 @@ int epic_interp_get_stage_times(epic_interp_t *h, float *ms_out, int n_stages,
  * knn_dist_out [H*W*K] float32 receive every pixel's list in key order (both
  * NULL, or both set).  K is clamped to N and limited by shared memory
  * (K * 512 bytes per 64 pixels; K <= 448 on GB300).  With metric 0 the
- * handle holds N * H * W * 4 bytes of distances plus up to
- * exact_chunk_bytes (1 GiB by default) of relaxation keys (grown on demand,
- * EPIC_ERR_OOM if it cannot be).  Runs
+ * handle holds up to exact_chunk_bytes (1 GiB by default) of relaxation keys
+ * and the distances of the 64 x 32 tiles that each match reaches within the
+ * bounds (8 KiB a tile; room for 16 per match to begin with, grown on demand,
+ * at most N * H * W * 4 bytes and the padding of edge tiles; EPIC_ERR_OOM if
+ * it cannot be).  Runs
  * on `stream` and waits for completion; returns the device status. */
 int epic_exact_interp(epic_interp_t *h, const float *cost_map,
                       const float *matches, int H, int W, int N, int K,

@@ -133,11 +133,9 @@ struct PairDev {
     int hash_cap;           // power of two
     int flow_vec_ok;        // flow pointer is 16-byte aligned
     pkey_t *keys;            // [H*W] packed (D, L)
-    // exact variant only (null elsewhere): a distance offset per seed (units),
-    // and a key map whose distances cap the keys written back (a pixel whose
-    // distance exceeds its cap is left unreached)
+    // cap map of the exact variant only (null elsewhere): a distance offset
+    // per seed (units)
     const unsigned long long *seed_init;   // [N]
-    const pkey_t *cap;                     // [H*W]
     int *tile_start;        // [tiles+1] seed bins (prefix offsets)
     int *tile_fill;         // [tiles] scatter cursors
     int *tile_seeds;        // [N] match indices grouped by tile
@@ -211,7 +209,6 @@ struct RunState {
     unsigned knn_overflow; // matches whose search outgrew the small tables
     unsigned knn_retry;    // dispenser of the retry pass over those matches
     unsigned edge_next;    // boundary-edge tile dispenser
-    unsigned wl_count[3];  // worklist lengths of the chunked relaxation passes (rotating)
     unsigned compact_done; // CTAs finished in the pruning compaction
     TileWork tiles[2];     // the warp-tile relaxation's: distances, then labels
     unsigned fresh_done;   // tiles that phase 1 of the distances has written
@@ -230,9 +227,6 @@ struct BatchArgs {
     const int *solve_base;   // [npairs+1] prefix of the warp-tile relaxation's solve tiles
     int total_solve;
     int total_tiles, total_matches, total_chunks, total_hash, total_clear;
-    int uniform_tiles;       // > 0: every pair has this many tiles (pair = tile / uniform_tiles)
-    int *wl;                 // chunked relaxation only: 3 worklists of total_tiles flat tile indices
-    int *wl_queued;          // [total_tiles] last pass + 1 a tile was queued for (0 = never)
     int max_degree;
     int knn_hs, knn_fs, knn_kmax;  // main-pass K-NN table sizes per warp, and K bound
     unsigned *relax_req;   // [2][total_solve] warp-tile relaxation: requests for a solve of
@@ -272,7 +266,6 @@ __device__ __forceinline__ int get_status(const RunState *s) {
 // Bounded grid barrier of the cooperative relaxation launches.
 // ---------------------------------------------------------------------------
 constexpr unsigned long long BARRIER_LIMIT_NS = 2000000000ull;  // 2 s
-constexpr int PASS_CHUNK = 8;  // tiles per dispenser step in chunked verification passes
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
     unsigned v;
@@ -343,11 +336,9 @@ struct LaunchCfg {
 // kernels' only parameter, so a captured launch sequence can be replayed for
 // any batch whose table has been uploaded to the same address).
 cudaError_t launch_prepare(const BatchArgs &a, const BatchArgs *dev, const LaunchCfg &lc);
-// chunked_passes: the verification passes hand out tiles in chunks (for
-// single-source runs, which need dozens of passes); see dt_kernel.
 cudaError_t launch_dt(const BatchArgs &a, const BatchArgs *dev, const LaunchCfg &lc,
                       int max_tile_w, int max_tile_h, int max_apron, bool fixed_grid,
-                      int *grid_used, bool chunked_passes = false);
+                      int *grid_used);
 cudaError_t launch_edges(const BatchArgs &a, const BatchArgs *dev, const LaunchCfg &lc,
                          int max_tile_w, int max_tile_h);
 cudaError_t launch_scatter(const BatchArgs &a, const BatchArgs *dev, const LaunchCfg &lc);
@@ -356,24 +347,69 @@ cudaError_t launch_knn_fit(const BatchArgs &a, const BatchArgs *dev, const Launc
 cudaError_t launch_writeout(const BatchArgs &a, const BatchArgs *dev, const LaunchCfg &lc);
 cudaError_t launch_compact(const BatchArgs &a, BatchArgs *dev, const LaunchCfg &lc);
 
-// Exact variant (per-pixel K nearest and fit).
+// Exact variant (per-pixel K nearest and fit; k_exact.cu).
 constexpr int EXACT_THREADS = 64;
+constexpr int EXACT_WEIGHTS = 16384;   // tabulated kernel weights (squared distances)
+constexpr int SINGLE_W = 64, SINGLE_H = 32, SINGLE_TILE = SINGLE_W * SINGLE_H;
 struct ExactArgs {
-    const float *D;          // [N][H*W] distances, or null: Euclidean
     const float4 *matches;   // [N]
     float *flow;             // [H*W*2]
     int *knn_idx;            // [H*W*K] or null
     float *knn_dist;         // [H*W*K] (with knn_idx)
-    int *fallback;           // [H*W] or null
     int H, W, N, K;
     float a, fallback_eps;
     int weight_squared, estimator;
+    int *slow_count;         // groups of pixels left to the scan, and their list
+    int *slow_list;          // [exact_groups(H, W)]
+    // Euclidean: matches by cells, kernel weights by squared distance
+    int cell_shift, cells_x;
+    const int *cell_start, *cell_match;
+    const double *weights;
+    // geodesic: per tile of 64 x 32 pixels the matches whose distances reach
+    // it and the distance tiles (row-major, +inf beyond the match's cap)
+    int tiles_x;
+    const int *tile_start;   // [tiles + 1]
+    const int2 *tile_entry;  // (match, distance tile)
+    const float *slots;      // [..][SINGLE_TILE]
 };
 size_t exact_smem_bytes(int K);
+long long exact_groups(int H, int W);
+// cells of 2^shift pixels a side, few enough for one CTA to bin into
+void exact_cells(int H, int W, int *shift, int *cells_x, int *cells);
 cudaError_t launch_cap_seed(const float *knn_dist, const int *knn_count, int N, int K, int ld,
                             unsigned long long *init, cudaStream_t stream);
-cudaError_t launch_keys_to_dist(const pkey_t *keys, long long n, float *D, cudaStream_t stream);
-cudaError_t launch_exact_fit(const ExactArgs &x, cudaStream_t stream);
+cudaError_t launch_exact_euclidean(const ExactArgs &x, int *cell_start, int *cell_match, double *weights,
+                                   int cells, int num_sms, cudaStream_t stream);
+cudaError_t launch_exact_geodesic(const ExactArgs &x, int num_sms, cudaStream_t stream);
+
+// The exact variant's single-source distances (k_single.cu).
+struct SingleArgs {
+    const float *C;          // [H*W]
+    const float4 *matches;   // [N]
+    const pkey_t *cap;       // [H*W] distances beyond a pixel's cap are not needed
+    int H, W, N;
+    int tiles_x, tiles_y;    // of SINGLE_W x SINGLE_H pixels
+    // per CTA: keys [H*W], then [tiles] each of a queue, the tiles touched,
+    // the tiles' places in the queue and their flags
+    pkey_t *keys;
+    int *queue, *touched;
+    unsigned *place;
+    unsigned char *flags;
+    // distance tiles: `used` counts all that are needed, the first `slot_cap`
+    // are written
+    float *slots;
+    int2 *slot_of;           // [slot_cap] (tile, match)
+    unsigned slot_cap;
+    unsigned *used, *next;   // (next: match dispenser)
+    int *tile_count;         // [tiles + 1]
+    int *tile_start;         // [tiles + 1]
+    int2 *tile_entry;        // [slot_cap] (match, distance tile) by tile
+    long long max_solves;    // per match
+    RunState *state;
+};
+int single_resident(int num_sms);   // CTAs resident at once
+cudaError_t launch_single(const SingleArgs &x, int ctas, cudaStream_t stream);
+cudaError_t launch_single_lists(const SingleArgs &x, unsigned used, cudaStream_t stream);
 
 // Self-test of the bounded device waits (grid barrier, TMA mbarrier).
 cudaError_t launch_wait_selftest(RunState *st, int which, unsigned long long limit_ns,

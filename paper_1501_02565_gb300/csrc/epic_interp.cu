@@ -68,9 +68,12 @@ struct epic_interp {
     // device staging for epic_interp_run_host
     float *io_C = nullptr, *io_M = nullptr, *io_F = nullptr;
     size_t io_C_n = 0, io_M_n = 0, io_F_n = 0;
-    // scratch of the exact variant (distance rows, relaxation chunk, tables)
+    // scratch of the exact variant: cap map, single-source maps and lists; its
+    // distance tiles
     char *ex_buf = nullptr;
     size_t ex_cap = 0;
+    char *ex_slots = nullptr;
+    size_t ex_slots_cap = 0;
     // scratch of the variational refinement
     void *rf_buf = nullptr;
     // set by the exact variant around its internal approximate run: keep the
@@ -124,8 +127,8 @@ int next_pow2(long long x) {
 // Tile shape for the relaxation of an H x W frame: the first installed rule
 // covering the frame, else the configured tile (64 x 32 by default; apron 4
 // for the sweep schedules of k_dt.cu, none for the warp tiles of
-// k_relax.cu).  With warp_tiles_ok = false (the exact variant's runs, which
-// need the capped relaxation of k_dt.cu), a warp-tile choice becomes the
+// k_relax.cu).  With warp_tiles_ok = false (the exact variant's cap map,
+// whose seeds have distances of their own, which k_dt.cu takes), a warp-tile choice becomes the
 // default k_dt.cu tile.
 constexpr int SWEEP_WARP_TILES = 2;
 
@@ -1196,207 +1199,29 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
     if (epic::exact_smem_bytes(K) > (size_t)h->smem_optin)
         return fail(h, EPIC_ERR_INVALID, "K too large for the per-pixel lists");
     const long long P = (long long)H * W;
-    float *D = nullptr;
-    if (metric == 0) {
-        // single-source relaxations, Cm matches at a time, each a pseudo-pair
-        // with one seed; their distances become row m of D [N][P]
-        int tw, th, ap, sw;
-        choose_tiles(c, h->rules, H, W, &tw, &th, &ap, &sw, false);
-        const int tx = (W + tw - 1) / tw, ty = (H + th - 1) / th, T = tx * ty;
-        const long long chunk_bytes = c.exact_chunk_bytes > 0 ? c.exact_chunk_bytes : (1LL << 30);
-        const long long Cm = std::max(1LL, std::min((long long)N, chunk_bytes / (P * 8)));
-        const size_t small_ints = (size_t)(T + 1) + T + 1 + T + 1 + 1 + 4;  // per pseudo-pair
-        const size_t d_bytes = align_up((size_t)N * P * sizeof(float), 256);
-        const size_t k_bytes = align_up((size_t)Cm * P * sizeof(pkey_t), 256);
-        const size_t s_bytes = align_up((size_t)Cm * small_ints * sizeof(int), 256);
-        const size_t args_bytes = align_up(sizeof(BatchArgs), 256);
-        const size_t pd_bytes = align_up(sizeof(PairDev) * Cm, 256);
-        const size_t pre_stride = align_up(sizeof(int) * (Cm + 1), 256);
-        const size_t t_bytes = args_bytes + pd_bytes + 5 * pre_stride;
-        // cap map: its keys, the bins and per-match scratch of its
-        // relaxation, the seed offsets, and the approximate run's flow
-        const size_t v_ints = (size_t)(T + 1) + T + N + T + N + N + 4;
-        const size_t c_bytes = align_up((size_t)P * sizeof(pkey_t), 256) +
-                               align_up(v_ints * sizeof(int), 256) +
-                               align_up((size_t)N * sizeof(unsigned long long), 256) +
-                               align_up((size_t)P * 2 * sizeof(float), 256);
-        // worklists of the chunked passes: three lists and the queued marks
-        const size_t w_bytes = align_up((size_t)4 * Cm * T * sizeof(int), 256);
-        const size_t need = d_bytes + k_bytes + s_bytes + align_up(t_bytes, 256) + c_bytes + w_bytes;
-        if (need > h->ex_cap) {
-            if ((e = cudaStreamSynchronize(stream)) != cudaSuccess)
-                return cuda_fail(h, e, "cudaStreamSynchronize");
-            if (h->ex_buf) cudaFree(h->ex_buf);
-            h->ex_buf = nullptr;
-            h->ex_cap = 0;
-            e = cudaMalloc(&h->ex_buf, need);
-            if (e != cudaSuccess) {
-                cudaGetLastError();
-                return cuda_fail(h, e, "exact-variant cudaMalloc");
-            }
-            h->ex_cap = need;
+    const long long groups = epic::exact_groups(H, W);
+    auto grow = [&](char **buf, size_t *cap, size_t need) -> int {
+        if (need <= *cap) return EPIC_OK;
+        if ((e = cudaStreamSynchronize(stream)) != cudaSuccess)
+            return cuda_fail(h, e, "cudaStreamSynchronize");
+        if (*buf) cudaFree(*buf);
+        *buf = nullptr;
+        *cap = 0;
+        if ((e = cudaMalloc(buf, need)) != cudaSuccess) {
+            cudaGetLastError();
+            return cuda_fail(h, e, "exact-variant cudaMalloc");
         }
-        char *b = h->ex_buf;
-        D = reinterpret_cast<float *>(b);
-        pkey_t *keys = reinterpret_cast<pkey_t *>(b + d_bytes);
-        int *small = reinterpret_cast<int *>(b + d_bytes + k_bytes);
-        char *tdev = b + d_bytes + k_bytes + s_bytes;
-        char *cb = tdev + align_up(t_bytes, 256);
-        pkey_t *vkeys = reinterpret_cast<pkey_t *>(cb);
-        int *vs = reinterpret_cast<int *>(cb + align_up((size_t)P * sizeof(pkey_t), 256));
-        unsigned long long *vinit = reinterpret_cast<unsigned long long *>(
-            reinterpret_cast<char *>(vs) + align_up(v_ints * sizeof(int), 256));
-        float *aflow = reinterpret_cast<float *>(
-            reinterpret_cast<char *>(vinit) + align_up((size_t)N * sizeof(unsigned long long), 256));
-        int *wl = reinterpret_cast<int *>(cb + c_bytes);   // [3][Cm * T], then [Cm * T] marks
-        std::vector<char> thost(t_bytes);
-        epic::LaunchCfg lc{h->num_sms, h->smem_optin, stream, h->smem_per_sm, h->smem_reserved};
-
-        // Cap map.  An approximate run keeps its K-NN lists: each match's
-        // K-th nearest graph distance bounds its K-th nearest geodesic
-        // distance.  A multi-source relaxation seeded with those bounds gives
-        // V(p) = min over m of (d(p, m) + bound(m)) >= the K-th nearest
-        // distance of p, and V is 1-Lipschitz in the relaxation's metric.
-        // The single-source runs below write back only distances within V,
-        // so each stops spreading about where its seed stops mattering.
-        {
-            h->force_keep = true;
-            epic_pair_desc_t ad{cost_map, matches, H, W, N, K, a, aflow};
-            const int rca = epic_interp_run_batch(h, &ad, 1, stream_);
-            h->force_keep = false;
-            if (rca) return rca;
-            const PairDev &Pa = h->pairs[0];
-            if ((e = epic::launch_cap_seed(Pa.knn_dist, Pa.knn_count, N, K, Pa.K, vinit, stream)))
-                return cuda_fail(h, e, "exact-variant cap seeds");
-            PairDev v{};
-            v.C = cost_map;
-            v.matches = reinterpret_cast<const float4 *>(matches);
-            v.H = H;
-            v.W = W;
-            v.N = N;
-            v.K = 1;
-            v.a = 1.f;
-            v.tile_w = tw;
-            v.tile_h = th;
-            v.apron = ap;
-            v.sweep = sw;
-            v.tiles_x = tx;
-            v.tiles_y = ty;
-            v.keys = vkeys;
-            v.tile_start = vs;
-            v.tile_fill = vs + T + 1;
-            v.tile_seeds = vs + 2 * T + 1;
-            v.tile_stamp = vs + 2 * T + 1 + N;
-            v.deg = vs + 3 * T + 1 + N;
-            v.wmin = reinterpret_cast<unsigned *>(vs + 3 * T + 1 + 2 * N);
-            v.info = vs + 3 * T + 1 + 3 * N;
-            v.seed_init = vinit;
-            std::vector<int> pre(5 * 2, 0);
-            pre[1] = T;          // tiles
-            pre[2 + 1] = N;      // matches
-            BatchArgs vb{};
-            vb.pairs = reinterpret_cast<const PairDev *>(tdev + args_bytes);
-            vb.npairs = 1;
-            auto vpre = [&](int k) {
-                return reinterpret_cast<const int *>(tdev + args_bytes + pd_bytes + k * pre_stride);
-            };
-            vb.tile_base = vpre(0);
-            vb.match_base = vpre(1);
-            vb.chunk_base = vpre(2);
-            vb.hash_base = vpre(3);
-            vb.clear_base = vpre(4);
-            vb.total_tiles = T;
-            vb.total_matches = N;
-            vb.max_degree = 1;
-            vb.max_passes = c.max_passes;
-            vb.weight_squared = 1;
-            vb.fallback_eps = c.fallback_eps;
-            vb.state = h->state;
-            memcpy(thost.data(), &vb, sizeof vb);
-            memcpy(thost.data() + args_bytes, &v, sizeof(PairDev));
-            for (int k = 0; k < 5; ++k)
-                memcpy(thost.data() + args_bytes + pd_bytes + k * pre_stride, pre.data() + k * 2,
-                       sizeof(int) * 2);
-            const BatchArgs *dev_v = reinterpret_cast<const BatchArgs *>(tdev);
-            if ((e = cudaMemcpyAsync(tdev, thost.data(), t_bytes, cudaMemcpyHostToDevice, stream)) ||
-                (e = epic::launch_prepare(vb, dev_v, lc)) ||
-                (e = epic::launch_dt(vb, dev_v, lc, tw, th, ap, false, nullptr)) ||
-                (e = cudaStreamSynchronize(stream)))
-                return cuda_fail(h, e, "exact-variant cap map");
-        }
-        for (long long m0 = 0; m0 < N; m0 += Cm) {
-            const int n = (int)std::min(Cm, (long long)N - m0);
-            std::vector<PairDev> pd(n);
-            for (int j = 0; j < n; ++j) {
-                PairDev &q = pd[j];
-                q = PairDev{};
-                q.C = cost_map;
-                q.matches = reinterpret_cast<const float4 *>(matches) + m0 + j;
-                q.H = H;
-                q.W = W;
-                q.N = 1;
-                q.K = 1;
-                q.a = 1.f;
-                q.tile_w = tw;
-                q.tile_h = th;
-                q.apron = ap;
-                q.sweep = sw;
-                q.tiles_x = tx;
-                q.tiles_y = ty;
-                q.keys = keys + (size_t)j * P;
-                int *sp = small + (size_t)j * small_ints;
-                q.tile_start = sp;
-                q.tile_fill = sp + T + 1;
-                q.tile_seeds = sp + 2 * T + 1;
-                q.tile_stamp = sp + 2 * T + 2;
-                q.deg = sp + 3 * T + 2;
-                q.wmin = reinterpret_cast<unsigned *>(sp + 3 * T + 3);
-                q.info = sp + 3 * T + 4;
-                q.cap = vkeys;
-            }
-            std::vector<int> pre(5 * (n + 1), 0);
-            for (int j = 0; j <= n; ++j) {
-                pre[j] = j * T;                 // tiles
-                pre[(n + 1) + j] = j;           // matches
-            }
-            BatchArgs ba{};
-            ba.pairs = reinterpret_cast<const PairDev *>(tdev + args_bytes);
-            ba.npairs = n;
-            auto pre_dev = [&](int k) {
-                return reinterpret_cast<const int *>(tdev + args_bytes + pd_bytes + k * pre_stride);
-            };
-            ba.tile_base = pre_dev(0);
-            ba.match_base = pre_dev(1);
-            ba.chunk_base = pre_dev(2);
-            ba.hash_base = pre_dev(3);
-            ba.clear_base = pre_dev(4);
-            ba.total_tiles = n * T;
-            ba.total_matches = n;
-            ba.uniform_tiles = T;
-            ba.wl = wl;
-            ba.wl_queued = wl + (size_t)3 * n * T;
-            ba.max_degree = 1;
-            ba.max_passes = c.max_passes;
-            ba.weight_squared = 1;
-            ba.fallback_eps = c.fallback_eps;
-            ba.state = h->state;
-            memcpy(thost.data(), &ba, sizeof ba);
-            memcpy(thost.data() + args_bytes, pd.data(), sizeof(PairDev) * n);
-            for (int k = 0; k < 5; ++k)
-                memcpy(thost.data() + args_bytes + pd_bytes + k * pre_stride, pre.data() + k * (n + 1),
-                       sizeof(int) * (n + 1));
-            const BatchArgs *dev_a = reinterpret_cast<const BatchArgs *>(tdev);
-            if ((e = cudaMemcpyAsync(tdev, thost.data(), t_bytes, cudaMemcpyHostToDevice, stream)) ||
-                (e = cudaMemsetAsync(ba.wl_queued, 0, sizeof(int) * (size_t)n * T, stream)) ||
-                (e = epic::launch_prepare(ba, dev_a, lc)) ||
-                (e = epic::launch_dt(ba, dev_a, lc, tw, th, ap, false, nullptr, true)) ||
-                (e = epic::launch_keys_to_dist(keys, (long long)n * P, D + m0 * P, stream)) ||
-                (e = cudaStreamSynchronize(stream)))
-                return cuda_fail(h, e, "exact-variant relaxation");
-        }
-    }
+        *cap = need;
+        return EPIC_OK;
+    };
+    // regions of ex_buf, each 256-byte aligned
+    size_t used = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = used;
+        used = align_up(used + bytes, 256);
+        return at;
+    };
     epic::ExactArgs x{};
-    x.D = D;
     x.matches = reinterpret_cast<const float4 *>(matches);
     x.flow = flow_out;
     x.knn_idx = knn_idx_out;
@@ -1409,7 +1234,184 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
     x.fallback_eps = c.fallback_eps;
     x.weight_squared = c.weight_squared ? 1 : 0;
     x.estimator = c.estimator;
-    if ((e = epic::launch_exact_fit(x, stream)) != cudaSuccess)
+    const size_t o_slow = take(sizeof(int) * (size_t)(groups + 1));
+    if (metric == 1) {
+        int cells = 0;
+        epic::exact_cells(H, W, &x.cell_shift, &x.cells_x, &cells);
+        const size_t o_start = take(sizeof(int) * (size_t)(cells + 1));
+        const size_t o_match = take(sizeof(int) * (size_t)N);
+        const size_t o_weights = take(sizeof(double) * epic::EXACT_WEIGHTS);
+        if ((rc = grow(&h->ex_buf, &h->ex_cap, used))) return rc;
+        char *b = h->ex_buf;
+        x.slow_count = reinterpret_cast<int *>(b + o_slow);
+        x.slow_list = x.slow_count + 1;
+        int *start = reinterpret_cast<int *>(b + o_start), *match = reinterpret_cast<int *>(b + o_match);
+        double *weights = reinterpret_cast<double *>(b + o_weights);
+        x.cell_start = start;
+        x.cell_match = match;
+        x.weights = weights;
+        if ((e = cudaMemsetAsync(x.slow_count, 0, sizeof(int), stream)) ||
+            (e = epic::launch_exact_euclidean(x, start, match, weights, cells, h->num_sms, stream)))
+            return cuda_fail(h, e, "exact-variant fit");
+        h->last_stream = stream;
+        return epic_interp_sync(h);
+    }
+    // Geodesic.  Cap map: an approximate run keeps its K-NN lists: each
+    // match's K-th nearest graph distance bounds its K-th nearest geodesic
+    // distance.  A multi-source relaxation seeded with those bounds gives
+    // V(p) = min over m of (d(p, m) + bound(m)) >= the K-th nearest distance
+    // of p, and V is 1-Lipschitz in the relaxation's metric.  The
+    // single-source runs below write back only distances within V, so each
+    // stops spreading about where its seed stops mattering.
+    int tw, th, ap, sw;
+    choose_tiles(c, h->rules, H, W, &tw, &th, &ap, &sw, false);
+    const int tx = (W + tw - 1) / tw, ty = (H + th - 1) / th, T = tx * ty;
+    // one BatchArgs, one descriptor, five prefix arrays of two ints
+    const size_t args_bytes = align_up(sizeof(BatchArgs), 256), pd_bytes = align_up(sizeof(PairDev), 256);
+    const size_t t_bytes = args_bytes + pd_bytes + 5 * 256;
+    const size_t v_ints = (size_t)(T + 1) + T + N + T + N + N + 4;
+    const size_t o_table = take(t_bytes);
+    const size_t o_vkeys = take(sizeof(pkey_t) * (size_t)P);
+    const size_t o_vints = take(sizeof(int) * v_ints);
+    const size_t o_vinit = take(sizeof(unsigned long long) * (size_t)N);
+    const size_t o_aflow = take(sizeof(float) * 2 * (size_t)P);
+    // single-source runs: a key map and a tile list per CTA, as many as the
+    // budget for keys allows and the GPU holds
+    const int sx = (W + epic::SINGLE_W - 1) / epic::SINGLE_W;
+    const int sy = (H + epic::SINGLE_H - 1) / epic::SINGLE_H;
+    const long long ST = (long long)sx * sy;
+    const long long chunk_bytes = c.exact_chunk_bytes > 0 ? c.exact_chunk_bytes : (1LL << 30);
+    const int ctas = (int)std::max(1LL, std::min({(long long)N, chunk_bytes / (P * 8),
+                                                  (long long)epic::single_resident(h->num_sms)}));
+    const size_t o_keys = take(sizeof(pkey_t) * (size_t)P * ctas);
+    const size_t o_queue = take(sizeof(int) * (size_t)ST * ctas);
+    const size_t o_touched = take(sizeof(int) * (size_t)ST * ctas);
+    const size_t o_place = take(sizeof(unsigned) * (size_t)ST * ctas);
+    const size_t o_flags = take((size_t)ST * ctas);
+    const size_t o_count = take(sizeof(int) * (size_t)(ST + 4));   // tile counts, then used and next
+    const size_t o_start = take(sizeof(int) * (size_t)(ST + 1));
+    if ((rc = grow(&h->ex_buf, &h->ex_cap, used))) return rc;
+    char *b = h->ex_buf;
+    pkey_t *vkeys = reinterpret_cast<pkey_t *>(b + o_vkeys);
+    int *vs = reinterpret_cast<int *>(b + o_vints);
+    unsigned long long *vinit = reinterpret_cast<unsigned long long *>(b + o_vinit);
+    float *aflow = reinterpret_cast<float *>(b + o_aflow);
+    char *tdev = b + o_table;
+    epic::LaunchCfg lc{h->num_sms, h->smem_optin, stream, h->smem_per_sm, h->smem_reserved};
+    {
+        h->force_keep = true;
+        epic_pair_desc_t ad{cost_map, matches, H, W, N, K, a, aflow};
+        const int rca = epic_interp_run_batch(h, &ad, 1, stream_);
+        h->force_keep = false;
+        if (rca) return rca;
+        const PairDev &Pa = h->pairs[0];
+        if ((e = epic::launch_cap_seed(Pa.knn_dist, Pa.knn_count, N, K, Pa.K, vinit, stream)))
+            return cuda_fail(h, e, "exact-variant cap seeds");
+        PairDev v{};
+        v.C = cost_map;
+        v.matches = reinterpret_cast<const float4 *>(matches);
+        v.H = H;
+        v.W = W;
+        v.N = N;
+        v.K = 1;
+        v.a = 1.f;
+        v.tile_w = tw;
+        v.tile_h = th;
+        v.apron = ap;
+        v.sweep = sw;
+        v.tiles_x = tx;
+        v.tiles_y = ty;
+        v.keys = vkeys;
+        v.tile_start = vs;
+        v.tile_fill = vs + T + 1;
+        v.tile_seeds = vs + 2 * T + 1;
+        v.tile_stamp = vs + 2 * T + 1 + N;
+        v.deg = vs + 3 * T + 1 + N;
+        v.wmin = reinterpret_cast<unsigned *>(vs + 3 * T + 1 + 2 * N);
+        v.info = vs + 3 * T + 1 + 3 * N;
+        v.seed_init = vinit;
+        auto vpre = [&](int k) {
+            return reinterpret_cast<const int *>(tdev + args_bytes + pd_bytes + k * 256);
+        };
+        BatchArgs vb{};
+        vb.pairs = reinterpret_cast<const PairDev *>(tdev + args_bytes);
+        vb.npairs = 1;
+        vb.tile_base = vpre(0);
+        vb.match_base = vpre(1);
+        vb.chunk_base = vpre(2);
+        vb.hash_base = vpre(3);
+        vb.clear_base = vpre(4);
+        vb.total_tiles = T;
+        vb.total_matches = N;
+        vb.max_degree = 1;
+        vb.max_passes = c.max_passes;
+        vb.weight_squared = 1;
+        vb.fallback_eps = c.fallback_eps;
+        vb.state = h->state;
+        std::vector<char> thost(t_bytes, 0);
+        memcpy(thost.data(), &vb, sizeof vb);
+        memcpy(thost.data() + args_bytes, &v, sizeof(PairDev));
+        const int ends[2] = {T, N};   // the prefixes are {0, tiles}, {0, matches}, then zeros
+        for (int k = 0; k < 2; ++k)
+            memcpy(thost.data() + args_bytes + pd_bytes + k * 256 + sizeof(int), &ends[k], sizeof(int));
+        const BatchArgs *dev_v = reinterpret_cast<const BatchArgs *>(tdev);
+        if ((e = cudaMemcpyAsync(tdev, thost.data(), t_bytes, cudaMemcpyHostToDevice, stream)) ||
+            (e = epic::launch_prepare(vb, dev_v, lc)) ||
+            (e = epic::launch_dt(vb, dev_v, lc, tw, th, ap, false, nullptr)))
+            return cuda_fail(h, e, "exact-variant cap map");
+        // (a copy from pageable memory has read its source when it returns)
+    }
+    epic::SingleArgs s{};
+    s.C = cost_map;
+    s.matches = x.matches;
+    s.cap = vkeys;
+    s.H = H;
+    s.W = W;
+    s.N = N;
+    s.tiles_x = sx;
+    s.tiles_y = sy;
+    s.keys = reinterpret_cast<pkey_t *>(b + o_keys);
+    s.queue = reinterpret_cast<int *>(b + o_queue);
+    s.touched = reinterpret_cast<int *>(b + o_touched);
+    s.place = reinterpret_cast<unsigned *>(b + o_place);
+    s.flags = reinterpret_cast<unsigned char *>(b + o_flags);
+    s.tile_count = reinterpret_cast<int *>(b + o_count);
+    s.used = reinterpret_cast<unsigned *>(s.tile_count + ST);
+    s.next = s.used + 1;
+    s.tile_start = reinterpret_cast<int *>(b + o_start);
+    s.max_solves = (long long)c.max_passes * ST;
+    s.state = h->state;
+    // distance tiles: room for 16 per match to begin with (11 on the flow
+    // workloads at K = 100); a run that needs more says how many
+    const size_t per_slot = sizeof(float) * epic::SINGLE_TILE + 2 * sizeof(int2);
+    unsigned long long want = std::min<unsigned long long>((unsigned long long)N * ST, 16ull * N + 1024);
+    unsigned n_used = 0;
+    for (;;) {
+        want = std::max<unsigned long long>(want, h->ex_slots_cap / per_slot);
+        want = std::min<unsigned long long>(want, 0x7fffffffull);
+        if ((rc = grow(&h->ex_slots, &h->ex_slots_cap, (size_t)want * per_slot))) return rc;
+        s.slot_cap = (unsigned)want;
+        s.slots = reinterpret_cast<float *>(h->ex_slots);
+        s.slot_of = reinterpret_cast<int2 *>(s.slots + (size_t)want * epic::SINGLE_TILE);
+        s.tile_entry = s.slot_of + want;
+        if ((e = cudaMemsetAsync(s.tile_count, 0, sizeof(int) * (size_t)(ST + 4), stream)) ||
+            (e = epic::launch_single(s, ctas, stream)) ||
+            (e = cudaMemcpyAsync(&n_used, s.used, sizeof n_used, cudaMemcpyDeviceToHost, stream)) ||
+            (e = cudaStreamSynchronize(stream)))
+            return cuda_fail(h, e, "exact-variant relaxation");
+        if (n_used <= s.slot_cap) break;
+        if (n_used > 0x7fffffffu) return fail(h, EPIC_ERR_CAPACITY, "exact variant: too many distance tiles");
+        want = n_used;
+    }
+    x.slow_count = reinterpret_cast<int *>(b + o_slow);
+    x.slow_list = x.slow_count + 1;
+    x.tiles_x = sx;
+    x.tile_start = s.tile_start;
+    x.tile_entry = s.tile_entry;
+    x.slots = s.slots;
+    if ((e = epic::launch_single_lists(s, n_used, stream)) ||
+        (e = cudaMemsetAsync(x.slow_count, 0, sizeof(int), stream)) ||
+        (e = epic::launch_exact_geodesic(x, h->num_sms, stream)))
         return cuda_fail(h, e, "exact-variant fit");
     h->last_stream = stream;
     return epic_interp_sync(h);
@@ -1560,6 +1562,7 @@ void epic_interp_destroy(epic_interp_t *h) {
     if (h->io_M) cudaFree(h->io_M);
     if (h->io_F) cudaFree(h->io_F);
     if (h->ex_buf) cudaFree(h->ex_buf);
+    if (h->ex_slots) cudaFree(h->ex_slots);
     if (h->rf_buf) cudaFree(h->rf_buf);
     for (cudaEvent_t x : h->tev) cudaEventDestroy(x);
     delete h;

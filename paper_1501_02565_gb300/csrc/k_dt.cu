@@ -261,21 +261,6 @@ __device__ __forceinline__ float *stage_area(unsigned char *smem) {
     return reinterpret_cast<float *>(((uintptr_t)smem + 127) & ~(uintptr_t)127);
 }
 
-// A key as written back: with a cap map (the exact variant's single-source
-// runs), a distance beyond the pixel's cap is left unreached, so the run
-// stops spreading where it can no longer matter.  The cap is 1-Lipschitz in
-// the same fixed-point metric, so every pixel on a shortest path to a
-// pixel within its cap is within its own cap: capped runs are exact there.
-__device__ __forceinline__ pkey_t capped(const PairDev &P, size_t p, pkey_t k) {
-    return P.cap && key_dunits(k) > key_dunits(P.cap[p]) ? KEY_INF : k;
-}
-
-// The pair a flat tile index belongs to (a division when all pairs have the
-// same tile count, as the exact variant's single-source pseudo-pairs do).
-__device__ __forceinline__ int tile_pair(const BatchArgs &a, int t) {
-    return a.uniform_tiles > 0 ? t / a.uniform_tiles : find_pair(a.tile_base, a.npairs, t);
-}
-
 // Phase 1: solve tile (tx, ty) on its region from its seeds alone.  Returns
 // false when the cost staging timed out (the CTA must leave the kernel).
 __device__ bool solve_fresh(const PairDev &P, int tx, int ty, pkey_t *K,
@@ -338,8 +323,7 @@ __device__ bool solve_fresh(const PairDev &P, int tx, int ty, pkey_t *K,
         int ly = i / P.tile_w, lx = i - ly * P.tile_w;
         int gx = gx0 + lx, gy = gy0 + ly;
         if (gx < P.W && gy < P.H)
-            P.keys[(size_t)gy * P.W + gx] =
-                capped(P, (size_t)gy * P.W + gx, K[(ly + off) * g.P + lx + off]);
+            P.keys[(size_t)gy * P.W + gx] = K[(ly + off) * g.P + lx + off];
     }
     __syncthreads();
     return true;
@@ -381,9 +365,7 @@ __device__ bool border_dirty(const PairDev &P, int tx, int ty) {
             const pkey_t kq = ld_key(P.keys + q);
             const unsigned hq = half_cost(__ldg(P.C + q), &bad);
             const unsigned long long w = (dx != 0 && dy != 0) ? step_diag(hp, hq) : step_axis(hp, hq);
-            // an improvement beyond the pixel's cap would be written back
-            // unreached, so it does not make the tile dirty
-            dirty |= capped(P, p, step_key(kq, w)) < kp;
+            dirty |= step_key(kq, w) < kp;
         }
     }
     return __syncthreads_or(dirty) != 0;
@@ -411,8 +393,7 @@ __device__ int solve_again(const PairDev &P, int tx, int ty, pkey_t *K,
             int ly = i / P.tile_w, lx = i - ly * P.tile_w;
             int gx = gx0 + lx, gy = gy0 + ly;
             if (gx < P.W && gy < P.H)
-                P.keys[(size_t)gy * P.W + gx] =
-                    capped(P, (size_t)gy * P.W + gx, K[(ly + 1) * g.P + lx + 1]);
+                P.keys[(size_t)gy * P.W + gx] = K[(ly + 1) * g.P + lx + 1];
         }
     }
     if (threadIdx.x == 0) P.tile_stamp[ty * P.tiles_x + tx] = pass;
@@ -420,32 +401,6 @@ __device__ int solve_again(const PairDev &P, int tx, int ty, pkey_t *K,
     return changed ? 1 : 0;
 }
 
-// Chunked passes: queue the eight neighbours of tile t (flat index; local
-// (tx, ty) in pair pi) for pass `next`, each at most once (threads 0-7).
-__device__ __forceinline__ void queue_neighbours(const BatchArgs &a, RunState *st, int pi,
-                                                 int tx, int ty, int next) {
-    if (threadIdx.x >= 8) return;
-    const PairDev &P = a.pairs[pi];
-    const int k = threadIdx.x;
-    const int x = tx + (k < 3 ? k - 1 : k < 5 ? 2 * k - 7 : k - 6);
-    const int y = ty + (k < 3 ? -1 : k < 5 ? 0 : 1);
-    if (x < 0 || x >= P.tiles_x || y < 0 || y >= P.tiles_y) return;
-    const int nt = a.tile_base[pi] + y * P.tiles_x + x;
-    if (atomicMax(a.wl_queued + nt, next + 1) < next + 1) {
-        const unsigned q = atomicAdd(&st->wl_count[next % 3], 1u);
-        a.wl[(size_t)(next % 3) * a.total_tiles + q] = nt;
-    }
-}
-
-// CHUNKED: how the verification passes hand out tiles.  false (the
-// interpolator's runs: a handful of passes, about half of the tiles
-// re-solved in the first): one tile at a time.  true (the single-source runs
-// of the exact variant: dozens of passes while distances cross the image
-// tile by tile, each re-solving a thin front): chunks of tiles whose
-// neighbour stamps are read in parallel.  The chunked loop keeps more state
-// and, at the four-CTA register budget, costs the interpolator's sweeps a
-// spill (2.21 -> 2.33 ms); the single-source runs go 3.1 -> 2.1 s per pair.
-template <bool CHUNKED>
 __global__ void __launch_bounds__(DT_THREADS) dt_kernel(const BatchArgs *__restrict__ ap) {
     const BatchArgs a = *ap;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -468,7 +423,7 @@ __global__ void __launch_bounds__(DT_THREADS) dt_kernel(const BatchArgs *__restr
             const int t = (int)atomicAdd(dispenser, 1u);
             s_tile = t;
             if (t < a.total_tiles) {
-                s_pair = tile_pair(a, t);
+                s_pair = find_pair(a.tile_base, a.npairs, t);
                 s_local = t - a.tile_base[s_pair];
             }
         }
@@ -498,120 +453,26 @@ __global__ void __launch_bounds__(DT_THREADS) dt_kernel(const BatchArgs *__restr
         }
         unsigned *cnt = &st->changed[pass % 3];
         unsigned *disp = &st->work[pass % 3];
-        if constexpr (!CHUNKED) {
-            for (int t = next_tile(disp); t < a.total_tiles; t = next_tile(disp)) {
-                const PairDev &P = a.pairs[s_pair];
-                const int tx = s_local % P.tiles_x, ty = s_local / P.tiles_x;
-                // threads 0-7 read the eight neighbour stamps at once
-                bool nb = false;
-                if (threadIdx.x < 8) {
-                    const int k = threadIdx.x;
-                    const int x = tx + (k < 3 ? k - 1 : k < 5 ? 2 * k - 7 : k - 6);
-                    const int y = ty + (k < 3 ? -1 : k < 5 ? 0 : 1);
-                    nb = x >= 0 && x < P.tiles_x && y >= 0 && y < P.tiles_y &&
-                         __ldcg(P.tile_stamp + y * P.tiles_x + x) >= pass;
-                }
-                if (__syncthreads_or(nb) && border_dirty(P, tx, ty)) {
-                    const Region g = make_region(P, 0, 0, P.tile_w, P.tile_h, 0);
-                    pkey_t *K = reinterpret_cast<pkey_t *>(smem);
-                    unsigned *h = reinterpret_cast<unsigned *>(smem + sizeof(pkey_t) * g.RH * g.P);
-                    if (solve_again(P, tx, ty, K, h, st, pass + 1, stage, tma) < 0) return;
-                    if (threadIdx.x == 0) atomicAdd(cnt, 1u);
-                }
-                __syncthreads();
+        for (int t = next_tile(disp); t < a.total_tiles; t = next_tile(disp)) {
+            const PairDev &P = a.pairs[s_pair];
+            const int tx = s_local % P.tiles_x, ty = s_local / P.tiles_x;
+            // threads 0-7 read the eight neighbour stamps at once
+            bool nb = false;
+            if (threadIdx.x < 8) {
+                const int k = threadIdx.x;
+                const int x = tx + (k < 3 ? k - 1 : k < 5 ? 2 * k - 7 : k - 6);
+                const int y = ty + (k < 3 ? -1 : k < 5 ? 0 : 1);
+                nb = x >= 0 && x < P.tiles_x && y >= 0 && y < P.tiles_y &&
+                     __ldcg(P.tile_stamp + y * P.tiles_x + x) >= pass;
             }
-        } else {
-            // Pass 0 scans every tile, PASS_CHUNK at a time: the first
-            // 8 x PASS_CHUNK threads read the chunk's neighbour stamps in
-            // parallel and flag the tiles with a neighbour written since phase
-            // 1; only those go on to the border test.  A tile that changes
-            // queues its eight neighbours for the next pass, and every later
-            // pass works through that list alone (a single-source run
-            // re-solves a thin front, and scanning every tile in each of its
-            // dozen passes cost more than the re-solves).  The loop state
-            // lives in shared memory, so nothing extra stays in registers
-            // across a re-solve.
-            __shared__ int s_t0, s_bits;
-            if (pass == 0) {
-                for (;;) {
-                    __syncthreads();
-                    if (threadIdx.x == 0) {
-                        s_t0 = (int)atomicAdd(disp, (unsigned)PASS_CHUNK);
-                        s_bits = 0;
-                    }
-                    __syncthreads();
-                    if (s_t0 >= a.total_tiles) break;
-                    if (threadIdx.x < 8 * PASS_CHUNK) {
-                        const int t = s_t0 + (threadIdx.x >> 3), k = threadIdx.x & 7;
-                        if (t < a.total_tiles) {
-                            const int pi = tile_pair(a, t);
-                            const PairDev &P = a.pairs[pi];
-                            const int lt = t - a.tile_base[pi];
-                            const int x = lt % P.tiles_x + (k < 3 ? k - 1 : k < 5 ? 2 * k - 7 : k - 6);
-                            const int y = lt / P.tiles_x + (k < 3 ? -1 : k < 5 ? 0 : 1);
-                            if (x >= 0 && x < P.tiles_x && y >= 0 && y < P.tiles_y &&
-                                __ldcg(P.tile_stamp + y * P.tiles_x + x) >= pass)
-                                atomicOr(&s_bits, 1 << (threadIdx.x >> 3));
-                        }
-                    }
-                    for (;;) {
-                        __syncthreads();
-                        if (threadIdx.x == 0) {
-                            const int b = s_bits;
-                            if (b) {
-                                const int t = s_t0 + __ffs(b) - 1;
-                                s_bits = b & (b - 1);
-                                s_tile = t;
-                                s_pair = tile_pair(a, t);
-                                s_local = t - a.tile_base[s_pair];
-                            } else {
-                                s_tile = -1;
-                            }
-                        }
-                        __syncthreads();
-                        if (s_tile < 0) break;
-                        const PairDev &P = a.pairs[s_pair];
-                        const int tx = s_local % P.tiles_x, ty = s_local / P.tiles_x;
-                        if (border_dirty(P, tx, ty)) {
-                            const Region g = make_region(P, 0, 0, P.tile_w, P.tile_h, 0);
-                            pkey_t *K = reinterpret_cast<pkey_t *>(smem);
-                            unsigned *h = reinterpret_cast<unsigned *>(smem + sizeof(pkey_t) * g.RH * g.P);
-                            const int r = solve_again(P, tx, ty, K, h, st, pass + 1, stage, tma);
-                            if (r < 0) return;
-                            if (r > 0) queue_neighbours(a, st, s_pair, tx, ty, pass + 1);
-                            if (threadIdx.x == 0) atomicAdd(cnt, 1u);
-                        }
-                    }
-                }
-            } else {
-                // the list of this pass was complete before the last barrier
-                const unsigned n = ld_acquire(&st->wl_count[pass % 3]);
-                const int *list = a.wl + (size_t)(pass % 3) * a.total_tiles;
-                for (;;) {
-                    __syncthreads();
-                    if (threadIdx.x == 0) {
-                        const unsigned q = atomicAdd(disp, 1u);
-                        s_tile = q < n ? list[q] : -1;
-                        if (s_tile >= 0) {
-                            s_pair = tile_pair(a, s_tile);
-                            s_local = s_tile - a.tile_base[s_pair];
-                        }
-                    }
-                    __syncthreads();
-                    if (s_tile < 0) break;
-                    const PairDev &P = a.pairs[s_pair];
-                    const int tx = s_local % P.tiles_x, ty = s_local / P.tiles_x;
-                    if (border_dirty(P, tx, ty)) {
-                        const Region g = make_region(P, 0, 0, P.tile_w, P.tile_h, 0);
-                        pkey_t *K = reinterpret_cast<pkey_t *>(smem);
-                        unsigned *h = reinterpret_cast<unsigned *>(smem + sizeof(pkey_t) * g.RH * g.P);
-                        const int r = solve_again(P, tx, ty, K, h, st, pass + 1, stage, tma);
-                        if (r < 0) return;
-                        if (r > 0) queue_neighbours(a, st, s_pair, tx, ty, pass + 1);
-                        if (threadIdx.x == 0) atomicAdd(cnt, 1u);
-                    }
-                }
+            if (__syncthreads_or(nb) && border_dirty(P, tx, ty)) {
+                const Region g = make_region(P, 0, 0, P.tile_w, P.tile_h, 0);
+                pkey_t *K = reinterpret_cast<pkey_t *>(smem);
+                unsigned *h = reinterpret_cast<unsigned *>(smem + sizeof(pkey_t) * g.RH * g.P);
+                if (solve_again(P, tx, ty, K, h, st, pass + 1, stage, tma) < 0) return;
+                if (threadIdx.x == 0) atomicAdd(cnt, 1u);
             }
+            __syncthreads();
         }
         if (!grid_sync(st, nblocks)) return;
         const unsigned dirty = ld_acquire(cnt);
@@ -620,7 +481,6 @@ __global__ void __launch_bounds__(DT_THREADS) dt_kernel(const BatchArgs *__restr
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             st->changed[(pass + 2) % 3] = 0;
             st->work[(pass + 2) % 3] = 0;
-            st->wl_count[(pass + 2) % 3] = 0;
         }
         if (dirty == 0) {
             if (blockIdx.x == 0 && threadIdx.x == 0) st->passes = pass + 1;
@@ -663,9 +523,9 @@ size_t dt_smem_bytes(int tile_w, int tile_h, int apron) {
 
 cudaError_t launch_dt(const BatchArgs &a, const BatchArgs *dev, const LaunchCfg &lc,
                       int max_tile_w, int max_tile_h, int max_apron, bool fixed_grid,
-                      int *grid_used, bool chunked_passes) {
+                      int *grid_used) {
     size_t smem = dt_smem_bytes(max_tile_w, max_tile_h, max_apron);
-    void (*kernel)(const BatchArgs *) = chunked_passes ? dt_kernel<true> : dt_kernel<false>;
+    void (*kernel)(const BatchArgs *) = dt_kernel;
     cudaError_t e = cudaFuncSetAttribute(
         kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

@@ -93,14 +93,20 @@ __device__ __forceinline__ void lower(unsigned &d, unsigned q, unsigned w) {
     d = __viaddmin_u32(q, w, d);
 }
 
-// The rounds of a solve.  (A thread notices a change of its block by the sum
-// of its distances, which only fall; a sum that falls by a multiple of 2^32
-// would end the rounds early, and the settling pass completes the tile.)
+// The sum of a block's distances, which only fall, so that it changes whenever
+// one does.
+__device__ __forceinline__ unsigned long long block_sum(const DistBlock &B) {
+    unsigned long long s = 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i)   // (IMAD.WIDE: not on the integer pipe)
+        asm("mad.wide.u32 %0, %1, 1, %0;" : "+l"(s) : "r"(B.d[i >> 2][i & 3]));
+    return s;
+}
+
+// The rounds of a solve.
 template <int MAXR>
 __device__ void dist_rounds(DistTile<MAXR> &T, DistBlock &B, int b, int cap) {
-    unsigned sum = 0;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) sum += B.d[i >> 2][i & 3];
+    unsigned long long sum = block_sum(B);
     for (int round = 0; round < cap; ++round) {
         unsigned w[4], e[4], n[6], s[6];
 #pragma unroll
@@ -134,9 +140,7 @@ __device__ void dist_rounds(DistTile<MAXR> &T, DistBlock &B, int b, int cap) {
                 lower(d, c < 3 ? B.d[r][c + 1] : e[r], B.wh[r][c + 1]);
                 B.d[r][c] = d;
             }
-        unsigned now = 0;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) now += B.d[i >> 2][i & 3];
+        const unsigned long long now = block_sum(B);
         const bool changed = now != sum;
         sum = now;
         if (changed) {
@@ -287,48 +291,112 @@ __device__ void block_weights(const DistTile<MAXR> &T, int b, const Staged &S, D
     auto hc = [&](int r, int c) {
         return r >= 0 && r < 4 && c >= 0 && c < 4 ? S.h[r & 3][c & 3] : around(T.h, b, r, c);
     };
-            // weights; a step to a cell of the block that lies outside the image
-            // (or below the ring row) is blocked by the cap
-            unsigned hr[6][6];
-    #pragma unroll
-            for (int r = 0; r < 6; ++r)
-    #pragma unroll
-                for (int c = 0; c < 6; ++c) hr[r][c] = hc(r - 1, c - 1);
-    #pragma unroll
-            for (int i = 0; i < 4; ++i)
-    #pragma unroll
-                for (int j = 0; j < 5; ++j) {
-                    B.wh[i][j] = hr[i + 1][j] + hr[i + 1][j + 1];
-                    B.wv[j][i] = hr[j][i + 1] + hr[j + 1][i + 1];
-                }
-    #pragma unroll
-            for (int r = 0; r < 5; ++r)
-    #pragma unroll
-                for (int c = 0; c < 5; ++c) {
-                    if (!((r == 0 && c == 4) || (r == 4 && c == 0)))
-                        B.wb[r][c] = diag_weight(hr[r][c], hr[r + 1][c + 1], wmax);
-                    if (!((r == 0 && c == 0) || (r == 4 && c == 4)))
-                        B.ws[r][c] = diag_weight(hr[r][c + 1], hr[r + 1][c], wmax);
-                }
-            if (S.nrow < 4 || S.ncol < 4) {
-                auto out = [&](int r, int c) {   // own cells only: the ring's are never lowered
-                    return r >= 0 && r < 4 && c >= 0 && c < 4 && (r >= S.nrow || c >= S.ncol);
-                };
-    #pragma unroll
-                for (int i = 0; i < 4; ++i)
-    #pragma unroll
-                    for (int j = 0; j < 5; ++j) {
-                        if (out(i, j - 1) || out(i, j)) B.wh[i][j] = wmax;
-                        if (out(j - 1, i) || out(j, i)) B.wv[j][i] = wmax;
-                    }
-    #pragma unroll
-                for (int r = 0; r < 5; ++r)
-    #pragma unroll
-                    for (int c = 0; c < 5; ++c) {
-                        if (out(r - 1, c - 1) || out(r, c)) B.wb[r][c] = wmax;
-                        if (out(r - 1, c) || out(r, c - 1)) B.ws[r][c] = wmax;
-                    }
+    // weights; a step to a cell of the block that lies outside the image
+    // (or below the ring row) is blocked by the cap
+    unsigned hr[6][6];
+#pragma unroll
+    for (int r = 0; r < 6; ++r)
+#pragma unroll
+        for (int c = 0; c < 6; ++c) hr[r][c] = hc(r - 1, c - 1);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            B.wh[i][j] = hr[i + 1][j] + hr[i + 1][j + 1];
+            B.wv[j][i] = hr[j][i + 1] + hr[j + 1][i + 1];
+        }
+#pragma unroll
+    for (int r = 0; r < 5; ++r)
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+            if (!((r == 0 && c == 4) || (r == 4 && c == 0)))
+                B.wb[r][c] = diag_weight(hr[r][c], hr[r + 1][c + 1], wmax);
+            if (!((r == 0 && c == 0) || (r == 4 && c == 4)))
+                B.ws[r][c] = diag_weight(hr[r][c + 1], hr[r + 1][c], wmax);
+        }
+    if (S.nrow < 4 || S.ncol < 4) {
+        auto out = [&](int r, int c) {   // own cells only: the ring's are never lowered
+            return r >= 0 && r < 4 && c >= 0 && c < 4 && (r >= S.nrow || c >= S.ncol);
+        };
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 5; ++j) {
+                if (out(i, j - 1) || out(i, j)) B.wh[i][j] = wmax;
+                if (out(j - 1, i) || out(j, i)) B.wv[j][i] = wmax;
             }
+#pragma unroll
+        for (int r = 0; r < 5; ++r)
+#pragma unroll
+            for (int c = 0; c < 5; ++c) {
+                if (out(r - 1, c - 1) || out(r, c)) B.wb[r][c] = wmax;
+                if (out(r - 1, c) || out(r, c - 1)) B.ws[r][c] = wmax;
+            }
+    }
+}
+
+// Which neighbours' border pixels this thread's border pixels improve (TB_*
+// bits).  changed: the block has changed (for a ring row that lies among the
+// blocks: any change of the last row's).  limit: below what distance each ring
+// pixel is improved (in ring_pixel's order); without it, below the staged one
+// (pixels outside the window are left to the settling pass).
+template <int MAXR>
+__device__ unsigned dist_offers(const DistTile<MAXR> &T, const TileGeo &g, const DistBlock &B,
+                                bool changed, const unsigned *limit = nullptr, unsigned win = 0) {
+    const int tid = threadIdx.x, bx = tid & 15, by = tid >> 4;
+    const int b = (by + 1) * RT_BX + bx + 1;
+    unsigned f = 0;
+    auto offers = [&](int r, int c, int r2, int c2, unsigned w) {
+        if (!limit) return B.d[r][c] + w < around(T.d, b, r2, c2);
+        const int lr = 4 * by + r2, lc = 4 * bx + c2;
+        const int i = r2 < 0 && by == 0 ? lc + 1
+                      : r2 > 3 && lr == MAXR ? RT_COLS + 2 + lc + 1
+                                             : 2 * (RT_COLS + 2) + 2 * lr + (c2 > 0 ? 1 : 0);
+        return B.d[r][c] < win && B.d[r][c] + w < limit[i];
+    };
+    bool up = false, down = false, left = false, right = false;
+    if (by == 0) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            up |= offers(0, c, -1, c, B.wv[0][c]);
+            if (c || bx) up |= offers(0, c, -1, c - 1, B.wb[0][c]);
+            if (c < 3 || bx < 15) up |= offers(0, c, -1, c + 1, B.ws[0][c + 1]);
+        }
+        if (bx == 0 && offers(0, 0, -1, -1, B.wb[0][0])) f |= TB_UL;
+        if (bx == 15 && offers(0, 3, -1, 4, B.ws[0][4])) f |= TB_UR;
+    }
+    if (g.rv == MAXR) {
+        if (4 * by + 4 == MAXR) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                down |= offers(3, c, 4, c, B.wv[4][c]);
+                if (c < 3 || bx < 15) down |= offers(3, c, 4, c + 1, B.wb[4][c + 1]);
+                if (c || bx) down |= offers(3, c, 4, c - 1, B.ws[4][c]);
+            }
+            if (bx == 0 && offers(3, 0, 4, -1, B.ws[4][0])) f |= TB_DL;
+            if (bx == 15 && offers(3, 3, 4, 4, B.wb[4][4])) f |= TB_DR;
+        }
+    } else if (changed && 4 * by < g.rv && 4 * by + 4 >= g.rv) {
+        // the ring row lies among the blocks: any change of the last row's
+        f |= TB_D | (bx == 0 ? TB_DL : 0u) | (bx == 15 ? TB_DR : 0u);
+    }
+    if (bx == 0) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            left |= offers(r, 0, r, -1, B.wh[r][0]);
+            if (r || by) left |= offers(r, 0, r - 1, -1, B.wb[r][0]);
+            if (4 * by + r + 1 < g.rv) left |= offers(r, 0, r + 1, -1, B.ws[r + 1][0]);
+        }
+    }
+    if (bx == 15) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            right |= offers(r, 3, r, 4, B.wh[r][4]);
+            if (r || by) right |= offers(r, 3, r - 1, 4, B.ws[r][4]);
+            if (4 * by + r + 1 < g.rv) right |= offers(r, 3, r + 1, 4, B.wb[r + 1][4]);
+        }
+    }
+    return f | (up ? TB_U : 0u) | (down ? TB_D : 0u) | (left ? TB_L : 0u) | (right ? TB_R : 0u);
 }
 
 // Solve tile (tx, ty), local index t.
@@ -337,7 +405,8 @@ __device__ void block_weights(const DistTile<MAXR> &T, int b, const Staged &S, D
 //           by then (pixels of the diagonal neighbours, which belong to tiles
 //           of the same half, stay unreached);
 //   AGAIN   from its current keys and the ring's.
-// The first two write every key of the tile, AGAIN a changed tile's.  Keys carry no label yet.
+// The first two write every key of the tile, AGAIN a changed tile's.  Keys
+// carry no label yet.
 // Returns, in every thread, what the solve did (TB_*; 0: nothing changed).
 template <int MAXR>
 __device__ unsigned solve_dist(const PairDev &P, int t, int tx, int ty, DistTile<MAXR> &T,
@@ -352,62 +421,12 @@ __device__ unsigned solve_dist(const PairDev &P, int t, int tx, int ty, DistTile
     unsigned f = mode != AGAIN ? TB_ANY : 0u;
     {
         block_weights(T, b, S, B);
-        unsigned before = 0, after = 0;   // (cells below the tile count, harmlessly)
-#pragma unroll
-        for (int i = 0; i < 16; ++i) before += B.d[i >> 2][i & 3];
+        const unsigned long long before = block_sum(B);   // (cells below the tile count, harmlessly)
         dist_rounds(T, B, b, 2 + RT_COLS * MAXR);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) after += B.d[i >> 2][i & 3];
+        const unsigned long long after = block_sum(B);
         if (before != after) f |= TB_ANY;
         if (mode == AGAIN && __syncthreads_or(before != after)) {
-            // which neighbours' border pixels, as this tile knows them, its
-            // own border pixels improve
-            auto offers = [&](int r, int c, int r2, int c2, unsigned w) {
-                return B.d[r][c] + w < around(T.d, b, r2, c2);
-            };
-            bool up = false, down = false, left = false, right = false;
-            if (by == 0) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    up |= offers(0, c, -1, c, B.wv[0][c]);
-                    if (c || bx) up |= offers(0, c, -1, c - 1, B.wb[0][c]);
-                    if (c < 3 || bx < 15) up |= offers(0, c, -1, c + 1, B.ws[0][c + 1]);
-                }
-                if (bx == 0 && offers(0, 0, -1, -1, B.wb[0][0])) f |= TB_UL;
-                if (bx == 15 && offers(0, 3, -1, 4, B.ws[0][4])) f |= TB_UR;
-            }
-            if (g.rv == MAXR) {
-                if (4 * by + 4 == MAXR) {
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        down |= offers(3, c, 4, c, B.wv[4][c]);
-                        if (c < 3 || bx < 15) down |= offers(3, c, 4, c + 1, B.wb[4][c + 1]);
-                        if (c || bx) down |= offers(3, c, 4, c - 1, B.ws[4][c]);
-                    }
-                    if (bx == 0 && offers(3, 0, 4, -1, B.ws[4][0])) f |= TB_DL;
-                    if (bx == 15 && offers(3, 3, 4, 4, B.wb[4][4])) f |= TB_DR;
-                }
-            } else if (before != after && 4 * by < g.rv && 4 * by + 4 >= g.rv) {
-                // the ring row lies among the blocks: any change of the last row's
-                f |= TB_D | (bx == 0 ? TB_DL : 0u) | (bx == 15 ? TB_DR : 0u);
-            }
-            if (bx == 0) {
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    left |= offers(r, 0, r, -1, B.wh[r][0]);
-                    if (r || by) left |= offers(r, 0, r - 1, -1, B.wb[r][0]);
-                    if (4 * by + r + 1 < g.rv) left |= offers(r, 0, r + 1, -1, B.ws[r + 1][0]);
-                }
-            }
-            if (bx == 15) {
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    right |= offers(r, 3, r, 4, B.wh[r][4]);
-                    if (r || by) right |= offers(r, 3, r - 1, 4, B.ws[r][4]);
-                    if (4 * by + r + 1 < g.rv) right |= offers(r, 3, r + 1, 4, B.wb[r + 1][4]);
-                }
-            }
-            f |= (up ? TB_U : 0u) | (down ? TB_D : 0u) | (left ? TB_L : 0u) | (right ? TB_R : 0u);
+            f |= dist_offers(T, g, B, before != after);
         }
     }
     if (f & TB_ANY) {

@@ -329,13 +329,81 @@ __device__ __forceinline__ void write_block(const PairDev &P, const TileGeo &g, 
     }
 }
 
+// Which neighbours' border pixels, as the tile knows them, this thread's border
+// pixels improve (TB_* bits; where weights need more than 32 bits, or the ring
+// row lies among the blocks: by its changed border pixels alone).
+template <int MAXR>
+__device__ unsigned settle_offers(const SettleTile<MAXR> &T, const TileGeo &g, const Block &B,
+                                  unsigned mask) {
+    const int tid = threadIdx.x, bx = tid & 15, by = tid >> 4;
+    const int b = (by + 1) * RT_BX + bx + 1;
+    const bool big = T.big != 0;
+    const int last = g.rv - 1 - 4 * by;   // the tile's bottom row in this block
+    bool up = false, down = false, left = false, right = false;
+    bool ul = false, ur = false, dl = false, dr = false;
+    if (big || g.rv < MAXR) {
+        up = by == 0 && (mask & 0xFu);
+        down = last >= 0 && last < 4 && ((mask >> (4 * last)) & 0xFu);
+        left = bx == 0 && (mask & 0x1111u);
+        right = bx == 15 && (mask & 0x8888u);
+        ul = up && left;
+        ur = up && right;
+        dl = down && left;
+        dr = down && right;
+    } else {
+        auto axis = [&](int r, int c, int r2, int c2, unsigned h) {
+            return key_axis(B.k[r][c], B.h[r][c], h) < around(T.K, b, r2, c2);
+        };
+        auto diag = [&](int r, int c, int r2, int c2, int e) {
+            return key_plus(B.k[r][c], T.wd[e][tid]) < around(T.K, b, r2, c2);
+        };
+        if (by == 0) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                up |= axis(0, c, -1, c, B.hn[c]);
+                if (c || bx) up |= diag(0, c, -1, c - 1, e_ul(0, c));
+                if (c < 3 || bx < 15) up |= diag(0, c, -1, c + 1, e_ur(0, c));
+            }
+            ul = bx == 0 && diag(0, 0, -1, -1, e_ul(0, 0));
+            ur = bx == 15 && diag(0, 3, -1, 4, e_ur(0, 3));
+        }
+        if (4 * by + 4 == MAXR) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                down |= axis(3, c, 4, c, B.hs[c]);
+                if (c || bx) down |= diag(3, c, 4, c - 1, e_ll(3, c));
+                if (c < 3 || bx < 15) down |= diag(3, c, 4, c + 1, e_lr(3, c));
+            }
+            dl = bx == 0 && diag(3, 0, 4, -1, e_ll(3, 0));
+            dr = bx == 15 && diag(3, 3, 4, 4, e_lr(3, 3));
+        }
+        if (bx == 0) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                left |= axis(r, 0, r, -1, B.hw[r]);
+                if (r || by) left |= diag(r, 0, r - 1, -1, e_ul(r, 0));
+                if (4 * by + r + 1 < MAXR) left |= diag(r, 0, r + 1, -1, e_ll(r, 0));
+            }
+        }
+        if (bx == 15) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                right |= axis(r, 3, r, 4, B.he[r]);
+                if (r || by) right |= diag(r, 3, r - 1, 4, e_ur(r, 3));
+                if (4 * by + r + 1 < MAXR) right |= diag(r, 3, r + 1, 4, e_lr(r, 3));
+            }
+        }
+    }
+    return (up ? TB_U : 0) | (down ? TB_D : 0) | (left ? TB_L : 0) | (right ? TB_R : 0) |
+           (ul ? TB_UL : 0) | (ur ? TB_UR : 0) | (dl ? TB_DL : 0) | (dr ? TB_DR : 0);
+}
+
 // Settle tile (tx, ty): relax it to its fixed point with the ring around it.
 // Returns what the solve did (TB_*; 0: nothing changed), the same in every
 // thread; the changed keys are written back (own_tiles fences them).
 template <int MAXR>
 __device__ unsigned settle_tile(const PairDev &P, int tx, int ty, SettleTile<MAXR> &T, RunState *st) {
-    const int tid = threadIdx.x, bx = tid & 15, by = tid >> 4;
-    const int b = (by + 1) * RT_BX + bx + 1;
+    const int tid = threadIdx.x;
     const TileGeo g = tile_geo(P, tx, ty);
     Block B;
     stage_tile(P, T, g, B, st);
@@ -345,70 +413,7 @@ __device__ unsigned settle_tile(const PairDev &P, int tx, int ty, SettleTile<MAX
         write_block(P, g, B, mask);
         f = TB_ANY;
     }
-    if (__syncthreads_or(mask != 0)) {
-        // which neighbours' border pixels, as this tile knows them, its own
-        // border pixels improve (weights that need more than 32 bits: by the
-        // changed border pixels alone)
-        const bool big = T.big != 0;
-        const int last = g.rv - 1 - 4 * by;   // the tile's bottom row in this block
-        bool up = false, down = false, left = false, right = false;
-        bool ul = false, ur = false, dl = false, dr = false;
-        if (big || g.rv < MAXR) {
-            up = by == 0 && (mask & 0xFu);
-            down = last >= 0 && last < 4 && ((mask >> (4 * last)) & 0xFu);
-            left = bx == 0 && (mask & 0x1111u);
-            right = bx == 15 && (mask & 0x8888u);
-            ul = up && left;
-            ur = up && right;
-            dl = down && left;
-            dr = down && right;
-        } else {
-            auto axis = [&](int r, int c, int r2, int c2, unsigned h) {
-                return key_axis(B.k[r][c], B.h[r][c], h) < around(T.K, b, r2, c2);
-            };
-            auto diag = [&](int r, int c, int r2, int c2, int e) {
-                return key_plus(B.k[r][c], T.wd[e][tid]) < around(T.K, b, r2, c2);
-            };
-            if (by == 0) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    up |= axis(0, c, -1, c, B.hn[c]);
-                    if (c || bx) up |= diag(0, c, -1, c - 1, e_ul(0, c));
-                    if (c < 3 || bx < 15) up |= diag(0, c, -1, c + 1, e_ur(0, c));
-                }
-                ul = bx == 0 && diag(0, 0, -1, -1, e_ul(0, 0));
-                ur = bx == 15 && diag(0, 3, -1, 4, e_ur(0, 3));
-            }
-            if (4 * by + 4 == MAXR) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    down |= axis(3, c, 4, c, B.hs[c]);
-                    if (c || bx) down |= diag(3, c, 4, c - 1, e_ll(3, c));
-                    if (c < 3 || bx < 15) down |= diag(3, c, 4, c + 1, e_lr(3, c));
-                }
-                dl = bx == 0 && diag(3, 0, 4, -1, e_ll(3, 0));
-                dr = bx == 15 && diag(3, 3, 4, 4, e_lr(3, 3));
-            }
-            if (bx == 0) {
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    left |= axis(r, 0, r, -1, B.hw[r]);
-                    if (r || by) left |= diag(r, 0, r - 1, -1, e_ul(r, 0));
-                    if (4 * by + r + 1 < MAXR) left |= diag(r, 0, r + 1, -1, e_ll(r, 0));
-                }
-            }
-            if (bx == 15) {
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    right |= axis(r, 3, r, 4, B.he[r]);
-                    if (r || by) right |= diag(r, 3, r - 1, 4, e_ur(r, 3));
-                    if (4 * by + r + 1 < MAXR) right |= diag(r, 3, r + 1, 4, e_lr(r, 3));
-                }
-            }
-        }
-        f |= (up ? TB_U : 0) | (down ? TB_D : 0) | (left ? TB_L : 0) | (right ? TB_R : 0) |
-             (ul ? TB_UL : 0) | (ur ? TB_UR : 0) | (dl ? TB_DL : 0) | (dr ? TB_DR : 0);
-    }
+    if (__syncthreads_or(mask != 0)) f |= settle_offers(T, g, B, mask);
     f = __reduce_or_sync(FULL, f);
     if (f && (tid & 31) == 0) atomicOr(&T.flags, f);
     __syncthreads();
