@@ -370,8 +370,8 @@ void epic_refine_params_default(epic_refine_params_t *p);
  * which each pixel's 2x2 (du, dv) system is solved exactly; derivatives are
  * central differences on edge-replicated images.  Device pointers (flow
  * 8-byte aligned, else EPIC_ERR_INVALID); the
- * handle holds about H*W*(channels + 12)*4 bytes of scratch (grown on demand,
- * EPIC_ERR_OOM if it cannot be).  Enqueued on `stream` without waiting; one
+ * handle holds about H*W*56 bytes of scratch (grown on demand, EPIC_ERR_OOM
+ * if it cannot be).  Enqueued on `stream` without waiting; one
  * refinement in flight per handle (the scratch is shared).  params NULL =
  * defaults. */
 int epic_refine(epic_interp_t *h, const float *I1, const float *I2, int H,
@@ -379,8 +379,9 @@ int epic_refine(epic_interp_t *h, const float *I1, const float *I2, int H,
                 const epic_refine_params_t *params, void *stream);
 
 /* Self-test of failure detection without a GPU fault.  Every device wait
- * of the library is bounded: the relaxation's grid barrier (2 s) and the TMA
- * staging's mbarrier wait (1 s) give up, record EPIC_ERR_TIMEOUT and let the
+ * of the library is bounded: the relaxation's grid barrier (2 s), its waits
+ * for other tiles and the refinement's (1 s) and the TMA staging's mbarrier
+ * wait (1 s) give up, record EPIC_ERR_TIMEOUT and let the
  * kernel return.  This runs one of those waits with a limit of limit_ms
  * (1..10000) where the awaited event never happens: which = 0, a grid
  * barrier that expects a second CTA which does not exist; which = 1, an

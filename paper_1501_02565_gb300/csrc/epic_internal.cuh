@@ -420,9 +420,10 @@ struct RefineArgs {
     float alpha0, gamma, kappa, eps, zeta, omega;
     int iterations, sor_iterations;
 };
-size_t refine_scratch_bytes(int H, int W, int C);
+size_t refine_scratch_bytes(int H, int W);
 cudaError_t launch_refine(const float *I1, const float *I2, int H, int W, int C, float *flow,
-                          const RefineArgs &r, void *scratch, int num_sms, cudaStream_t stream);
+                          const RefineArgs &r, void *scratch, int num_sms, RunState *state,
+                          cudaStream_t stream);
 
 // Image-gradient cost map.
 cudaError_t launch_gradcost(const float *img, int F, int H, int W, int channels, float floor_,

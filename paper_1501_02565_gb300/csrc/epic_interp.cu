@@ -1459,7 +1459,7 @@ int epic_refine(epic_interp_t *h, const float *I1, const float *I2, int H, int W
     cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
     cudaError_t e = cudaSetDevice(h->device);
     if (e != cudaSuccess) return cuda_fail(h, e, "cudaSetDevice");
-    const size_t need = epic::refine_scratch_bytes(H, W, channels);
+    const size_t need = epic::refine_scratch_bytes(H, W);
     if (need > h->rf_cap) {
         if ((e = cudaStreamSynchronize(stream)) != cudaSuccess)
             return cuda_fail(h, e, "cudaStreamSynchronize");
@@ -1474,7 +1474,8 @@ int epic_refine(epic_interp_t *h, const float *I1, const float *I2, int H, int W
     }
     epic::RefineArgs r{prm.alpha0, prm.gamma, prm.kappa, prm.eps, prm.zeta, prm.omega,
                        prm.iterations, prm.sor_iterations};
-    e = epic::launch_refine(I1, I2, H, W, channels, flow, r, h->rf_buf, h->num_sms, stream);
+    e = epic::launch_refine(I1, I2, H, W, channels, flow, r, h->rf_buf, h->num_sms, h->state,
+                            stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "refine launch");
     h->last_stream = stream;
     return EPIC_OK;
