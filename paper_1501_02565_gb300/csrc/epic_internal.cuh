@@ -85,7 +85,9 @@ __device__ __forceinline__ unsigned half_cost(float c, bool *bad) {
 // derives s from these two fields with this function, so they agree.
 constexpr int STAMP_PENDING = (int)0x80000000;   // a warp tile not yet written this run
 constexpr int MAX_UNIT_SHIFT = 20;
-constexpr int SWEEP_WARP = 2;   // relaxation schedule of the warp tiles
+constexpr int SWEEP_WARP = 2;        // relaxation schedule of the warp tiles
+constexpr int SWEEP_WARP_UNIT = 3;   // the same with the unit 2^-31 whatever the costs
+__host__ __device__ constexpr bool warp_tiles(int sweep) { return sweep >= SWEEP_WARP; }
 __host__ __device__ __forceinline__ int unit_shift_of(unsigned cmax_bits, int reach, int tw,
                                                       int th) {
     if (cmax_bits > 0x7f800000u) return 0;   // NaN or negative: reported as an invalid cost
@@ -179,8 +181,8 @@ struct PairDev {
     int seed_reach;
 };
 
-// The distance unit shift of a pair (0 for the sweep schedules of k_dt.cu,
-// which keep the unit 2^-31).
+// The distance unit shift of a pair (0 for the sweep schedules of k_dt.cu and
+// SWEEP_WARP_UNIT, which keep the unit 2^-31).
 __device__ __forceinline__ int unit_shift(const PairDev &P) {
     return P.sweep == SWEEP_WARP
                ? unit_shift_of(P.cmax_bits, P.seed_reach, P.tile_w, P.tile_h)

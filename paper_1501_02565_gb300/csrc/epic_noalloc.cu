@@ -28,24 +28,33 @@ using epic::pkey_t;
 
 constexpr int NA_MAX_PIXELS = 1 << 19;   // e.g. 1024 x 512
 constexpr int NA_MAX_MATCHES = 1 << 15;
-constexpr int NA_MAX_TILES = 1 << 14;
-constexpr int NA_TILE_W = 64, NA_TILE_H = 32, NA_APRON = 4;
+constexpr int NA_MAX_TILES = 1 << 14;    // of 64 x 32 pixels
+// Tiles of 64 x 16 pixels, what the tile autotuner picks for frames above
+// 64 K pixels: a call for 1024 x 436 takes 366 us by 64 x 32 apron tiles and
+// three argument copies, 219 us by these and one (timed in turn; k_relax.cu, its distance unit is held at 2^-31, so that what this entry
+// point refuses and how it rounds do not depend on the frame).
+constexpr int NA_TILE_W = 64, NA_TILE_H = 16, NA_TILES = 2 * NA_MAX_TILES;
 
 // byte offsets inside the scratch array (each 256-byte aligned)
 constexpr size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 constexpr size_t OFF_KEYS = 0;
 constexpr size_t OFF_TSTART = align256(OFF_KEYS + sizeof(pkey_t) * NA_MAX_PIXELS);
-constexpr size_t OFF_TFILL = align256(OFF_TSTART + sizeof(int) * (NA_MAX_TILES + 1));
-constexpr size_t OFF_TSEEDS = align256(OFF_TFILL + sizeof(int) * NA_MAX_TILES);
+constexpr size_t OFF_TFILL = align256(OFF_TSTART + sizeof(int) * (NA_TILES + 1));
+constexpr size_t OFF_TSEEDS = align256(OFF_TFILL + sizeof(int) * NA_TILES);
 constexpr size_t OFF_TSTAMP = align256(OFF_TSEEDS + sizeof(int) * NA_MAX_MATCHES);
-constexpr size_t OFF_DEG = align256(OFF_TSTAMP + sizeof(int) * NA_MAX_TILES);
+constexpr size_t OFF_REQ = align256(OFF_TSTAMP + sizeof(int) * NA_TILES);
+constexpr size_t OFF_DEG = align256(OFF_REQ + 2 * sizeof(unsigned) * NA_TILES);
 constexpr size_t OFF_WMIN = align256(OFF_DEG + sizeof(int) * NA_MAX_MATCHES);
 constexpr size_t OFF_INFO = align256(OFF_WMIN + sizeof(unsigned) * NA_MAX_MATCHES);
-constexpr size_t OFF_STATE = align256(OFF_INFO + 4 * sizeof(int));
-constexpr size_t OFF_PAIR = align256(OFF_STATE + sizeof(epic::RunState));
-constexpr size_t OFF_PREFIX = align256(OFF_PAIR + sizeof(epic::PairDev));
-constexpr size_t OFF_ARGS = align256(OFF_PREFIX + 5 * 2 * sizeof(int));
-constexpr size_t NA_SCRATCH_BYTES = align256(OFF_ARGS + sizeof(epic::BatchArgs));
+// what every call writes, in one copy
+struct CallBlock {
+    alignas(128) epic::RunState state;   // starts at zero
+    alignas(128) epic::PairDev pair;
+    alignas(128) epic::BatchArgs args;
+    int prefix[12];                     // of a one-pair batch: {0, count}
+};
+constexpr size_t OFF_CALL = align256(OFF_INFO + 4 * sizeof(int));
+constexpr size_t NA_SCRATCH_BYTES = align256(OFF_CALL + sizeof(CallBlock));
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NA_SCRATCH_BYTES];
 
@@ -70,7 +79,8 @@ extern "C" int epic_geodesic_labels_noalloc(const float *cost_map, const float *
     const long long P = (long long)H * W;
     const long long tiles_x = (W + NA_TILE_W - 1) / NA_TILE_W;
     const long long tiles_y = (H + NA_TILE_H - 1) / NA_TILE_H;
-    if (P > NA_MAX_PIXELS || N > NA_MAX_MATCHES || tiles_x * tiles_y > NA_MAX_TILES)
+    const long long tiles_32 = tiles_x * ((H + 31) / 32);
+    if (P > NA_MAX_PIXELS || N > NA_MAX_MATCHES || tiles_32 > NA_MAX_TILES)
         return EPIC_ERR_CAPACITY;
     unsigned char *base = nullptr;
     int rc = scratch_address(&base);
@@ -83,7 +93,9 @@ extern "C" int epic_geodesic_labels_noalloc(const float *cost_map, const float *
             cudaSuccess)
         return EPIC_ERR_CUDA;
 
-    epic::PairDev Pd{};
+    CallBlock call{};
+    CallBlock *dev_call = reinterpret_cast<CallBlock *>(base + OFF_CALL);
+    epic::PairDev &Pd = call.pair;
     Pd.C = cost_map;
     Pd.matches = reinterpret_cast<const float4 *>(matches);
     Pd.flow = nullptr;
@@ -94,7 +106,9 @@ extern "C" int epic_geodesic_labels_noalloc(const float *cost_map, const float *
     Pd.a = 1.f;
     Pd.tile_w = NA_TILE_W;
     Pd.tile_h = NA_TILE_H;
-    Pd.apron = NA_APRON;
+    Pd.apron = 0;
+    Pd.sweep = epic::SWEEP_WARP_UNIT;
+    Pd.stack = 1;
     Pd.tiles_x = (int)tiles_x;
     Pd.tiles_y = (int)tiles_y;
     Pd.hash_cap = 0;
@@ -106,27 +120,21 @@ extern "C" int epic_geodesic_labels_noalloc(const float *cost_map, const float *
     Pd.deg = reinterpret_cast<int *>(base + OFF_DEG);
     Pd.wmin = reinterpret_cast<unsigned *>(base + OFF_WMIN);
     Pd.info = reinterpret_cast<int *>(base + OFF_INFO);
-    epic::RunState *state = reinterpret_cast<epic::RunState *>(base + OFF_STATE);
-    // prefix arrays of a one-pair batch: {0, count}
     const int T = (int)(tiles_x * tiles_y);
-    const int prefix[10] = {0, T, 0, N, 0, 0, 0, 0, 0, 0};
-    if (cudaMemcpyAsync(base + OFF_PAIR, &Pd, sizeof(Pd), cudaMemcpyHostToDevice, stream) ||
-        cudaMemcpyAsync(base + OFF_PREFIX, prefix, sizeof(prefix), cudaMemcpyHostToDevice,
-                        stream) ||
-        // the run state (status, pass counters, barrier) starts at zero
-        cudaMemsetAsync(state, 0, sizeof(epic::RunState), stream))
-        return EPIC_ERR_CUDA;
-    // (copies from pageable host memory have consumed their source by the
-    // time cudaMemcpyAsync returns)
-    const int *pre = reinterpret_cast<const int *>(base + OFF_PREFIX);
-    epic::BatchArgs a{};
-    a.pairs = reinterpret_cast<const epic::PairDev *>(base + OFF_PAIR);
+    call.prefix[1] = call.prefix[11] = T;
+    call.prefix[3] = N;
+    const int *pre = dev_call->prefix;
+    epic::BatchArgs &a = call.args;
+    a.pairs = &dev_call->pair;
     a.npairs = 1;
     a.tile_base = pre + 0;
     a.match_base = pre + 2;
     a.chunk_base = pre + 4;
     a.hash_base = pre + 6;
     a.clear_base = pre + 8;
+    a.solve_base = pre + 10;
+    a.total_solve = T;
+    a.relax_req = reinterpret_cast<unsigned *>(base + OFF_REQ);
     a.total_tiles = T;
     a.total_matches = N;
     a.total_chunks = 0;
@@ -136,19 +144,18 @@ extern "C" int epic_geodesic_labels_noalloc(const float *cost_map, const float *
     a.max_passes = 4096;
     a.weight_squared = 1;
     a.fallback_eps = 1e-10f;
-    a.state = state;
-    const epic::BatchArgs *dev_a = reinterpret_cast<const epic::BatchArgs *>(base + OFF_ARGS);
-    if (cudaMemcpyAsync(base + OFF_ARGS, &a, sizeof(a), cudaMemcpyHostToDevice, stream))
+    a.state = &dev_call->state;
+    // (a copy from pageable host memory has consumed its source by the time
+    // cudaMemcpyAsync returns)
+    if (cudaMemcpyAsync(dev_call, &call, sizeof(call), cudaMemcpyHostToDevice, stream))
         return EPIC_ERR_CUDA;
     epic::LaunchCfg lc{num_sms, smem_optin, stream};
-    if (epic::launch_prepare(a, dev_a, lc) != cudaSuccess ||
-        epic::launch_dt(a, dev_a, lc, NA_TILE_W, NA_TILE_H, NA_APRON, false, nullptr) !=
-            cudaSuccess ||
-        epic::launch_split_keys(&Pd, reinterpret_cast<const epic::PairDev *>(base + OFF_PAIR),
-                                labels_out, dist_out, stream) != cudaSuccess)
+    if (epic::launch_prepare(a, &dev_call->args, lc) != cudaSuccess ||
+        epic::launch_relax(a, &dev_call->args, lc, NA_TILE_H, false, nullptr) != cudaSuccess ||
+        epic::launch_split_keys(&Pd, &dev_call->pair, labels_out, dist_out, stream) != cudaSuccess)
         return EPIC_ERR_CUDA;
     int status = 0;
-    if (cudaMemcpyAsync(&status, &state->status, sizeof(int), cudaMemcpyDeviceToHost, stream) ||
+    if (cudaMemcpyAsync(&status, &dev_call->state.status, sizeof(int), cudaMemcpyDeviceToHost, stream) ||
         cudaStreamSynchronize(stream))
         return EPIC_ERR_CUDA;
     return status;

@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(1024) prepare_kernel(const BatchArgs *__restri
         const int T = P.tiles_x * P.tiles_y;
         for (int t = threadIdx.x; t < T; t += blockDim.x) {
             P.tile_start[t] = 0;
-            if (P.sweep == SWEEP_WARP) P.tile_stamp[t] = STAMP_PENDING;
+            if (warp_tiles(P.sweep)) P.tile_stamp[t] = STAMP_PENDING;
         }
         for (int m = threadIdx.x; m < P.N; m += blockDim.x) {
             P.deg[m] = 0;
