@@ -150,8 +150,9 @@ struct PairDev {
     unsigned *wmin2;        // [N] float bits of the second-lightest edge (+inf if none)
     int *wnear;             // [N] other end of the lightest edge (-1 if none)
     int *row;               // [N + 1] CSR row offsets into adj
-    uint4 *adj;              // [2 * hash_cap] CSR rows: (neighbour, w bits, the
-                             // neighbour's lightest-edge bits, 0)
+    uint4 *adj;              // [2 * hash_cap] CSR rows: (neighbour, w bits, bits of
+                             // the neighbour's lightest other edge, the neighbour's
+                             // row_word)
     float4 *models;         // [N * 2] (c_u, c_v, b11, b12), (b21, b22, x_m, y_m)
     int *fallback;          // [N]
     int *knn_idx;           // [N*K] or null
@@ -187,6 +188,16 @@ __device__ __forceinline__ int unit_shift(const PairDev &P) {
     return P.sweep == SWEEP_WARP
                ? unit_shift_of(P.cmax_bits, P.seed_reach, P.tile_w, P.tile_h)
                : 0;
+}
+
+// A CSR row in a word: its first entry and its degree, ROW_LONG if they do not
+// fit (then P.row has them).
+constexpr int ROW_DEGREE_BITS = 10;
+constexpr unsigned ROW_LONG = 0xFFFFFFFFu;
+__host__ __device__ __forceinline__ unsigned row_word(int start, int degree) {
+    return start < (1 << (32 - ROW_DEGREE_BITS)) && degree < (1 << ROW_DEGREE_BITS) - 1
+               ? (unsigned)start << ROW_DEGREE_BITS | (unsigned)degree
+               : ROW_LONG;
 }
 
 struct GridBarrier {

@@ -33,9 +33,9 @@
 //                the K-NN search does not depend on it).
 // rowmin_kernel, bound_edge_kernel
 //                per node the two lightest edges; then in every entry
-//                (m -> n) the lightest edge at n other than (n, m).  The
-//                K-NN search reads it with the entry (no dependent load)
-//                for its step bound.
+//                (m -> n) the lightest edge at n other than (n, m), and n's
+//                row.  The K-NN search reads them with the entry (no
+//                dependent load) for its step bound and for n's own entries.
 #include "epic_internal.cuh"
 
 namespace epic {
@@ -434,7 +434,9 @@ __global__ void __launch_bounds__(256) bound_edge_kernel(const BatchArgs *__rest
         if (j >= P.row[P.N]) continue;
         const uint4 ed = P.adj[j];
         const int n = (int)ed.x, m = (int)ed.w;
-        P.adj[j].z = P.wnear[n] == m ? P.wmin2[n] : P.wmin[n];
+        const int r = P.row[n];
+        reinterpret_cast<uint2 *>(P.adj + j)[1] =
+            make_uint2(P.wnear[n] == m ? P.wmin2[n] : P.wmin[n], row_word(r, P.row[n + 1] - r));
     }
 }
 

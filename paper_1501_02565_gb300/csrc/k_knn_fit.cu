@@ -19,8 +19,8 @@
 // match needs ~5x fewer steps than one-node-at-a-time settling; excluding
 // the parent edge from the bound saves another ~13 % of the steps.
 // Per-warp shared memory holds
-//   * the frontier: packed keys (t bits << 32 | node), their table slots and
-//     t + w_x, rebuilt every step so that only current entries survive,
+//   * the frontier: distances, table slots, t + w_x and the nodes' CSR rows,
+//     rebuilt every step so that only current entries survive,
 //   * an open-addressing table node -> tentative distance (0 = settled):
 //     a lane claims a node's slot with compare-and-swap and lowers its
 //     distance with atomicMin, so several lanes may relax into one node,
@@ -35,11 +35,22 @@
 // kept, and every batch of the finished list is sorted before the fit.  All
 // edges of all batch nodes are relaxed in one pass: lanes take (node, edge)
 // pairs found from a warp prefix sum of the batch nodes' degrees (CSR row
-// lengths).  A newly pushed node's w_x comes with the adjacency entry
-// (precomputed per CSR entry by the graph stage), since the step's bound is
+// lengths).  A newly pushed node's w_x and its own CSR row come with the
+// adjacency entry (precomputed per CSR entry by the graph stage), so that a
+// batch's rows are at hand when it is settled and the step's bound is
 // kept as a running minimum over the entries pushed and kept (no separate
-// pass over the frontier).  The step's smallest
-// key and bound are then two 32-bit warp reductions (redux.sync).
+// pass over the frontier).  The step's smallest distance and bound are then two
+// 32-bit warp reductions (redux.sync); the smallest key's node is looked for
+// only where it decides.  Lanes find the batch node that owns their edge from
+// the ranges' starts as a bit mask and a popcount.
+//
+// What bounds it: instruction issue (73 % of the slots, 11 K warp
+// instructions per search of K = 100: 15 steps, 23 groups of 32 edges).  The
+// 64-pair mixed batch takes 5.38 ms, 2048 x 1024 299 us; with the rows loaded
+// when a batch is settled, keys of 64 bits in the frontier, the frontier read
+// twice in the last steps and the owner searched by shuffles 5.74 ms and 314
+// us.  Rows held beside the settled list instead of in it cost 128 bytes a warp
+// and with them table space: 5.57 ms and a quarter more for the second launch.
 //
 // The fit uses centred coordinates x~ = p_n - p_m and fits the flow
 // u = p' - p (the same least-squares problem as fitting p', Eq. 2, with
@@ -115,12 +126,12 @@ __device__ __forceinline__ void acc_add(F2 &acc, float v) {
 
 __device__ __forceinline__ double to_d(F2 v) { return (double)v.hi + (double)v.lo; }
 
-// One frontier entry: packed key (t bits << 32 | node), its node-table slot
-// and t + w_x, moved as one 16-byte access.
+// One frontier entry: distance (float bits), slot in the node table, t + w_x
+// and the node's CSR row (row_word), moved as one 16-byte access.
 struct __align__(16) FEnt {
-    pkey_t k;
-    unsigned sl;
+    unsigned t, sl;
     float tw;
+    unsigned row;
 };
 
 // Per-warp tables: frontier [fs], node table [hs] x 2 words, settled list
@@ -209,89 +220,94 @@ __global__ void __launch_bounds__(KNN_WARPS * 32, 4)
             hv[i] = DIST_INF;
         }
         __syncwarp();
-        // each lane's running minimum of the keys and of t + w_x over the
+        // each lane's running minimum of the distances and of t + w_x over the
         // frontier entries it kept or pushed since the last step: the step's
-        // smallest key and bound B are their warp minima.  Stale entries
-        // (a node pushed again with a smaller key) only add larger values
+        // smallest distance and bound B are their warp minima.  Stale entries
+        // (a node pushed again with a smaller distance) only add larger values
         // than the node's current entry, so the minima are exact.
-        pkey_t rk = EMPTY64;
+        unsigned rk = EMPTY32;
         float rb = __int_as_float(0x7f800000);
         if (lane == 0) {
             const unsigned s0 = node_slot((unsigned)m, HS);
             hk[s0] = (unsigned)m;
             hv[s0] = dist_word(0u);
-            rk = make_key(0.f, (unsigned)m);
+            rk = 0u;
             rb = __fadd_rn(0.f, __uint_as_float(__ldg(wmin + m)));
-            fe[0] = FEnt{rk, s0, rb};
+            const int r0 = __ldg(P.row + m);
+            fe[0] = FEnt{0u, s0, rb, row_word(r0, __ldg(P.row + m + 1) - r0)};
         }
         __syncwarp();
         int fn = 1, cnt = 0;
         bool overflow = false;
         while (cnt < K) {
-            // (1) smallest current key and the batch bound B, as warp
+            // (1) smallest current distance and the batch bound B, as warp
             //     reductions of 32-bit words: distances are non-negative, so
             //     their float bits order like the values (+inf included)
-            const unsigned kd = __reduce_min_sync(0xffffffffu, (unsigned)(rk >> 32));
-            const unsigned kn =
-                __reduce_min_sync(0xffffffffu, (unsigned)(rk >> 32) == kd ? (unsigned)rk : EMPTY32);
-            const pkey_t kmin = ((pkey_t)kd << 32) | kn;
+            const unsigned kd = __reduce_min_sync(0xffffffffu, rk);
             const float bound = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(rb)));
-            if (kmin == EMPTY64) break;  // component exhausted
-            rk = EMPTY64;
+            if (kd == EMPTY32) break;  // component exhausted
+            rk = EMPTY32;
             rb = __int_as_float(0x7f800000);
+            // the smallest key's node, where it counts: when no entry is below
+            // the bound, and for a batch cut to one key
+            auto smallest_node = [&]() {
+                unsigned n = EMPTY32;
+                for (int i = lane; i < fn; i += 32) {
+                    const FEnt f = fe[i];
+                    if (f.t == kd && hv[f.sl] == dist_word(kd)) n = min(n, hk[f.sl]);
+                }
+                return __reduce_min_sync(0xffffffffu, n);
+            };
+            const bool below = __uint_as_float(kd) < bound;
+            unsigned kn = below ? EMPTY32 : smallest_node();
             // (2) the batch: current entries below the bound (and the
             //     smallest).  A batch that reaches K is finished by sorting it
             //     in lanes; one reaching K with more than a warp of entries is
             //     cut to the smallest key alone.
             // (fn counts every frontier entry, an upper bound on the batch:
             // while cnt + fn < K the batch cannot reach K and is not counted)
+            auto load = [&](int i, FEnt &f) {   // whether entry i is current
+                f = FEnt{EMPTY32, 0u, 0.f, 0u};
+                if (i < fn) f = fe[i];
+                return i < fn && hv[f.sl] == dist_word(f.t);
+            };
+            auto in_batch = [&](const FEnt &f) {
+                return __uint_as_float(f.t) < bound || (!below && f.t == kd && hk[f.sl] == kn);
+            };
+            // (the frontier is 35 entries on average: up to 64 stay in registers
+            // for both passes)
+            FEnt f0, f1;
+            const bool v0 = load(lane, f0), v1 = fn > 32 && load(lane + 32, f1);
             int nwin = 0;
-            for (int b0 = 0; cnt + fn >= K && b0 < fn; b0 += 32) {
-                const int i = b0 + lane;
-                bool inb = false;
-                if (i < fn) {
-                    const FEnt f = fe[i];
-                    const pkey_t k = f.k;
-                    const unsigned cur = hv[f.sl];
-                    inb = cur == dist_word((unsigned)(k >> 32)) &&
-                          (key_dist(k) < bound || k == kmin);
+            if (cnt + fn >= K) {
+                nwin = __popc(__ballot_sync(0xffffffffu, v0 && in_batch(f0)));
+                if (fn > 32) nwin += __popc(__ballot_sync(0xffffffffu, v1 && in_batch(f1)));
+                for (int b0 = 64; b0 < fn; b0 += 32) {
+                    FEnt f;
+                    const bool v = load(b0 + lane, f);
+                    nwin += __popc(__ballot_sync(0xffffffffu, v && in_batch(f)));
                 }
-                nwin += __popc(__ballot_sync(0xffffffffu, inb));
             }
             const bool final_batch = cnt + nwin >= K && nwin <= 32;
             const bool single = cnt + nwin >= K && nwin > 32;
+            if (single && below) kn = smallest_node();
             // (3) partition: kept entries are compacted to the front (writes
             //     never pass reads); batch entries are settled into the list
             //     or, for the final batch, handed to lanes
             int wpos = 0, nb = 0;
             pkey_t bk = EMPTY64;
-            for (int b0 = 0; b0 < fn; b0 += 32) {
-                const int i = b0 + lane;
-                pkey_t k = EMPTY64;
-                unsigned sl = 0;
-                float tw = 0.f;
-                bool valid = false;
-                if (i < fn) {
-                    const FEnt f = fe[i];
-                    k = f.k;
-                    sl = f.sl;
-                    tw = f.tw;
-                    const unsigned cur = hv[sl];
-                    valid = cur == dist_word((unsigned)(k >> 32));
-                }
-                const bool inb = valid && (single ? k == kmin
-                                                  : (key_dist(k) < bound || k == kmin));
+            auto part = [&](const FEnt &f, bool valid) {
+                const bool inb = valid && (single ? f.t == kd && hk[f.sl] == kn : in_batch(f));
                 const bool keep = valid && !inb;
                 const unsigned kb = __ballot_sync(0xffffffffu, keep);
                 const unsigned bb = __ballot_sync(0xffffffffu, inb);
-                __syncwarp();
                 if (keep) {
-                    const int p = wpos + __popc(kb & lt_mask);
-                    fe[p] = FEnt{k, sl, tw};
-                    rk = k < rk ? k : rk;
-                    rb = fminf(rb, tw);
+                    fe[wpos + __popc(kb & lt_mask)] = f;
+                    rk = min(rk, f.t);
+                    rb = fminf(rb, f.tw);
                 }
                 if (final_batch) {
+                    const pkey_t k = inb ? ((pkey_t)f.t << 32) | hk[f.sl] : EMPTY64;
                     unsigned rem = bb;
                     while (rem) {
                         const int src = __ffs(rem) - 1;
@@ -303,15 +319,24 @@ __global__ void __launch_bounds__(KNN_WARPS * 32, 4)
                 } else {
                     if (inb) {
                         const int p = cnt + nb + __popc(bb & lt_mask);
-                        hv[sl] = SETTLED;
-                        rn[p] = key_label(k);
-                        rd[p] = key_dist(k);
-                        bs[p] = (unsigned short)cnt;
+                        hv[f.sl] = SETTLED;
+                        rn[p] = f.row;   // (node and batch start follow)
+                        rd[p] = __uint_as_float(f.t);
+                        bs[p] = (unsigned short)f.sl;
                     }
                     nb += __popc(bb);
                 }
                 wpos += __popc(kb);
                 __syncwarp();
+            };
+            __syncwarp();
+            part(f0, v0);
+            if (fn > 32) part(f1, v1);
+            for (int b0 = 64; b0 < fn; b0 += 32) {
+                FEnt f;
+                const bool v = load(b0 + lane, f);
+                __syncwarp();
+                part(f, v);
             }
             fn = wpos;
             if (final_batch) {
@@ -338,54 +363,66 @@ __global__ void __launch_bounds__(KNN_WARPS * 32, 4)
             }
             const int c0 = cnt;
             cnt += nb;
+            unsigned brow = ROW_LONG;   // CSR row of the batch's node `lane`
+            for (int i = lane; i < nb; i += 32) {
+                const unsigned sl = bs[c0 + i];
+                if (i < 32) brow = rn[c0 + i];
+                rn[c0 + i] = hk[sl];
+                bs[c0 + i] = (unsigned short)c0;
+            }
             __syncwarp();
             if (cnt >= K) break;
             // (4) relax every edge of every batch node in one pass
             for (int b0 = 0; b0 < nb && !overflow; b0 += 32) {
                 const int bi = b0 + lane;
                 const bool hb = bi < nb;
-                const pkey_t vk = hb ? make_key(rd[c0 + bi], rn[c0 + bi]) : EMPTY64;
+                const float vd = hb ? rd[c0 + bi] : 0.f;
                 // CSR row of the batch node: its first entry and its degree
                 int rbeg = 0, dg = 0;
                 if (hb) {
-                    const unsigned v = key_label(vk);
-                    rbeg = __ldg(P.row + v);
-                    dg = __ldg(P.row + v + 1) - rbeg;
+                    if (bi < 32 && brow != ROW_LONG) {
+                        rbeg = (int)(brow >> ROW_DEGREE_BITS);
+                        dg = (int)(brow & ((1u << ROW_DEGREE_BITS) - 1u));
+                    } else {
+                        const unsigned v = rn[c0 + bi];
+                        rbeg = __ldg(P.row + v);
+                        dg = __ldg(P.row + v + 1) - rbeg;
+                    }
                 }
-                // the chunk's batch nodes sit in lanes [0, nbc): the scan and
-                // the owner search need only ceil(log2 nbc) levels (batches
-                // average ~5 nodes)
+                // the chunk's batch nodes sit in lanes [0, nbc): the scan needs
+                // only ceil(log2 nbc) levels (batches average ~5 nodes)
                 const int nbc = min(nb - b0, 32);
-                int top = 1;
-                while (top < nbc) top <<= 1;
                 int incl = dg;
-                for (int o = 1; o < top; o <<= 1) {
+                for (int o = 1; o < nbc; o <<= 1) {
                     const int t = __shfl_up_sync(0xffffffffu, incl, o);
                     if (lane >= o) incl += t;
                 }
                 const int excl = incl - dg;
                 const int total = __shfl_sync(0xffffffffu, incl, nbc - 1);
+                const int rel = rbeg - excl;   // (edge e of the batch is entry rel + e)
+                const bool has = lane < nbc;
                 for (int e0 = 0; e0 < total; e0 += 32) {
                     const int e = e0 + lane;
-                    // owner: the last lane whose edge range starts at or before e
-                    int owner = 0;
-                    for (int stp = top >> 1; stp; stp >>= 1) {
-                        const int cand = owner + stp;
-                        const int ex = __shfl_sync(0xffffffffu, excl, cand & 31);
-                        if (cand < nbc && ex <= e) owner = cand;
-                    }
-                    const pkey_t ok = __shfl_sync(0xffffffffu, vk, owner);
-                    const int oex = __shfl_sync(0xffffffffu, excl, owner);
-                    const int obeg = __shfl_sync(0xffffffffu, rbeg, owner);
+                    // owner: the last node whose edge range starts at or before
+                    // e.  The starts within this window are its bits (nodes of
+                    // a batch have edges, so they differ), those before it are
+                    // counted.
+                    const unsigned starts = __reduce_or_sync(
+                        0xffffffffu, has && excl >= e0 && excl < e0 + 32 ? 1u << (excl - e0) : 0u);
+                    const int before = __popc(__ballot_sync(0xffffffffu, has && excl < e0));
+                    const int owner = before + __popc(starts & (lt_mask * 2u + 1u)) - 1;
+                    const float od = __shfl_sync(0xffffffffu, vd, owner);
+                    const int orel = __shfl_sync(0xffffffffu, rel, owner);
                     const bool act = e < total;
                     bool push = false;
-                    unsigned slot = 0, u = 0, uw = 0;
+                    unsigned slot = 0, uw = 0, urow = 0;
                     float nd = 0.f;
                     if (act) {
-                        const uint4 ed = __ldg(adj + obeg + (e - oex));
-                        u = ed.x;
+                        const uint4 ed = __ldg(adj + orel + e);
+                        const unsigned u = ed.x;
                         uw = ed.z;
-                        nd = __fadd_rn(key_dist(ok), __uint_as_float(ed.y));
+                        urow = ed.w;
+                        nd = __fadd_rn(od, __uint_as_float(ed.y));
                         unsigned sl = node_slot(u, HS);
                         int probes = 0;
                         for (;;) {
@@ -409,22 +446,16 @@ __global__ void __launch_bounds__(KNN_WARPS * 32, 4)
                         int w2 = 0;
                         for (int q0 = 0; q0 < fn; q0 += 32) {
                             const int i = q0 + lane;
-                            pkey_t k = 0;
-                            unsigned sl2 = 0;
-                            float tw2 = 0.f;
+                            FEnt f{0u, 0u, 0.f, 0u};
                             bool keep = false;
                             if (i < fn) {
-                                const FEnt f = fe[i];
-                                k = f.k;
-                                sl2 = f.sl;
-                                tw2 = f.tw;
-                                const unsigned cur = hv[sl2];
-                                keep = cur == dist_word((unsigned)(k >> 32));
+                                f = fe[i];
+                                keep = hv[f.sl] == dist_word(f.t);
                             }
                             const unsigned kb = __ballot_sync(0xffffffffu, keep);
                             __syncwarp();
                             if (keep) {
-                                fe[w2 + __popc(kb & lt_mask)] = FEnt{k, sl2, tw2};
+                                fe[w2 + __popc(kb & lt_mask)] = f;
                             }
                             w2 += __popc(kb);
                             __syncwarp();
@@ -434,10 +465,9 @@ __global__ void __launch_bounds__(KNN_WARPS * 32, 4)
                     }
                     if (push && !overflow) {
                         const int p = fn + __popc(bal & lt_mask);
-                        const pkey_t nk = make_key(nd, u);
                         const float tw = __fadd_rn(nd, __uint_as_float(uw));
-                        fe[p] = FEnt{nk, slot, tw};
-                        rk = nk < rk ? nk : rk;
+                        fe[p] = FEnt{__float_as_uint(nd), slot, tw, urow};
+                        rk = min(rk, __float_as_uint(nd));
                         rb = fminf(rb, tw);
                     }
                     fn += np;
