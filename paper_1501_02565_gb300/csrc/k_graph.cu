@@ -9,18 +9,26 @@
 // touching pair.  Each candidate D(p) + step(p, q) + D(q) is summed exactly
 // in the relaxation's fixed point and rounded once to float32.
 //
-// edges_kernel   every pixel looks at its four forward neighbours (right,
-//                down-left, down, down-right: each unordered pixel pair once)
-//                and forms (min label, max label, weight).  A work item is
-//                a stack of relaxation tiles at least 32 rows high.
-//                Candidates are merged per item (64 x 32 pixels hold only
-//                tens of distinct label pairs): first over the pixel's four directions, then
-//                across the lanes of a warp (match.any groups), then in a
-//                shared-memory table with atomicMin on the weight; the tile's
-//                unique entries are then inserted into the pair's global
-//                open-addressing table.  Tiles are taken from a counter.  A match whose source pixel is owned
-//                by a smaller index (a duplicate) is joined to the owner at
-//                distance D = 0.
+// edges_kernel   every pixel compares its label with its four forward
+//                neighbours' (right, down-left, down, down-right: each
+//                unordered pixel pair once).  The pairs that differ (about 0.8
+//                per pixel on a match per 90 pixels) are collected by the warp
+//                and processed 32 at a time, so that every lane has one:
+//                (min label, max label, weight) goes to a shared-memory table
+//                with the smallest weight of each pair, and the table's
+//                entries to the pair's global open-addressing table.  A work
+//                item is a stack of relaxation tiles of 32 rows, a tile or a
+//                part of one (edge_split), taken from a counter.  A match
+//                whose source pixel is owned by a smaller index (a duplicate)
+//                is joined to the owner at distance D = 0.
+//                64-pair mixed batch 742 us, 1024 x 436 22 us, 256 x 128 13.6
+//                us; with the weights computed pixel by pixel (most lanes of a
+//                warp idle), match.any groups per direction, items of 32 rows
+//                on every frame and an item's loads a few at a time 1131, 41
+//                and 34 us.  What bounds it: latency within an item (loads,
+//                table probes, barriers; five CTAs an SM).  All of a thread's
+//                probes of the global table in flight at once take a third
+//                off the flush and nothing off the whole.
 //                The insertion that creates an edge counts it in both
 //                endpoints' degrees; every insertion lowers both endpoints'
 //                lightest-edge weight.
@@ -77,47 +85,53 @@ constexpr int EDGE_ROWS = 32;     // a work item stacks relaxation tiles to this
 __host__ __device__ __forceinline__ int edge_stack(int tile_h) {
     return tile_h >= EDGE_ROWS ? 1 : EDGE_ROWS / tile_h;
 }
-
-// Claim the shared-table slot of key k (or find it); -1 if the probe
-// sequence is full.  A newly claimed slot is counted in *fill.
-__device__ __forceinline__ int smem_claim(pkey_t *sk, pkey_t k, int *fill) {
-    unsigned s = hash_slot(k, TILE_TABLE);
-    for (int probe = 0; probe < 64; ++probe) {
-        const pkey_t prev = atomicCAS(sk + s, EMPTY64, k);
-        if (prev == EMPTY64) atomicAdd(fill, 1);
-        if (prev == EMPTY64 || prev == k) return (int)s;
-        s = (s + 1) & (TILE_TABLE - 1);
+constexpr int EDGE_PAIRS = 128;
+__device__ __forceinline__ int find_pair_in(const int *base, int n, int i) {   // find_pair, of a shared copy
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (base[mid] <= i) lo = mid; else hi = mid - 1;
     }
-    return -1;
+    return lo;
+}
+// Runs of fewer tiles than this take an item per tile, or parts of a tile, so
+// that every SM has items: 2048 x 1024 (2048 tiles) takes 41 us by the tile, 48
+// stacked; 1024 x 436 (448 tiles) 22 us in halves, 23.5 in quarters, 41 stacked.
+constexpr int EDGE_STACK_TILES = 2432;
+__device__ __forceinline__ int edge_split(int total_tiles) {
+    return total_tiles < 304 ? 4 : total_tiles < 1216 ? 2 : 1;
 }
 
-// Insert one candidate per active lane.  Lanes holding the same label pair
-// are grouped with one match.any; the group's lowest lane claims the slot in
-// the shared table and every member lowers the slot's weight (or, if the
-// table is full, inserts straight into the global table).
-__device__ __forceinline__ void warp_insert(const PairDev &P, bool have, pkey_t k,
-                                            unsigned wbits, pkey_t *sk, unsigned *sw,
+// Lower the weight of pair k in the shared table (straight in the global table
+// if the probe sequence is full).  A newly claimed slot is counted in *fill.
+// The pairs along a cell boundary repeat: a look at the slot and at its weight
+// comes before either atomic.
+__device__ __forceinline__ void smem_insert(const PairDev &P, pkey_t k, unsigned wbits, pkey_t *sk, unsigned *sw,
                                             int *fill, RunState *st) {
-    if (!__any_sync(0xffffffffu, have)) return;
-    const unsigned lane = threadIdx.x & 31;
-    const unsigned grp = __match_any_sync(0xffffffffu, have ? k : EMPTY64);
-    const int leader = __ffs(grp) - 1;
-    int slot = -1;
-    if (have && lane == (unsigned)leader) slot = smem_claim(sk, k, fill);
-    slot = __shfl_sync(0xffffffffu, slot, leader);
-    if (have) {
-        if (slot >= 0)
-            atomicMin(sw + slot, wbits);
-        else
-            table_insert(P, k, wbits, st);
+    unsigned s = hash_slot(k, TILE_TABLE);
+    for (int probe = 0; probe < 64; ++probe) {
+        pkey_t cur = *(volatile pkey_t *)(sk + s);
+        if (cur == EMPTY64) {
+            cur = atomicCAS(sk + s, EMPTY64, k);
+            if (cur == EMPTY64) {
+                atomicAdd(fill, 1);
+                cur = k;
+            }
+        }
+        if (cur == k) {
+            if (*(volatile unsigned *)(sw + s) > wbits) atomicMin(sw + s, wbits);
+            return;
+        }
+        s = (s + 1) & (TILE_TABLE - 1);
     }
+    table_insert(P, k, wbits, st);
 }
 
 __global__ void __launch_bounds__(EDGE_THREADS) edges_kernel(const BatchArgs *__restrict__ ap) {
     const BatchArgs a = *ap;
     RunState *st = a.state;
     if (get_status(st) != 0) return;
-    __shared__ int s_tile, s_pair, s_local;
+    __shared__ int s_tile, s_sub, s_pair, s_local;
     __shared__ pkey_t sk[TILE_TABLE];
     __shared__ unsigned sw[TILE_TABLE];
     // the shared table collects the edges of consecutive tiles of one pair
@@ -143,20 +157,36 @@ __global__ void __launch_bounds__(EDGE_THREADS) edges_kernel(const BatchArgs *__
     // row below (every forward neighbour), staged with coalesced loads that
     // are all in flight at once; cells outside the image hold KEY_INF
     extern __shared__ __align__(16) unsigned char edge_smem[];
-    // tiles are handed out from a counter: their cost varies with the number
+    // a warp's candidates: (cell of p) * 4 + direction
+    __shared__ unsigned s_cand[EDGE_THREADS / 32][5 * 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    unsigned *cand = s_cand[wid];
+    // the prefix of tiles, for batches of few pairs
+    __shared__ int s_base[EDGE_PAIRS];
+    const bool s_few = a.npairs <= EDGE_PAIRS;
+    if (s_few)
+        for (int i = threadIdx.x; i < a.npairs; i += EDGE_THREADS) s_base[i] = a.tile_base[i];
+    __syncthreads();
+    int next = threadIdx.x == 0 ? (int)atomicAdd(&st->edge_next, 1u) : 0;   // thread 0: the next item
+    const int split = edge_split(a.total_tiles);
+    const bool stacked = a.total_tiles >= EDGE_STACK_TILES;
+    // items are handed out from a counter: their cost varies with the number
     // of cell boundaries they hold
     for (;;) {
         if (threadIdx.x == 0) {
-            // an item starts at every edge_stack-th row of tiles; the tiles
-            // in between belong to the item above them
+            // a stacked item starts at every edge_stack-th row of tiles; the
+            // tiles in between belong to the item above them
             for (;;) {
-                const int t = (int)atomicAdd(&st->edge_next, 1u);
+                const int u = next, t = u / split;
+                next = (int)atomicAdd(&st->edge_next, 1u);   // (not waited for until the next item)
                 s_tile = t;
+                s_sub = u - t * split;
                 if (t >= a.total_tiles) break;
-                const int pi = find_pair(a.tile_base, a.npairs, t);
+                const int pi = s_few ? find_pair_in(s_base, a.npairs, t) : find_pair(a.tile_base, a.npairs, t);
                 const PairDev &Q = a.pairs[pi];
                 const int lt = t - a.tile_base[pi];
-                if ((lt / Q.tiles_x) % edge_stack(Q.tile_h) == 0) {
+                if (!stacked || (lt / Q.tiles_x) % edge_stack(Q.tile_h) == 0) {
                     s_pair = pi;
                     s_local = lt;
                     break;
@@ -181,113 +211,112 @@ __global__ void __launch_bounds__(EDGE_THREADS) edges_kernel(const BatchArgs *__
         const pkey_t *keys = P.keys;
         const float *C = P.C;
         const int tx = s_local % TX, ty = s_local / TX;
-        const int RH = edge_stack(TH) * TH;   // rows of the item
-        const int npx = TW * RH;
+        // rows of the item: a stack of tiles, a tile or a part of one
+        const int sub_h = (TH + split - 1) / split;
+        const int yb = ty * TH + s_sub * sub_h;
+        const int RH = stacked ? edge_stack(TH) * TH : min(sub_h, TH - s_sub * sub_h);
+        if (RH <= 0) {   // (a tile of fewer rows than parts)
+            __syncthreads();
+            continue;
+        }
         const int SC = TW + 2, SR = RH + 1;   // staged columns x0-1 .. x0+tw
         const int us = unit_shift(P);                      // the pair's distance unit
         const float unit = ldexpf(ONE_PER_UNIT, us);       // the distance of one unit
-        pkey_t *skey = reinterpret_cast<pkey_t *>(edge_smem);
-        unsigned *sh = reinterpret_cast<unsigned *>(skey + SC * SR);
+        // keys in two planes (the first pass reads labels only)
+        unsigned *klo = reinterpret_cast<unsigned *>(edge_smem);
+        unsigned *khi = klo + SC * SR, *sh = khi + SC * SR;
+        const int x0 = tx * TW;
         {
-            // warp w stages rows w, w + 8, ...; its lanes take consecutive columns
-            const int x0 = tx * TW - 1, y0 = ty * TH;
-            const int nw = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+            // STAGE cells per thread at a time, for their loads to overlap
+            constexpr int STAGE = 5;
+            const unsigned inv = 0xFFFFFFFFu / (unsigned)SC + 1;   // (cell * inv) >> 32 is its row
             bool bad = false;
-            for (int r = wid; r < SR; r += nw) {
-                const int gy = y0 + r;
-                for (int c = lane; c < SC; c += 32) {
-                    const int gx = x0 + c;
-                    const bool in = gx >= 0 && gx < W && gy < H;
-                    const size_t q = (size_t)gy * W + gx;
-                    skey[r * SC + c] = in ? __ldg(keys + q) : KEY_INF;
-                    sh[r * SC + c] = in ? half_cost_s(__ldg(C + q), us, &bad) : 0u;
+            for (int i0 = threadIdx.x; i0 < SC * SR; i0 += STAGE * EDGE_THREADS) {
+                pkey_t k[STAGE];
+                float f[STAGE];
+#pragma unroll
+                for (int j = 0; j < STAGE; ++j) {
+                    const int i = i0 + j * EDGE_THREADS;
+                    const int r = __umulhi(i, inv), gx = x0 - 1 + i - r * SC, gy = yb + r;
+                    k[j] = KEY_INF;
+                    f[j] = 0.f;
+                    if (i < SC * SR && gx >= 0 && gx < W && gy < H) {
+                        const size_t q = (size_t)gy * W + gx;
+                        k[j] = __ldg(keys + q);
+                        f[j] = __ldg(C + q);
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < STAGE; ++j) {
+                    const int i = i0 + j * EDGE_THREADS;
+                    if (i >= SC * SR) break;
+                    klo[i] = (unsigned)k[j];
+                    khi[i] = (unsigned)(k[j] >> 32);
+                    sh[i] = half_cost_s(f[j], us, &bad);
                 }
             }
         }
         __syncthreads();
-        // tile widths are powers of two for the warp tiles (64): a shift
-        const int tws = (TW & (TW - 1)) == 0 ? __ffs(TW) - 1 : -1;
-        for (int i0 = 0; i0 < npx; i0 += blockDim.x) {  // warp-uniform trip count
-            const int i = i0 + threadIdx.x;
-            const int ly = tws >= 0 ? i >> tws : i / TW, lx = i - ly * TW;
-            const int x = tx * TW + lx, y = ty * TH + ly;
-            const bool act = i < npx && x < W && y < H;
-            pkey_t kp = 0;
-            unsigned hp = 0;
-            if (act) {
-                kp = skey[ly * SC + lx + 1];
-                hp = sh[ly * SC + lx + 1];
-            }
-            // the four forward candidates of this pixel; a label pair seen in
-            // an earlier direction is folded into that one (min weight), so
-            // a pixel inserts each pair once
-            pkey_t ck[4];
-            unsigned cw[4];
-            bool cv[4];
-#pragma unroll
-            for (int d = 0; d < 4; ++d) {
-                const int dx = d == 0 ? 1 : d == 1 ? -1 : d == 2 ? 0 : 1;
-                const int dy = d == 0 ? 0 : 1;
-                const int qx = x + dx, qy = y + dy;
-                bool have = act && qx >= 0 && qx < W && qy < H;
-                pkey_t k = 0;
-                unsigned wb = 0;
-                const int sq = (ly + dy) * SC + lx + 1 + dx;   // staged cell of q
-                if (have) {
-                    const pkey_t kq = skey[sq];
-                    const unsigned lp = key_label(kp), lq = key_label(kq);
-                    have = lp != lq;
-                    if (have && (lp >= NM || lq >= NM ||
-                                 !key_reached(kp) || !key_reached(kq))) {
-                        // an unreached pixel (or a distance beyond the fixed-
-                        // point range): the cost map was not in [0, C_MAX)
-                        set_status(st, EPIC_ERR_INVALID);
-                        have = false;
-                    }
-                    if (have) {
-                        const unsigned hq = sh[sq];
-                        const unsigned long long stp = (dx != 0 && dy != 0)
-                                                           ? step_diag(hp, hq)
-                                                           : step_axis(hp, hq);
-                        // exact sum in fixed point, rounded once to float32
-                        const unsigned long long units = key_dunits(kp) + stp + key_dunits(kq);
-                        const float w = __fmul_rn(__ull2float_rn(units), unit);   // units_dist
-                        k = lp < lq ? (((pkey_t)lp << 32) | lq) : (((pkey_t)lq << 32) | lp);
-                        wb = __float_as_uint(w);
-                    }
-                }
-#pragma unroll
-                for (int j = 0; j < d; ++j) {
-                    if (have && cv[j] && ck[j] == k) {
-                        cw[j] = min(cw[j], wb);
-                        have = false;
-                    }
-                }
-                ck[d] = k;
-                cw[d] = wb;
-                cv[d] = have;
-            }
-            // this pixel's distinct candidates to the front (usually one or
-            // two of the four directions), then one warp insertion round per
-            // candidate rank that any lane holds
-#pragma unroll
-            for (int d = 1; d < 4; ++d) {
-#pragma unroll
-                for (int j = 0; j < d; ++j) {
-                    if (!cv[j] && cv[d]) {
-                        ck[j] = ck[d];
-                        cw[j] = cw[d];
-                        cv[j] = true;
-                        cv[d] = false;
-                    }
+        // A warp walks strips of 32 columns down: a pixel's labels and its
+        // neighbours' are compared, and the pairs that differ are collected,
+        // 32 at a time with every lane at work on one.
+        int n = 0;   // of the warp's candidates
+        auto take = [&](int first, int count) {
+            __syncwarp();
+            if (lane < count) {
+                const unsigned code = cand[first + lane];
+                const int p = (int)(code >> 2), dir = (int)(code & 3u);
+                const int q = p + (dir == 0 ? 1 : SC - 2 + dir);
+                const pkey_t kp = (pkey_t)khi[p] << 32 | klo[p], kq = (pkey_t)khi[q] << 32 | klo[q];
+                const unsigned lp = key_label(kp), lq = key_label(kq);
+                if (lp >= NM || lq >= NM || !key_reached(kp) || !key_reached(kq)) {
+                    // an unreached pixel (or a distance beyond the fixed-
+                    // point range): the cost map was not in [0, C_MAX)
+                    set_status(st, EPIC_ERR_INVALID);
+                } else {
+                    const unsigned long long stp = (dir & 1) ? step_diag(sh[p], sh[q]) : step_axis(sh[p], sh[q]);
+                    // exact sum in fixed point, rounded once to float32
+                    const unsigned long long units = key_dunits(kp) + stp + key_dunits(kq);
+                    const float w = __fmul_rn(__ull2float_rn(units), unit);   // units_dist
+                    const pkey_t k = lp < lq ? (((pkey_t)lp << 32) | lq) : (((pkey_t)lq << 32) | lp);
+                    smem_insert(P, k, __float_as_uint(w), sk, sw, &s_fill, st);
                 }
             }
-#pragma unroll
-            for (int d = 0; d < 4; ++d) {
-                if (!__any_sync(0xffffffffu, cv[d])) break;
-                warp_insert(P, cv[d], ck[d], cw[d], sk, sw, &s_fill, st);
+            __syncwarp();
+        };
+        const int groups = (TW + 31) / 32;                                  // of columns
+        const int strip = (RH * groups + EDGE_THREADS / 32 - 1) / (EDGE_THREADS / 32);   // rows of a strip
+        const int strips = groups * ((RH + strip - 1) / strip);
+        for (int w = wid; w < strips; w += EDGE_THREADS / 32) {
+            const int r0 = w / groups * strip, r1 = min(r0 + strip, RH);
+            const int lx = (w % groups) * 32 + lane, x = x0 + lx;
+            const bool col = lx < TW && x < W;
+            const bool left = col && x > 0, right = col && x + 1 < W;
+            const int c = min(lx, TW - 1) + 1;   // staged column
+            unsigned lp = klo[r0 * SC + c] & LABEL_NONE, lr = klo[r0 * SC + c + 1] & LABEL_NONE;
+            for (int r = r0; r < r1 && yb + r < H; ++r) {
+                const bool down = yb + r + 1 < H;
+                const unsigned *below = klo + (r + 1) * SC + c;
+                const unsigned l1 = below[-1] & LABEL_NONE, l2 = below[0] & LABEL_NONE, l3 = below[1] & LABEL_NONE;
+                const unsigned code = (unsigned)(r * SC + c) * 4u;
+                auto push = [&](bool have, unsigned dir) {
+                    const unsigned b = __ballot_sync(0xffffffffu, have);
+                    if (have) cand[n + __popc(b & lt_mask)] = code + dir;
+                    n += __popc(b);
+                };
+                push(right && lp != lr, 0u);
+                push(left && down && lp != l1, 1u);
+                push(col && down && lp != l2, 2u);
+                push(right && down && lp != l3, 3u);
+                lp = l2;
+                lr = l3;
+                while (n >= 32) {
+                    n -= 32;
+                    take(n, 32);
+                }
             }
         }
+        take(0, n);
         __syncthreads();
     }
     if (s_tab_pair >= 0) flush_table(a.pairs[s_tab_pair]);
