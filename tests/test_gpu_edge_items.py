@@ -1,7 +1,7 @@
 """The graph's edges (edges_kernel in csrc/k_graph.cu) where its work items
 change: parts of a tile, tiles and stacks of tiles (chosen by the number of
-tiles), tile heights that do not divide into parts, frames narrower than a warp
-and cut tiles.  The set of edges must be the set of label pairs that touch in
+tiles), tile heights that do not divide into parts, tiles taller than the rows
+staged at once, frames narrower than a warp and cut tiles.  The set of edges must be the set of label pairs that touch in
 the GPU's own assignment map, and each weight the smallest D(p) + step + D(q)
 along the border, computed here in float64 from the float32 distances (parity.py's
 tolerance of weights)."""
@@ -38,6 +38,8 @@ def _edges(C, L, D):
     (100, 131, 300, {"tile_w": 64, "tile_h": 7, "sweep": 2}), (131, 300, 900, {"tile_w": 256, "tile_h": 16, "sweep": 0}),
     (61, 90, 200, {"tile_w": 8, "tile_h": 8, "sweep": 0}), (436, 1024, 5000, {}), (375, 1242, 4000, {}),
     (1100, 1500, 9000, {}), (1300, 2048, 20000, {}), (700, 64, 2, {}),
+    (150, 300, 400, {"tile_w": 256, "tile_h": 70, "apron": 0, "sweep": 0}),
+    (300, 200, 300, {"tile_w": 64, "tile_h": 256, "apron": 0, "sweep": 0}),
 ])
 def test_edges_of_the_assignment_map(H, W, N, cfg):
     rng = np.random.default_rng(H + W)
