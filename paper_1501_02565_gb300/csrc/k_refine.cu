@@ -558,8 +558,8 @@ size_t refine_scratch_bytes(int H, int W) {
            rf_align((SOR_MAX_TILES + 1) * sizeof(unsigned));
 }
 
-cudaError_t launch_refine(const float *I1, const float *I2, int H, int W, int C, float *flow,
-                          const RefineArgs &r, void *scratch, int num_sms, RunState *state, cudaStream_t stream) {
+static cudaError_t refine_frames(const float *I1, const float *I2, int H, int W, int C, float *flow,
+                          const RefineArgs &r, void *scratch, int num_sms, RunState *state, cudaStream_t stream, bool one_launch) {
     const size_t P = (size_t)H * W;
     char *base = static_cast<char *>(scratch);
     auto take = [&](size_t bytes) {
@@ -574,7 +574,7 @@ cudaError_t launch_refine(const float *I1, const float *I2, int H, int W, int C,
     x.swap[1] = reinterpret_cast<ulonglong2 *>(take(P * sizeof(ulonglong2)));
     x.progress = reinterpret_cast<unsigned *>(take((SOR_MAX_TILES + 1) * sizeof(unsigned)));
     SorGrid g;
-    const bool one_wave = sor_one_wave(W, H, num_sms, &g);
+    const bool one_wave = one_launch && sor_one_wave(W, H, num_sms, &g);
     if (!one_wave) g = sor_grid_of(64, 48, W, H);
     const int threads = sor_threads(g);
     const int nhalf = 2 * r.sor_iterations;
@@ -625,6 +625,15 @@ cudaError_t launch_refine(const float *I1, const float *I2, int H, int W, int C,
         }
     }
     return cudaSuccess;
+}
+
+cudaError_t launch_refine(const float *I1, const float *I2, int H, int W, int C, float *flow,
+                          const RefineArgs &r, void *scratch, int num_sms, RunState *state, cudaStream_t stream) {
+    cudaError_t e = refine_frames(I1, I2, H, W, C, flow, r, scratch, num_sms, state, stream, true);
+    if (e != cudaErrorCooperativeLaunchTooLarge) return e;
+    // a context with a part of the GPU's SMs
+    cudaGetLastError();
+    return refine_frames(I1, I2, H, W, C, flow, r, scratch, num_sms, state, stream, false);
 }
 
 }  // namespace epic
