@@ -135,10 +135,10 @@ typedef struct {
                              Every schedule gives the same result. */
     long long exact_chunk_bytes; /* epic_exact_interp with metric 0: device
                              bytes of packed keys its single-source
-                             relaxations may hold at once (8 bytes per pixel
-                             per match); at most
-                             max(1, min(N, exact_chunk_bytes / (8 H W)))
-                             matches run at a time.
+                             relaxations may hold at once, in tiles of 64 x
+                             32 pixels (16 KiB) that a match in work has
+                             reached; at least one match is in work, with
+                             every tile of the frame.
                              0 = 1 GiB (default).  Only speed and memory
                              depend on it, never the results. */
 } epic_config_t;

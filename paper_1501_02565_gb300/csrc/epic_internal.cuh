@@ -402,10 +402,13 @@ struct SingleArgs {
     const pkey_t *cap;       // [H*W] distances beyond a pixel's cap are not needed
     int H, W, N;
     int tiles_x, tiles_y;    // of SINGLE_W x SINGLE_H pixels
-    // per CTA: keys [H*W], then [tiles] each of a queue, the tiles touched,
-    // the tiles' places in the queue and their flags
+    const int *list;         // [N] the matches, null: all in order
+    // per CTA: keys [pool_tiles][SINGLE_TILE], then [tiles] each of a queue,
+    // the tiles touched, the tiles' places in the pool and in the queue and
+    // their flags
     pkey_t *keys;
-    int *queue, *touched;
+    int pool_tiles;
+    int *queue, *touched, *place_of;
     unsigned *place;
     unsigned char *flags;
     // distance tiles: `used` counts all that are needed, the first `slot_cap`
@@ -414,6 +417,8 @@ struct SingleArgs {
     int2 *slot_of;           // [slot_cap] (tile, match)
     unsigned slot_cap;
     unsigned *used, *next;   // (next: match dispenser)
+    int *left;               // matches that touch more tiles than a pool holds
+    unsigned *left_count;
     int *tile_count;         // [tiles + 1]
     int *tile_start;         // [tiles + 1]
     int2 *tile_entry;        // [slot_cap] (match, distance tile) by tile

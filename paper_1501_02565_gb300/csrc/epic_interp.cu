@@ -1275,20 +1275,30 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
     const size_t o_vints = take(sizeof(int) * v_ints);
     const size_t o_vinit = take(sizeof(unsigned long long) * (size_t)N);
     const size_t o_aflow = take(sizeof(float) * 2 * (size_t)P);
-    // single-source runs: a key map and a tile list per CTA, as many as the
-    // budget for keys allows and the GPU holds
+    // single-source runs: a pool of key tiles and a tile list per CTA, as many
+    // as the budget for keys allows and the GPU holds
     const int sx = (W + epic::SINGLE_W - 1) / epic::SINGLE_W;
     const int sy = (H + epic::SINGLE_H - 1) / epic::SINGLE_H;
     const long long ST = (long long)sx * sy;
     const long long chunk_bytes = c.exact_chunk_bytes > 0 ? c.exact_chunk_bytes : (1LL << 30);
-    const int ctas = (int)std::max(1LL, std::min({(long long)N, chunk_bytes / (P * 8),
-                                                  (long long)epic::single_resident(h->num_sms)}));
-    const size_t o_keys = take(sizeof(pkey_t) * (size_t)P * ctas);
+    // (a pool of 64 tiles holds what a match touches on the flow workloads, 14
+    // on average, several times; the few that touch more run a second time,
+    // with pools of all tiles)
+    const long long tile_bytes = (long long)sizeof(pkey_t) * epic::SINGLE_TILE;
+    const long long resident = epic::single_resident(h->num_sms);
+    auto ctas_for = [&](long long pool) {
+        return (int)std::max(1LL, std::min({(long long)N, chunk_bytes / (pool * tile_bytes), resident}));
+    };
+    const int ctas_all = ctas_for(ST), ctas = std::max(ctas_all, ctas_for(std::min(ST, 64LL)));
+    const int pool = (int)(ctas == ctas_all ? ST : std::min(ST, chunk_bytes / (ctas * tile_bytes)));
+    const size_t o_keys = take((size_t)tile_bytes * std::max((size_t)ctas_all * (size_t)ST, (size_t)ctas * (size_t)pool));
+    const size_t o_left = take(sizeof(int) * (size_t)N);
+    const size_t o_places = take(sizeof(int) * (size_t)ST * ctas);
     const size_t o_queue = take(sizeof(int) * (size_t)ST * ctas);
     const size_t o_touched = take(sizeof(int) * (size_t)ST * ctas);
     const size_t o_place = take(sizeof(unsigned) * (size_t)ST * ctas);
     const size_t o_flags = take((size_t)ST * ctas);
-    const size_t o_count = take(sizeof(int) * (size_t)(ST + 4));   // tile counts, then used and next
+    const size_t o_count = take(sizeof(int) * (size_t)(ST + 4));   // tile counts, then used, next and left
     const size_t o_start = take(sizeof(int) * (size_t)(ST + 1));
     if ((rc = grow(&h->ex_buf, &h->ex_cap, used))) return rc;
     char *b = h->ex_buf;
@@ -1378,6 +1388,9 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
     s.tile_count = reinterpret_cast<int *>(b + o_count);
     s.used = reinterpret_cast<unsigned *>(s.tile_count + ST);
     s.next = s.used + 1;
+    s.left_count = s.used + 2;
+    s.left = reinterpret_cast<int *>(b + o_left);
+    s.place_of = reinterpret_cast<int *>(b + o_places);
     s.tile_start = reinterpret_cast<int *>(b + o_start);
     s.max_solves = (long long)c.max_passes * ST;
     s.state = h->state;
@@ -1385,7 +1398,8 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
     // workloads at K = 100); a run that needs more says how many
     const size_t per_slot = sizeof(float) * epic::SINGLE_TILE + 2 * sizeof(int2);
     unsigned long long want = std::min<unsigned long long>((unsigned long long)N * ST, 16ull * N + 1024);
-    unsigned n_used = 0;
+    unsigned n_used = 0, n_done[3];   // used, next, left
+    s.pool_tiles = pool;
     for (;;) {
         want = std::max<unsigned long long>(want, h->ex_slots_cap / per_slot);
         want = std::min<unsigned long long>(want, 0x7fffffffull);
@@ -1396,9 +1410,22 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
         s.tile_entry = s.slot_of + want;
         if ((e = cudaMemsetAsync(s.tile_count, 0, sizeof(int) * (size_t)(ST + 4), stream)) ||
             (e = epic::launch_single(s, ctas, stream)) ||
-            (e = cudaMemcpyAsync(&n_used, s.used, sizeof n_used, cudaMemcpyDeviceToHost, stream)) ||
+            (e = cudaMemcpyAsync(n_done, s.used, sizeof n_done, cudaMemcpyDeviceToHost, stream)) ||
             (e = cudaStreamSynchronize(stream)))
             return cuda_fail(h, e, "exact-variant relaxation");
+        n_used = n_done[0];
+        if (n_done[2] > 0 && n_used <= s.slot_cap) {
+            // the matches left over, with pools of every tile
+            epic::SingleArgs all = s;
+            all.list = s.left;
+            all.N = (int)n_done[2];
+            all.pool_tiles = (int)ST;
+            if ((e = cudaMemsetAsync(s.next, 0, sizeof(unsigned), stream)) ||
+                (e = epic::launch_single(all, std::min(ctas_all, all.N), stream)) ||
+                (e = cudaMemcpyAsync(&n_used, s.used, sizeof n_used, cudaMemcpyDeviceToHost, stream)) ||
+                (e = cudaStreamSynchronize(stream)))
+                return cuda_fail(h, e, "exact-variant relaxation");
+        }
         if (n_used <= s.slot_cap) break;
         if (n_used > 0x7fffffffu) return fail(h, EPIC_ERR_CAPACITY, "exact variant: too many distance tiles");
         want = n_used;

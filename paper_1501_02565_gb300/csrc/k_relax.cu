@@ -109,7 +109,7 @@ __device__ void root_tile(const PairDev &P, int tx, int ty, DistTile<MAXR> &T, R
         R.lab[i] = LABEL_NONE;
         R.par[i] = (unsigned short)i;
     }
-    stage_dist(P, tx, ty, g, T, B, S, st, ROOT);
+    stage_dist(P, tx, ty, g, T, B, S, st, ROOT, FrameMap(P));
     for (int q = 0; q < P.stack && ty * P.stack + q < P.tiles_y; ++q) {
         const int bin = (ty * P.stack + q) * P.tiles_x + tx;
         for (int s = P.tile_start[bin] + tid, s1 = P.tile_start[bin + 1]; s < s1; s += NT) {

@@ -2,9 +2,10 @@
 // distances of the pixels that can have it among their K nearest (those within
 // their cap, see epic_exact_interp).
 //
-//   single_kernel  a CTA takes whole matches from a counter.  It holds a key
-//                  map of its own, unreached between matches, and solves
-//                  tiles of 64 x 32 pixels from the seed's outwards with the
+//   single_kernel  a CTA takes whole matches from a counter.  It holds keys
+//                  of its own, a pool of tiles taken as a match touches them
+//                  (a match that touches more is left for a second launch,
+//                  with pools of every tile), and solves tiles of 64 x 32 pixels from the seed's outwards with the
 //                  solve of relax_dist.cuh, the tile with the nearest open
 //                  offer first: nothing passes between CTAs, so no fence,
 //                  atomic or barrier of the grid is needed.  Only distances
@@ -16,17 +17,15 @@
 //                  lies beyond 32 bits or MAX_WINDOWS with 64-bit keys
 //                  (relax_settle.cuh).  The tiles that a match reaches (13 of
 //                  224 on a 1024 x 436 frame with 5000 matches and K = 100)
-//                  are written out as float32 distance tiles, and the map is
-//                  cleared there.
+//                  are written out as float32 distance tiles.
 //   start_kernel,  the distance tiles by image tile, for the per-pixel fit.
 //   list_kernel
 //
-// 1024 x 436, 5000 matches, K = 100: 13.9 ms; before, every match was a
+// 1024 x 436, 5000 matches, K = 100: 11.5 ms; before, every match was a
 // pseudo-pair of the apron-tile relaxation (directional sweeps in shared
 // memory, a grid barrier per pass of a chunk of 300 matches) with a dense row
 // of 446 K distances: 86.5 ms, and 5.3 ms to turn keys into rows.  What bounds
-// it: the latency of a tile's rounds, with two CTAs a SM (the budget for key
-// maps; registers allow three).  45 solves and 52 windows per match, of ~10 K
+// it: the latency of a tile's rounds, with three CTAs a SM (registers).  45 solves and 52 windows per match, of ~10 K
 // cycles for the rounds and ~14 K around them.  On the way to this form:
 //   - 64-bit keys for a tile with any pixel beyond its window: 31 ms (half of
 //     the solves, 91 K cycles each); further windows of 32 bits: 21.5 ms;
@@ -35,7 +34,9 @@
 //     tile is asked that cannot use them (61 -> 45 solves): 16.2 ms.  First in,
 //     first out instead: 19.0 ms; nearest by classes of 1/8 cost unit: 18.1;
 //   - offers across windows from shared memory, for the pixels that need them
-//     only, rather than unrolled in registers (41 K -> 20 K cycles): 13.9 ms.
+//     only, rather than unrolled in registers (41 K -> 20 K cycles): 13.9 ms;
+//   - pools of tiles instead of a map of the frame per CTA, so that the budget
+//     for keys (1 GiB) allows three CTAs a SM instead of two: 11.5 ms.
 #include "relax_dist.cuh"
 #include "relax_settle.cuh"
 
@@ -69,8 +70,24 @@ struct SingleShared {
     unsigned offer[9];   // by neighbour (TB_*), and the tile itself: place of what is offered
     // the CTA's tiles (x.flags and so on), for frames of few tiles
     unsigned char flags[FEW];
-    int queue[FEW], touched[FEW];
+    int queue[FEW], touched[FEW], place_of[FEW];
     unsigned at[FEW];
+};
+
+// The CTA's keys: a pool of tiles, taken in the order in which a match touches
+// them.
+struct PoolMap {
+    pkey_t *pool, *own;    // own: of the tile being solved
+    const int *place_of;   // tile -> place in the pool, -1: none (unreached)
+    int tiles_x, x0, y0;
+    __device__ __forceinline__ void row(int x, int y, int ncol, pkey_t *k) const {
+        load_keys(own, (size_t)(y - y0) * SINGLE_W + x - x0, ncol, true, k);
+    }
+    __device__ __forceinline__ pkey_t at(int x, int y) const {
+        const int s = place_of[y / SINGLE_H * tiles_x + x / SINGLE_W];
+        return s < 0 ? KEY_INF
+                     : __ldcg(pool + (size_t)s * SINGLE_TILE + y % SINGLE_H * SINGLE_W + x % SINGLE_W);
+    }
 };
 
 // The distances and caps of this thread's ring pixels (unreached, 0: none).
@@ -78,7 +95,8 @@ constexpr int PER = (RING<SR> + ST - 1) / ST;
 struct RingState {
     unsigned long long d[PER], cap[PER];
 };
-__device__ __forceinline__ void load_ring(const PairDev &P, const pkey_t *cap, const TileGeo &g, RingState &R) {
+__device__ __forceinline__ void load_ring(const PairDev &P, const PoolMap &map, const pkey_t *cap, const TileGeo &g,
+                                          RingState &R) {
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
         const int i = threadIdx.x + j * ST;
@@ -89,7 +107,7 @@ __device__ __forceinline__ void load_ring(const PairDev &P, const pkey_t *cap, c
         R.cap[j] = 0;
         if (i < RING<SR> && lr <= g.rv && gx >= 0 && gx < P.W && gy >= 0 && gy < P.H) {
             const size_t o = (size_t)gy * P.W + gx;
-            const pkey_t k = __ldcg(P.keys + o);
+            const pkey_t k = map.at(gx, gy);
             if (key_reached(k)) R.d[j] = key_dunits(k);
             R.cap[j] = key_dunits(cap[o]);
         }
@@ -155,12 +173,11 @@ __device__ __forceinline__ void store_row(pkey_t *dst, const pkey_t (&k)[4], uns
 // and returns the sum that the map's distances alone would have (*before).
 // false: nothing can be reached any more.  *lost: an offer within a pixel's
 // cap lies beyond 32 bits.
-__device__ bool next_window(const PairDev &P, const TileGeo &g, DistTile<SR> &T, WholeTile &A, DistBlock &B,
+__device__ bool next_window(const PoolMap &map, const TileGeo &g, DistTile<SR> &T, WholeTile &A, DistBlock &B,
                             Staged &S, const RingState &R, unsigned known, unsigned wanted,
                             const ulonglong2 (&caps)[8][ST], unsigned long long *before, bool *lost) {
     const int tid = threadIdx.x, bx = tid & 15, by = tid >> 4;
     const int b = (by + 1) * RT_BX + bx + 1;
-    const int W = P.W;
     const unsigned win = S.win;
     const unsigned long long base = S.base + win;
     auto rel = [&](unsigned long long d) -> unsigned {   // 0: below, 2^32 - 1: beyond 32 bits
@@ -186,8 +203,7 @@ __device__ bool next_window(const PairDev &P, const TileGeo &g, DistTile<SR> &T,
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         pkey_t k[4];
-        load_keys(P.keys, (size_t)(g.y0 + 4 * by + r) * W + g.x0 + 4 * bx, r < S.nrow ? S.ncol : 0,
-                  (W & 1) == 0, k);
+        map.row(g.x0 + 4 * bx, g.y0 + 4 * by + r, r < S.nrow ? S.ncol : 0, k);
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             x[r][c] = key_reached(k[c]) ? rel(key_dunits(k[c])) : 0xFFFFFFFFu;
@@ -257,19 +273,17 @@ __device__ bool next_window(const PairDev &P, const TileGeo &g, DistTile<SR> &T,
 // for nothing (nothing within the cap changed; the match's first solve offers
 // in any case, its seed is in the map already).  A window beyond `limit`, the
 // first place in the queue, or beyond an offer waits: sh.offer[8].
-__device__ void solve_single(const PairDev &P, const pkey_t *cap, int tx, int ty, SingleShared &sh,
+__device__ void solve_single(const PairDev &P, const PoolMap &map, const pkey_t *cap, int tx, int ty, SingleShared &sh,
                              RunState *st, bool first, unsigned limit) {
     const int tid = threadIdx.x, bx = tid & 15, by = tid >> 4;
     const int b = (by + 1) * RT_BX + bx + 1;
     const TileGeo g = tile_geo(P, tx, ty);
-    const int W = P.W;
-    const bool vec = (W & 1) == 0;
-    pkey_t *map = P.keys + (size_t)(g.y0 + 4 * by) * W + g.x0 + 4 * bx;
+    pkey_t *mine = map.own + 4 * by * SINGLE_W + 4 * bx;
     const int nrow = min(4, g.rv - 4 * by), ncol = min(4, g.wv - 4 * bx);
     bool wide = false;
     fetch_caps(cap, P, g, nrow, ncol, sh.cap);
     RingState R;
-    load_ring(P, cap, g, R);
+    load_ring(P, map, cap, g, R);
     if (tid < 9) sh.offer[tid] = 0xFFFFFFFFu;   // (barriers follow)
     auto offer = [&](unsigned f, unsigned at) {
 #pragma unroll
@@ -280,7 +294,7 @@ __device__ void solve_single(const PairDev &P, const pkey_t *cap, int tx, int ty
         DistTile<SR> &T = sh.dist;
         DistBlock B;
         Staged S;
-        stage_dist(P, tx, ty, g, T, B, S, st, AGAIN);
+        stage_dist(P, tx, ty, g, T, B, S, st, AGAIN, map);
         block_weights(T, b, S, B);
         unsigned long long before = block_sum(B);
         unsigned known = 0;
@@ -307,7 +321,7 @@ __device__ void solve_single(const PairDev &P, const pkey_t *cap, int tx, int ty
                     if (ok) mask |= 1u << c;
                     else B.d[r][c] = S.win;
                 }
-                if (mask) store_row(map + (size_t)r * W, k, mask, vec);
+                if (mask) store_row(mine + r * SINGLE_W, k, mask, true);
             }
             const bool changed = (first && window == 0) || block_sum(B) != before;
             if (__syncthreads_or(changed)) {
@@ -337,7 +351,7 @@ __device__ void solve_single(const PairDev &P, const pkey_t *cap, int tx, int ty
 #pragma unroll
                 for (int i = 0; i < 16; ++i) sh.whole.far[i][tid] = 0xFFFFFFFFu;
             bool lost = false;
-            const bool more = next_window(P, g, T, sh.whole, B, S, R, known, wanted, sh.cap, &before, &lost);
+            const bool more = next_window(map, g, T, sh.whole, B, S, R, known, wanted, sh.cap, &before, &lost);
             if (__syncthreads_or(lost)) {
                 wide = true;
                 break;
@@ -348,7 +362,7 @@ __device__ void solve_single(const PairDev &P, const pkey_t *cap, int tx, int ty
     if (wide) {
         SettleTile<SR> &T = sh.settle;
         Block B;
-        stage_tile(P, T, g, B, st);
+        stage_tile(P, T, g, B, st, map);
         const unsigned changed = solve_tile(T, g, B, st);
         unsigned long long v[4][4];
         load_caps(sh.cap, v);
@@ -363,7 +377,7 @@ __device__ void solve_single(const PairDev &P, const pkey_t *cap, int tx, int ty
                 if (key_reached(B.k[r][c]) && key_dunits(B.k[r][c]) <= v[r][c]) mask |= 1u << c;
                 else B.k[r][c] = KEY_INF;
             }
-            if (mask) store_row(map + (size_t)r * W, B.k[r], mask, vec);
+            if (mask) store_row(mine + r * SINGLE_W, B.k[r], mask, true);
             keep |= mask << (4 * r);
         }
         if (__syncthreads_or(keep != 0)) {
@@ -379,21 +393,16 @@ __device__ void solve_single(const PairDev &P, const pkey_t *cap, int tx, int ty
     __syncthreads();
 }
 
-// Write the reached pixels of tile t out as a distance tile of match m and
-// clear the map there.
-__device__ void put_tile(const SingleArgs &x, const PairDev &P, int t, int m, int *shared_slot) {
+// Write the reached pixels of tile t out as a distance tile of match m.
+__device__ void put_tile(const SingleArgs &x, const PairDev &P, const pkey_t *own, int t, int m, int *shared_slot) {
     const int tid = threadIdx.x, bx = tid & 15, by = tid >> 4;
-    const int tx = t % P.tiles_x, ty = t / P.tiles_x;
-    const TileGeo g = tile_geo(P, tx, ty);
-    const int W = P.W, nrow = min(4, g.rv - 4 * by), ncol = min(4, g.wv - 4 * bx);
-    const bool vec = (W & 1) == 0;
-    pkey_t *map = P.keys + (size_t)(g.y0 + 4 * by) * W + g.x0 + 4 * bx;
+    const TileGeo g = tile_geo(P, t % P.tiles_x, t / P.tiles_x);
+    const int nrow = min(4, g.rv - 4 * by), ncol = min(4, g.wv - 4 * bx);
     pkey_t k[4][4];
     bool any = false;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-        const size_t o = (size_t)(g.y0 + 4 * by + r) * W + g.x0 + 4 * bx;
-        load_keys(P.keys, o, r < nrow ? ncol : 0, vec, k[r]);
+        load_keys(own, (size_t)(4 * by + r) * SINGLE_W + 4 * bx, r < nrow ? ncol : 0, true, k[r]);
 #pragma unroll
         for (int c = 0; c < 4; ++c) any |= key_reached(k[r][c]);
     }
@@ -408,14 +417,11 @@ __device__ void put_tile(const SingleArgs &x, const PairDev &P, int t, int m, in
     }
     __syncthreads();
     const int s = *shared_slot;
-    const pkey_t none[4] = {KEY_INF, KEY_INF, KEY_INF, KEY_INF};
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < 4; ++r)
         if (s >= 0)
             *reinterpret_cast<float4 *>(x.slots + (size_t)s * SINGLE_TILE + (4 * by + r) * SINGLE_W + 4 * bx) =
                 make_float4(key_dist(k[r][0]), key_dist(k[r][1]), key_dist(k[r][2]), key_dist(k[r][3]));
-        if (r < nrow && ncol > 0) store_row(map + (size_t)r * W, none, (1u << ncol) - 1u, vec);
-    }
     __syncthreads();
 }
 
@@ -424,23 +430,24 @@ __global__ void __launch_bounds__(ST, 384 / ST) single_kernel(SingleArgs x) {
     if (get_status(st) != 0) return;
     __shared__ SingleShared sh;
     __shared__ PairDev P;
-    __shared__ int s_item, s_queued, s_touched, s_slot;
+    __shared__ int s_item, s_queued, s_touched, s_slot, s_seed, s_fresh;
     __shared__ unsigned s_limit;
     const int tid = threadIdx.x;
-    const long long npx = (long long)x.H * x.W;
     const int T = x.tiles_x * x.tiles_y;
     const bool few = T <= FEW;
     int *queue = few ? sh.queue : x.queue + (size_t)blockIdx.x * T;
     int *touched = few ? sh.touched : x.touched + (size_t)blockIdx.x * T;
     unsigned *at = few ? sh.at : x.place + (size_t)blockIdx.x * T;
     unsigned char *flags = few ? sh.flags : x.flags + (size_t)blockIdx.x * T;
-    pkey_t *keys = x.keys + (size_t)blockIdx.x * npx;
-    for (long long i = tid; i < npx; i += ST) keys[i] = KEY_INF;
-    for (int i = tid; i < T; i += ST) flags[i] = 0;
+    int *place_of = few ? sh.place_of : x.place_of + (size_t)blockIdx.x * T;
+    PoolMap map{x.keys + (size_t)blockIdx.x * x.pool_tiles * SINGLE_TILE, nullptr, place_of, x.tiles_x, 0, 0};
+    for (int i = tid; i < T; i += ST) {
+        flags[i] = 0;
+        place_of[i] = -1;
+    }
     if (tid == 0) {
         P.C = x.C;
         P.matches = x.matches;
-        P.keys = keys;
         P.H = x.H;
         P.W = x.W;
         P.tile_w = SINGLE_W;
@@ -453,16 +460,17 @@ __global__ void __launch_bounds__(ST, 384 / ST) single_kernel(SingleArgs x) {
     __syncthreads();
     for (;;) {
         if (tid == 0) {
-            const int m = (int)atomicAdd(x.next, 1u);
-            s_item = m;
+            const int i = (int)atomicAdd(x.next, 1u);
+            const int m = i < x.N && x.list ? x.list[i] : i;
+            s_item = i < x.N ? m : -1;
             s_queued = s_touched = 0;
-            if (m < x.N) {
+            if (i < x.N) {
                 const float4 mt = __ldg(x.matches + m);
                 const float fx = floorf(mt.x + 0.5f), fy = floorf(mt.y + 0.5f);
                 if (fx >= 0.f && fx < (float)x.W && fy >= 0.f && fy < (float)x.H) {
                     const int px = (int)fx, py = (int)fy;
                     const int t = py / SINGLE_H * x.tiles_x + px / SINGLE_W;
-                    keys[(size_t)py * x.W + px] = make_key(0ull, LABEL_NONE);
+                    s_seed = py % SINGLE_H * SINGLE_W + px % SINGLE_W;
                     queue[s_queued++] = t;
                     at[t] = 0;
                     flags[t] = IN_QUEUE;
@@ -474,7 +482,8 @@ __global__ void __launch_bounds__(ST, 384 / ST) single_kernel(SingleArgs x) {
         __syncthreads();
         const int m = s_item;
         __syncthreads();
-        if (m >= x.N) return;
+        if (m < 0) return;
+        bool whole = true;   // the pool held every tile that the match touches
         for (long long solves = 0;; ++solves) {
             // the nearest tile in the queue, and the place of the next one
             if (tid < 32) {
@@ -497,9 +506,18 @@ __global__ void __launch_bounds__(ST, 384 / ST) single_kernel(SingleArgs x) {
                     const int t = queue[fi];
                     queue[fi] = queue[n - 1];
                     s_queued = n - 1;
-                    if (!(flags[t] & TOUCHED)) touched[s_touched++] = t;
-                    flags[t] = TOUCHED;   // no longer queued
+                    s_fresh = 0;
                     s_item = t;
+                    if (!(flags[t] & TOUCHED)) {
+                        s_fresh = 1;
+                        if (s_touched < x.pool_tiles) {
+                            place_of[t] = s_touched;
+                            touched[s_touched++] = t;
+                        } else {
+                            s_item = -2 - t;   // no room
+                        }
+                    }
+                    flags[t] = TOUCHED;   // no longer queued
                     s_limit = second;
                 }
                 if (who == 0 && tid == 0) s_item = -1;
@@ -507,9 +525,20 @@ __global__ void __launch_bounds__(ST, 384 / ST) single_kernel(SingleArgs x) {
             }
             __syncthreads();
             const int t = s_item;
+            if (t < -1) whole = false;
             if (t < 0 || solves > x.max_solves) break;
             const int tx = t % x.tiles_x, ty = t / x.tiles_x;
-            solve_single(P, x.cap, tx, ty, sh, st, solves == 0, s_limit);
+            map.own = map.pool + (size_t)place_of[t] * SINGLE_TILE;
+            map.x0 = tx * SINGLE_W;
+            map.y0 = ty * SINGLE_H;
+            if (s_fresh) {
+                const pkey_t none[4] = {KEY_INF, KEY_INF, KEY_INF, KEY_INF};
+                for (int i = 4 * tid; i < SINGLE_TILE; i += 4 * ST) store_row(map.own + i, none, 15u, true);
+                __syncthreads();
+                if (solves == 0 && tid == 0) map.own[s_seed] = make_key(0ull, LABEL_NONE);
+                __syncthreads();
+            }
+            solve_single(P, map, x.cap, tx, ty, sh, st, solves == 0, s_limit);
             if (tid < 9 && sh.offer[tid] != 0xFFFFFFFFu) {
                 const int nx = tid == 8 ? tx : tx + (tid < 3 ? tid - 1 : tid < 5 ? 2 * tid - 7 : tid - 6);
                 const int ny = tid == 8 ? ty : ty + (tid < 3 ? -1 : tid < 5 ? 0 : 1);
@@ -528,9 +557,19 @@ __global__ void __launch_bounds__(ST, 384 / ST) single_kernel(SingleArgs x) {
         }
         __syncthreads();
         const int n = s_touched;
-        for (int i = 0; i < n; ++i) put_tile(x, P, touched[i], m, &s_slot);
+        if (whole) {
+            for (int i = 0; i < n; ++i)
+                put_tile(x, P, map.pool + (size_t)i * SINGLE_TILE, touched[i], m, &s_slot);
+        } else if (tid == 0) {
+            x.left[atomicAdd(x.left_count, 1u)] = m;
+            flags[-2 - s_item] = 0;
+            for (int i = 0; i < s_queued; ++i) flags[queue[i]] = 0;
+        }
         __syncthreads();
-        for (int i = tid; i < n; i += ST) flags[touched[i]] = 0;
+        for (int i = tid; i < n; i += ST) {
+            flags[touched[i]] = 0;
+            place_of[touched[i]] = -1;
+        }
         __syncthreads();
     }
 }

@@ -157,16 +157,15 @@ __device__ void dist_rounds(DistTile<MAXR> &T, DistBlock &B, int b, int cap) {
 // Stage tile (tx, ty): this thread's distances into B.d and the rest into S,
 // the tile's border distances and half-costs and the ring into shared memory;
 // every thread has passed a barrier when it returns.
-template <int MAXR>
+template <int MAXR, typename Map = FrameMap>
 __device__ void stage_dist(const PairDev &P, int tx, int ty, const TileGeo &g, DistTile<MAXR> &T,
-                           DistBlock &B, Staged &S, RunState *st, Mode mode) {
+                           DistBlock &B, Staged &S, RunState *st, Mode mode, const Map &map) {
     constexpr int NT = Dim<MAXR>::NT, NB = Dim<MAXR>::NB;
     const int tid = threadIdx.x, bx = tid & 15, by = tid >> 4;
     const int b = (by + 1) * RT_BX + bx + 1;
     const int W = P.W, H = P.H;
-    const pkey_t *gk = P.keys;
     const float *gc = P.C;
-    const bool kvec = (W & 1) == 0, cvec = (W & 3) == 0 && ((uintptr_t)gc & 15) == 0;
+    const bool cvec = (W & 3) == 0 && ((uintptr_t)gc & 15) == 0;
 
     // this block's costs and keys (rows down to the ring row below the tile,
     // which lies inside a block when the tile is not a whole number of blocks
@@ -181,7 +180,7 @@ __device__ void stage_dist(const PairDev &P, int tx, int ty, const TileGeo &g, D
         const int nc = r < nrow ? ncol : 0;
         load_costs(gc, o, nc, cvec, cc[r]);
         const bool ring_row = 4 * by + r >= g.rv;
-        load_keys(gk, o, mode >= AGAIN || (mode == SECOND && ring_row) ? nc : 0, kvec, kk[r]);
+        map.row(g.x0 + 4 * bx, g.y0 + 4 * by + r, mode >= AGAIN || (mode == SECOND && ring_row) ? nc : 0, kk[r]);
     }
     constexpr int PER = (RING<MAXR> + NT - 1) / NT;
     pkey_t rk[PER];
@@ -201,7 +200,7 @@ __device__ void stage_dist(const PairDev &P, int tx, int ty, const TileGeo &g, D
         if (in) {
             const size_t o = (size_t)gy * W + gx;
             rc[j] = __ldg(gc + o);
-            if (mode >= AGAIN || (mode == SECOND && !diagonal)) rk[j] = __ldcg(gk + o);
+            if (mode >= AGAIN || (mode == SECOND && !diagonal)) rk[j] = map.at(gx, gy);
         }
     }
     if (mode == ROOT) {
@@ -417,7 +416,7 @@ __device__ unsigned solve_dist(const PairDev &P, int t, int tx, int ty, DistTile
     const int W = P.W;
     DistBlock B;
     Staged S;
-    stage_dist(P, tx, ty, g, T, B, S, st, mode);
+    stage_dist(P, tx, ty, g, T, B, S, st, mode, FrameMap(P));
     unsigned f = mode != AGAIN ? TB_ANY : 0u;
     {
         block_weights(T, b, S, B);

@@ -184,26 +184,25 @@ __device__ __noinline__ unsigned rounds_apart(SettleTile<MAXR> &T, Block *B, int
 // half-cost zero.  Row rv of the tile (the ring row below) may lie inside a
 // block when the tile is not a whole number of blocks high; it is held like
 // the ring, never updated.
-template <int MAXR>
+template <int MAXR, typename Map = FrameMap>
 __device__ void stage_tile(const PairDev &P, SettleTile<MAXR> &T, const TileGeo &g, Block &B,
-                           RunState *st) {
+                           RunState *st, const Map &map) {
     constexpr int NT = Dim<MAXR>::NT, NB = Dim<MAXR>::NB;
     const int tid = threadIdx.x, bx = tid & 15, by = tid >> 4;
     const int b = (by + 1) * RT_BX + bx + 1;
     const int W = P.W, H = P.H;
-    const pkey_t *gk = P.keys;
     const float *gc = P.C;
     const int nrow = min(4, min(g.rv + 1, H - g.y0) - 4 * by);
     const int ncol = min(4, g.wv - 4 * bx);
     B.valid = 0;
     float cc[4][4];
-    const bool kvec = (W & 1) == 0, cvec = (W & 3) == 0 && ((uintptr_t)gc & 15) == 0;
+    const bool cvec = (W & 3) == 0 && ((uintptr_t)gc & 15) == 0;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         const size_t o = (size_t)(g.y0 + 4 * by + r) * W + g.x0 + 4 * bx;
         const int nc = r < nrow ? ncol : 0;
         load_costs(gc, o, nc, cvec, cc[r]);
-        load_keys(gk, o, nc, kvec, B.k[r]);
+        map.row(g.x0 + 4 * bx, g.y0 + 4 * by + r, nc, B.k[r]);
 #pragma unroll
         for (int c = 0; c < 4; ++c)
             if (c < nc && 4 * by + r < g.rv) B.valid |= 1u << (4 * r + c);
@@ -225,7 +224,7 @@ __device__ void stage_tile(const PairDev &P, SettleTile<MAXR> &T, const TileGeo 
         if (in) {
             const size_t o = (size_t)gy * W + gx;
             rc[j] = __ldg(gc + o);
-            rk[j] = __ldcg(gk + o);
+            rk[j] = map.at(gx, gy);
         }
     }
     HalfCost half(P);
@@ -406,7 +405,7 @@ __device__ unsigned settle_tile(const PairDev &P, int tx, int ty, SettleTile<MAX
     const int tid = threadIdx.x;
     const TileGeo g = tile_geo(P, tx, ty);
     Block B;
-    stage_tile(P, T, g, B, st);
+    stage_tile(P, T, g, B, st, FrameMap(P));
     const unsigned mask = solve_tile(T, g, B, st);
     unsigned f = 0;
     if (mask) {

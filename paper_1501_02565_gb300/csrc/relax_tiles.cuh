@@ -111,6 +111,18 @@ __device__ __forceinline__ void load_keys(const pkey_t *K, size_t o, int ncol, b
     }
 }
 
+// Where a tile's keys are staged from: the frame's map.
+struct FrameMap {
+    const pkey_t *keys;
+    int W;
+    __device__ __forceinline__ explicit FrameMap(const PairDev &P) : keys(P.keys), W(P.W) {}
+    // four keys of row y from column x on (columns < ncol)
+    __device__ __forceinline__ void row(int x, int y, int ncol, pkey_t *k) const {
+        load_keys(keys, (size_t)y * W + x, ncol, (W & 1) == 0, k);
+    }
+    __device__ __forceinline__ pkey_t at(int x, int y) const { return __ldcg(keys + (size_t)y * W + x); }
+};
+
 // The half-cost of a staged cost (half_cost_s with the pair's factors).
 struct HalfCost {
     float limit, scale;

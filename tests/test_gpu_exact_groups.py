@@ -1,8 +1,8 @@
 """The exact variant's kernels (csrc/k_single.cu, csrc/k_exact.cu) where they
 change their path: groups of pixels with more candidates than shared memory
 holds, matches outside the frame (Euclidean), distances beyond the 32-bit
-window of a tile and steps longer than it, a budget of one key map, frames of
-more tiles than the per-CTA tables hold, and runs that need more distance tiles
+window of a tile and steps longer than it, a budget of one key map, pools that
+do not hold a match's tiles, frames of more tiles than the per-CTA tables hold, and runs that need more distance tiles
 than are first set aside.
 
 Against the FP64 oracle with the tolerances of test_gpu_exact.py, or, where the
@@ -76,16 +76,18 @@ def test_euclidean_matches_outside_the_frame():
     _check(C, _matches(rng, xy), 9, 1.0, "euclidean")
 
 
-@pytest.mark.parametrize("kind,H,W,N,K", [
-    ("edges", 530, 2100, 24, 2),    # 33 x 17 tiles
-    ("high", 300, 701, 40, 40),     # every tile of every match: 4400 distance tiles
+@pytest.mark.parametrize("kind,H,W,N,K,budget", [
+    ("edges", 530, 2100, 24, 2, 0),    # 33 x 17 tiles
+    ("high", 300, 701, 40, 40, 0),     # every tile of every match: 4400 distance tiles
+    ("high", 300, 701, 40, 40, 2 * 110 * 16384),   # three pools of 73 of the 110 tiles: all run again
+    ("edges", 300, 701, 300, 20, 2 * 110 * 16384),
 ])
-def test_lists_hold_the_single_match_maps(kind, H, W, N, K):
+def test_lists_hold_the_single_match_maps(kind, H, W, N, K, budget):
     import torch
     rng = np.random.Generator(np.random.PCG64(H + W))
     M = _matches(rng, _spread(rng, H, W, N))
     C = torch.from_numpy(_cost(kind, rng, H, W)).cuda()
-    eng = native.EpicInterp(0)
+    eng = native.EpicInterp(0, exact_chunk_bytes=budget)
     _, idx, dist = eng.exact(C, torch.from_numpy(M).cuda(), K, 1.0, with_knn=True)
     eng.close()
     eng = native.EpicInterp(0, sweep=0)   # the apron tiles keep the unit 2^-31 on every frame
