@@ -196,6 +196,14 @@ int solve_stack(long long tiles, int max_th) {
     return tiles >= epic::RELAX_STACK_TILES && 2 * max_th <= epic::RELAX_MAX_ROWS ? 2 : 1;
 }
 
+// Waits, on every way out of a call, for the copies from the call's own memory
+// (CUDA reads pageable memory when it copies, which may be after the call that
+// orders the copy).  Declared after that memory.
+struct CopiesEnd {
+    cudaStream_t stream;
+    ~CopiesEnd() { cudaStreamSynchronize(stream); }
+};
+
 struct Layout {
     size_t keys, tile_start, tile_fill, tile_seeds, tile_stamp, hkeys, hw, deg, wmin, wmin2, wnear,
         row, adj, models,
@@ -1308,6 +1316,8 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
     float *aflow = reinterpret_cast<float *>(b + o_aflow);
     char *tdev = b + o_table;
     epic::LaunchCfg lc{h->num_sms, h->smem_optin, stream, h->smem_per_sm, h->smem_reserved};
+    std::vector<char> thost(t_bytes, 0);   // the cap map's table
+    CopiesEnd copies_end{stream};
     {
         h->force_keep = true;
         epic_pair_desc_t ad{cost_map, matches, H, W, N, K, a, aflow};
@@ -1358,7 +1368,6 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
         vb.weight_squared = 1;
         vb.fallback_eps = c.fallback_eps;
         vb.state = h->state;
-        std::vector<char> thost(t_bytes, 0);
         memcpy(thost.data(), &vb, sizeof vb);
         memcpy(thost.data() + args_bytes, &v, sizeof(PairDev));
         const int ends[2] = {T, N};   // the prefixes are {0, tiles}, {0, matches}, then zeros
@@ -1369,7 +1378,6 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
             (e = epic::launch_prepare(vb, dev_v, lc)) ||
             (e = epic::launch_dt(vb, dev_v, lc, tw, th, ap, false, nullptr)))
             return cuda_fail(h, e, "exact-variant cap map");
-        // (a copy from pageable memory has read its source when it returns)
     }
     epic::SingleArgs s{};
     s.C = cost_map;

@@ -146,18 +146,20 @@ extern "C" int epic_geodesic_labels_noalloc(const float *cost_map, const float *
     a.weight_squared = 1;
     a.fallback_eps = 1e-10f;
     a.state = &dev_call->state;
-    // (a copy from pageable host memory has consumed its source by the time
-    // cudaMemcpyAsync returns)
-    if (cudaMemcpyAsync(dev_call, &call, sizeof(call), cudaMemcpyHostToDevice, stream))
+    // `call` is read when the copy is done, which may be later than it is
+    // ordered: an error below waits for the stream before `call` goes
+    auto failed = [&]() -> int {
+        cudaStreamSynchronize(stream);
         return EPIC_ERR_CUDA;
+    };
+    if (cudaMemcpyAsync(dev_call, &call, sizeof(call), cudaMemcpyHostToDevice, stream)) return failed();
     epic::LaunchCfg lc{num_sms, smem_optin, stream};
     if (epic::launch_prepare(a, &dev_call->args, lc) != cudaSuccess ||
         epic::launch_relax(a, &dev_call->args, lc, NA_TILE_H, false, nullptr) != cudaSuccess ||
         epic::launch_split_keys(&Pd, &dev_call->pair, labels_out, dist_out, stream) != cudaSuccess)
-        return EPIC_ERR_CUDA;
+        return failed();
     int status = 0;
-    if (cudaMemcpyAsync(&status, &dev_call->state.status, sizeof(int), cudaMemcpyDeviceToHost, stream) ||
-        cudaStreamSynchronize(stream))
-        return EPIC_ERR_CUDA;
+    if (cudaMemcpyAsync(&status, &dev_call->state.status, sizeof(int), cudaMemcpyDeviceToHost, stream)) return failed();
+    if (cudaStreamSynchronize(stream)) return EPIC_ERR_CUDA;
     return status;
 }
