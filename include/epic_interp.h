@@ -93,7 +93,11 @@ typedef struct {
     int max_N, max_K;     /* largest match count / neighbourhood size
                              (max_K at most EPIC_MAX_K) */
     int max_pairs;        /* largest batch the arena is first sized for */
-    int max_passes;       /* cap on relaxation verification passes */
+    int max_passes;       /* cap on the relaxation's work, over which a run
+                             ends with EPIC_ERR_NOT_CONVERGED: verification
+                             passes with sweep 0 or 1; with sweep 2, tile
+                             solves of the whole run in either of its phases,
+                             two per tile and pass */
     int weight_squared;   /* 1: Eq. 2 rows scaled by k, i.e. minimise
                              sum k^2 |r|^2 (default); 0: minimise sum k |r|^2 */
     float fallback_eps;   /* fit is degenerate when det M <= eps (tr M/3)^3

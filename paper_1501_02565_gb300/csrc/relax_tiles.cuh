@@ -237,7 +237,9 @@ __device__ bool own_tiles(const BatchArgs &a, RunState *st, TileWork *q, unsigne
                           OwnShared &S, unsigned nblocks, Solve solve) {
     const unsigned Tt = (unsigned)a.total_solve;
     const unsigned mine = (Tt - blockIdx.x + nblocks - 1) / nblocks;   // tiles owned
-    const unsigned long long cap = (unsigned long long)a.max_passes * mine;
+    // solves of the whole run: a pass is two for each of its tiles (a stack
+    // counts once), whichever tiles and CTAs they fall to
+    const unsigned long long cap = 2ull * (unsigned long long)a.max_passes * (unsigned)a.total_tiles;
     unsigned long long solved = 0;
     const int tid = threadIdx.x;
     unsigned long long t0 = wait_ns();   // thread 0: when something was last seen to move
@@ -260,7 +262,10 @@ __device__ bool own_tiles(const BatchArgs &a, RunState *st, TileWork *q, unsigne
                         S.state = -2;
                     else {
                         const unsigned now = *(volatile unsigned *)&q->solves;
-                        if (now != seen) {
+                        if (now > cap) {
+                            set_status(st, EPIC_ERR_NOT_CONVERGED);
+                            S.state = -2;
+                        } else if (now != seen) {
                             seen = now;
                             t0 = wait_ns();
                         } else if (wait_ns() - t0 > IDLE_LIMIT_NS) {
@@ -310,7 +315,7 @@ __device__ bool own_tiles(const BatchArgs &a, RunState *st, TileWork *q, unsigne
                 atomicSub(&q->open, (int)n);
                 atomicAdd(&q->solves, 1u);
             }
-            if (++solved > cap) {
+            if (++solved > cap) {   // (a CTA that never looks at the run's)
                 if (tid == 0) set_status(st, EPIC_ERR_NOT_CONVERGED);
                 return false;
             }
