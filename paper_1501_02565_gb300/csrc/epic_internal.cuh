@@ -177,9 +177,11 @@ struct PairDev {
     CUtensorMap tm_cost_again;
     // written on the device by the prepare kernel (zero from the host): the
     // float bits of the pair's largest cost and the tile-step reach of its
-    // seeds, from which unit_shift() derives the distance unit
+    // seeds, from which unit_shift() derives the distance unit; the sum of its
+    // costs, for settles_only()
     unsigned cmax_bits;
     int seed_reach;
+    float cost_sum;
 };
 
 // The distance unit shift of a pair (0 for the sweep schedules of k_dt.cu and
@@ -188,6 +190,19 @@ __device__ __forceinline__ int unit_shift(const PairDev &P) {
     return P.sweep == SWEEP_WARP
                ? unit_shift_of(P.cmax_bits, P.seed_reach, P.tile_w, P.tile_h)
                : 0;
+}
+
+// Whether a pair's relaxation is all settling (see k_relax.cu): its costs are so
+// high that the 32-bit window of a tile, one cost unit at the unit 2^-31, holds
+// few of its steps.  The line, from builds that take either way for all pairs
+// (relaxation of eight 1024 x 436 pairs, all phases and settling alone, us):
+// costs U(0.05, 0.3) 443 and 469, U(0.1, 0.4) 485 and 423, U(0.3, 0.99) 487 and
+// 410, all 1.0 399 and 313; one such pair: 158 and 183, 168 and 167, 186 and 171,
+// 143 and 124.  (The sum is of floats in any order: at the line the choice may
+// vary, the result does not.)
+__device__ __forceinline__ bool settles_only(const PairDev &P) {
+    const float line = 0.25f * (float)P.H * (float)P.W;   // at the unit 2^-31; no unit is finer
+    return P.cost_sum > line && P.cost_sum > ldexpf(line, unit_shift(P));
 }
 
 // A CSR row in a word: its first entry and its degree, ROW_LONG if they do not

@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(1024) compact_kernel(BatchArgs *ap, unsigned *
             P.matches = P.pruned;
             P.N = nk;
             P.K = min(P.K2, nk);
+            P.cost_sum = 0.f;   // (the second pass sums again)
         }
         __syncthreads();
     }

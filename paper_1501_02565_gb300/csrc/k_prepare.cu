@@ -11,7 +11,8 @@
 // * For the warp-tile relaxation, each pair's largest cost and the reach of
 //   its seeds over the tile grid (a Chebyshev distance transform of the
 //   seeded tiles) are recorded; they fix the pair's distance unit (see
-//   unit_shift in epic_internal.cuh).
+//   unit_shift in epic_internal.cuh).  So is the sum of its costs (see
+//   settles_only there).
 #include "epic_internal.cuh"
 
 namespace epic {
@@ -139,13 +140,15 @@ __device__ void seed_reach(const PairDev &P, int T, int *d) {
     __syncthreads();
 }
 
-// Largest cost of every warp-tile pair (float bits; costs are >= 0, so the
-// bits order like the values, and a NaN or negative cost shows as a value
-// above +inf).  Work items are the write-out chunks (1024 pixels); each CTA
+// Largest cost (float bits; costs are >= 0, so the bits order like the values,
+// and a NaN or negative cost shows as a value above +inf) and the sum of the
+// costs of every warp-tile pair.  Work items are the write-out chunks (1024 pixels); each CTA
 // takes a contiguous run, its four groups of 256 threads an item at a time
-// (four pixels a thread), and a warp's running maximum goes out with one
-// atomic whenever its pair changes.
-__device__ void cost_max(const BatchArgs &a) {
+// (four pixels a thread).  A warp's running maximum and sum go out whenever its
+// pair changes: those of the CTA's first pair together at the end, others with
+// an atomic each (the warps of a single frame are 9.7 K: 2048 x 1024 took 58 us
+// with an atomic per warp for either, 49 for the maximum alone, 46 so).
+__device__ void cost_stats(const BatchArgs &a) {
     // the CTAs that binned a pair's seeds take no part when enough others
     // are left (they would finish last)
     const int first = a.npairs < (int)gridDim.x / 2 ? a.npairs : 0;
@@ -154,13 +157,36 @@ __device__ void cost_max(const BatchArgs &a) {
     const int per = (a.total_chunks + nb - 1) / nb;
     const int c0 = b * per, c1 = min(a.total_chunks, c0 + per);
     const int grp = threadIdx.x >> 8, gt = threadIdx.x & 255;   // warp-uniform group
+    if (c0 >= c1) return;
+    __shared__ unsigned s_max[32];
+    __shared__ float s_sum[32];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int first_pair = find_pair(a.chunk_base, a.npairs, c0);
+    if (lane == 0) {
+        s_max[wid] = 0;
+        s_sum[wid] = 0.f;
+    }
+    auto put = [&](int p, unsigned m, float v) {
+        atomicMax(const_cast<unsigned *>(&a.pairs[p].cmax_bits), m);
+        atomicAdd(const_cast<float *>(&a.pairs[p].cost_sum), v);
+    };
     int pi = -1;
     unsigned mx = 0;
+    float sum = 0.f;
     auto flush = [&]() {
         const unsigned wm = __reduce_max_sync(0xffffffffu, mx);
-        if (pi >= 0 && (threadIdx.x & 31) == 0)
-            atomicMax(const_cast<unsigned *>(&a.pairs[pi].cmax_bits), wm);
+#pragma unroll
+        for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (pi >= 0 && lane == 0) {
+            if (pi == first_pair) {
+                s_max[wid] = wm;
+                s_sum[wid] = sum;
+            } else {
+                put(pi, wm, sum);
+            }
+        }
         mx = 0;
+        sum = 0.f;
     };
     for (int c = c0 + grp; c < c1; c += 4) {
         const int p = find_pair(a.chunk_base, a.npairs, c);
@@ -176,12 +202,24 @@ __device__ void cost_max(const BatchArgs &a) {
             const float4 v = __ldg(reinterpret_cast<const float4 *>(P.C + i));
             mx = max(max(mx, __float_as_uint(v.x)), max(__float_as_uint(v.y), max(
                          __float_as_uint(v.z), __float_as_uint(v.w))));
+            sum += v.x + v.y + (v.z + v.w);
         } else {
-            for (int j = 0; j < 4 && i + j < npx; ++j)
-                mx = max(mx, __float_as_uint(__ldg(P.C + i + j)));
+            for (int j = 0; j < 4 && i + j < npx; ++j) {
+                const float v = __ldg(P.C + i + j);
+                mx = max(mx, __float_as_uint(v));
+                sum += v;
+            }
         }
     }
     flush();
+    __syncthreads();
+    if (wid == 0) {
+        const unsigned wm = __reduce_max_sync(0xffffffffu, s_max[lane]);
+        sum = s_sum[lane];
+#pragma unroll
+        for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0) put(first_pair, wm, sum);
+    }
 }
 
 __global__ void __launch_bounds__(1024, 2) prepare_kernel(const BatchArgs *__restrict__ ap) {
@@ -259,7 +297,7 @@ __global__ void __launch_bounds__(1024, 2) prepare_kernel(const BatchArgs *__res
             P.hw[i] = 0xFFFFFFFFu;
         }
     }
-    cost_max(a);
+    cost_stats(a);
 }
 
 }  // namespace

@@ -36,6 +36,10 @@
 //           win), pixels outside a tile's distance window, and plateaus of
 //           cost zero (a pixel whose parent is not strictly nearer is given
 //           up by the look for roots).
+// Pairs of costs so high that a tile's window holds few steps (settles_only in
+// epic_internal.cuh) are settled from their seeds: the other phases would be
+// passed through for nothing (eight pairs of constant cost 1.0: relaxation 405
+// -> 328 us, the call 880 -> 802).
 // Carrying labels through every round of the first two phases instead makes
 // each of their steps five times as expensive (see relax_dist.cuh): that form
 // took 5.8 ms for the 64-pair mixed batch, this one 4.07 ms.  The form before,
@@ -94,6 +98,47 @@ union RelaxShared {
 };
 static_assert(sizeof(RelaxShared<32>) <= 48 * 1024, "a tile fits in static shared memory");
 
+// The labels of tile (tx, ty)'s seeds, the smallest of those on a pixel.
+template <int MAXR>
+__device__ __forceinline__ void seed_labels(const PairDev &P, int tx, int ty, const TileGeo &g, RootCells<MAXR> &R) {
+    constexpr int NT = Dim<MAXR>::NT;
+    for (int q = 0; q < P.stack && ty * P.stack + q < P.tiles_y; ++q) {
+        const int bin = (ty * P.stack + q) * P.tiles_x + tx;
+        for (int s = P.tile_start[bin] + threadIdx.x, s1 = P.tile_start[bin + 1]; s < s1; s += NT) {
+            const int m = P.tile_seeds[s];
+            const float4 mt = __ldg(P.matches + m);
+            const int px = (int)floorf(mt.x + 0.5f) - g.x0;
+            const int py = (int)floorf(mt.y + 0.5f) - g.y0;
+            if (px >= 0 && px < g.wv && py >= 0 && py < g.rv)
+                atomicMin(&R.lab[(py + 1) * ROOT_PITCH + px + 1], (unsigned)m);
+        }
+    }
+}
+
+// The keys that the settling of tile (tx, ty), local index t, starts from when
+// it is all of the relaxation: its seeds', and unreached elsewhere.
+template <int MAXR>
+__device__ void seed_tile(const PairDev &P, int t, int tx, int ty, RootCells<MAXR> &R, RunState *st) {
+    constexpr int NT = Dim<MAXR>::NT;
+    const TileGeo g = tile_geo(P, tx, ty);
+    for (int i = threadIdx.x; i < RootCells<MAXR>::N; i += NT) R.lab[i] = LABEL_NONE;
+    __syncthreads();
+    seed_labels(P, tx, ty, g, R);
+    __syncthreads();
+    for (int i = threadIdx.x; i < RT_COLS * g.rv; i += NT) {
+        const int r = i / RT_COLS, c = i % RT_COLS;
+        const unsigned m = R.lab[(r + 1) * ROOT_PITCH + c + 1];
+        if (c < g.wv) P.keys[(size_t)(g.y0 + r) * P.W + g.x0 + c] = m == LABEL_NONE ? KEY_INF : make_key(0ull, m);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        *(volatile int *)(P.tile_stamp + t) = 0;
+        __threadfence();
+        atomicAdd(&st->fresh_done, 1u);
+    }
+}
+
 // The roots of tile (tx, ty)'s pixels.
 template <int MAXR>
 __device__ void root_tile(const PairDev &P, int tx, int ty, DistTile<MAXR> &T, RootCells<MAXR> &R,
@@ -110,17 +155,7 @@ __device__ void root_tile(const PairDev &P, int tx, int ty, DistTile<MAXR> &T, R
         R.par[i] = (unsigned short)i;
     }
     stage_dist(P, tx, ty, g, T, B, S, st, ROOT, FrameMap(P));
-    for (int q = 0; q < P.stack && ty * P.stack + q < P.tiles_y; ++q) {
-        const int bin = (ty * P.stack + q) * P.tiles_x + tx;
-        for (int s = P.tile_start[bin] + tid, s1 = P.tile_start[bin + 1]; s < s1; s += NT) {
-            const int m = P.tile_seeds[s];
-            const float4 mt = __ldg(P.matches + m);
-            const int px = (int)floorf(mt.x + 0.5f) - g.x0;
-            const int py = (int)floorf(mt.y + 0.5f) - g.y0;
-            if (px >= 0 && px < g.wv && py >= 0 && py < g.rv)
-                atomicMin(&R.lab[(py + 1) * ROOT_PITCH + px + 1], (unsigned)m);
-        }
-    }
+    seed_labels(P, tx, ty, g, R);
     block_weights(T, b, S, B);
     __syncthreads();
     const int i0 = (4 * by + 1) * ROOT_PITCH + 4 * bx + 1;   // this block's first cell
@@ -325,8 +360,12 @@ __global__ void __launch_bounds__(Dim<MAXR>::NT, 384 / Dim<MAXR>::NT)
         const PairDev &P = a.pairs[pi];
         const int lt = t - a.solve_base[pi];
         const int tx = lt % P.tiles_x, ty = lt / P.tiles_x;
-        if (half && !wait_edge_neighbours(P, tx, ty, st)) return;
-        solve_dist(P, lt, tx, ty, T, st, half ? SECOND : FIRST);
+        if (settles_only(P)) {
+            seed_tile(P, lt, tx, ty, shared.root, st);
+        } else {
+            if (half && !wait_edge_neighbours(P, tx, ty, st)) return;
+            solve_dist(P, lt, tx, ty, T, st, half ? SECOND : FIRST);
+        }
         __syncthreads();
     }
     // spread: a tile or its ring may still be being written for the first time
@@ -334,6 +373,7 @@ __global__ void __launch_bounds__(Dim<MAXR>::NT, 384 / Dim<MAXR>::NT)
     bool written = false;
     if (!own_tiles(a, st, &st->tiles[0], a.relax_req, T.own, nblocks,
               [&](const PairDev &P, int lt, int tx, int ty) -> unsigned {
+                  if (settles_only(P)) return 0u;
                   if (!written) {
                       if (!wait_tile_and_ring(P, tx, ty, st)) return 0u;
                       written = __syncthreads_or(threadIdx.x == 0 && ld_acquire(&st->fresh_done) ==
@@ -344,12 +384,12 @@ __global__ void __launch_bounds__(Dim<MAXR>::NT, 384 / Dim<MAXR>::NT)
         return;
     __syncthreads();
     each_tile(a, nblocks, [&](const PairDev &P, int tx, int ty) {
-        root_tile(P, tx, ty, T, shared.root, st);
+        if (!settles_only(P)) root_tile(P, tx, ty, T, shared.root, st);
     });
     __threadfence();
     if (!grid_sync(st, nblocks)) return;
     each_tile(a, nblocks, [&](const PairDev &P, int tx, int ty) {
-        chase_tile(P, tx, ty, shared.chase);
+        if (!settles_only(P)) chase_tile(P, tx, ty, shared.chase);
     });
     __threadfence();
     if (!grid_sync(st, nblocks)) return;
