@@ -240,7 +240,8 @@ __device__ bool next_window(const PoolMap &map, const TileGeo &g, DistTile<SR> &
 #pragma unroll
     for (int i = 0; i < ST / 32; ++i) m = min(m, T.red[0][i]);
     S.base = base + m;
-    auto in = [&](unsigned d) { return d <= m ? 0u : min(d - m, win); };
+    // (2^32 - 1, unreached or beyond 32 bits, is no distance)
+    auto in = [&](unsigned d) { return d <= m ? 0u : d == 0xFFFFFFFFu ? win : min(d - m, win); };
     unsigned long long sum = 0;
 #pragma unroll
     for (int r = 0; r < 4; ++r)
