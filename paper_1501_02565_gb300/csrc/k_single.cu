@@ -171,8 +171,8 @@ __device__ __forceinline__ void store_row(pkey_t *dst, const pkey_t (&k)[4], uns
 // one (relative to S.base, exact: a step may be longer than a window).  Sets
 // S.base, the block's distances (from the offers and the map) and the planes,
 // and returns the sum that the map's distances alone would have (*before).
-// false: nothing can be reached any more.  *lost: an offer within a pixel's
-// cap lies beyond 32 bits.
+// false: nothing can be reached any more.  *lost: what matters lies beyond 32
+// bits.
 __device__ bool next_window(const PoolMap &map, const TileGeo &g, DistTile<SR> &T, WholeTile &A, DistBlock &B,
                             Staged &S, const RingState &R, unsigned known, unsigned wanted,
                             const ulonglong2 (&caps)[8][ST], unsigned long long *before, bool *lost) {
@@ -184,19 +184,21 @@ __device__ bool next_window(const PoolMap &map, const TileGeo &g, DistTile<SR> &
         return d < base ? 0u : (unsigned)min(d - base, 0xFFFFFFFFull);
     };
     unsigned m = 0xFFFFFFFFu;   // the first distance of the window
+    // whether a distance of the ring, of the map lies beyond 32 bits
+    bool ring_beyond = false, map_beyond = false;
     int re[PER];
-    unsigned rd[PER];
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
         const int i = tid + j * ST;
         int lr, lc;
         ring_pixel<SR>(i, &lr, &lc);
         re[j] = i < RING<SR> ? plane_of(lr & 3, lc & 3) * Dim<SR>::NB + ring_entry(lr, lc) : -1;
-        rd[j] = rel(R.d[j]);
         if (re[j] >= 0) {
             A.d[lr + 1][lc + 1] = (&T.d[0][0])[re[j]];
             A.h[lr + 1][lc + 1] = (&T.h[0][0])[re[j]];
-            if (rd[j]) m = min(m, rd[j]);
+            const unsigned rd = rel(R.d[j]);
+            if (R.d[j] >= base) m = min(m, rd);
+            ring_beyond |= rd == 0xFFFFFFFFu && R.d[j] != ~0ull;
         }
     }
     unsigned x[4][4];           // the map's
@@ -207,7 +209,10 @@ __device__ bool next_window(const PoolMap &map, const TileGeo &g, DistTile<SR> &
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             x[r][c] = key_reached(k[c]) ? rel(key_dunits(k[c])) : 0xFFFFFFFFu;
-            if (!((known >> (4 * r + c)) & 1u)) m = min(m, x[r][c]);
+            if (!((known >> (4 * r + c)) & 1u)) {
+                m = min(m, x[r][c]);
+                map_beyond |= x[r][c] == 0xFFFFFFFFu && key_reached(k[c]);
+            }
             A.d[4 * by + r + 1][4 * bx + c + 1] = B.d[r][c];
             A.h[4 * by + r + 1][4 * bx + c + 1] = S.h[r][c];
         }
@@ -239,6 +244,8 @@ __device__ bool next_window(const PoolMap &map, const TileGeo &g, DistTile<SR> &
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < ST / 32; ++i) m = min(m, T.red[0][i]);
+    // what lies beyond 32 bits of `base` may lie in the window, or be all there is
+    *lost |= (map_beyond && m > 0xFFFFFFFFu - win) || (ring_beyond && m == 0xFFFFFFFFu);
     S.base = base + m;
     // (2^32 - 1, unreached or beyond 32 bits, is no distance)
     auto in = [&](unsigned d) { return d <= m ? 0u : d == 0xFFFFFFFFu ? win : min(d - m, win); };
@@ -257,7 +264,8 @@ __device__ bool next_window(const PoolMap &map, const TileGeo &g, DistTile<SR> &
         }
 #pragma unroll
     for (int j = 0; j < PER; ++j)
-        if (re[j] >= 0) (&T.d[0][0])[re[j]] = in(rd[j]);
+        if (re[j] >= 0)
+            (&T.d[0][0])[re[j]] = R.d[j] < S.base ? 0u : (unsigned)min(R.d[j] - S.base, (unsigned long long)win);
     *before = sum;
     bool more = false;
 #pragma unroll
