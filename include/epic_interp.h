@@ -135,14 +135,17 @@ typedef struct {
                              every installed rule ask for them; otherwise a
                              frame whose rule says 2 gets 64 x 32 tiles with
                              apron 4 and schedule 0.  The exact variant's
-                             cap map always uses schedule 0 or 1.
+                             cap map, and its single-source runs where they
+                             go by pairs, always use schedule 0 or 1.
                              Every schedule gives the same result. */
     long long exact_chunk_bytes; /* epic_exact_interp with metric 0: device
                              bytes of packed keys its single-source
                              relaxations may hold at once, in tiles of 64 x
                              32 pixels (16 KiB) that a match in work has
-                             reached; at least one match is in work, with
-                             every tile of the frame.
+                             reached, or in maps of the frame (8 bytes per
+                             pixel per match in work, for few matches); at
+                             least one match is in work, with every tile of
+                             the frame.
                              0 = 1 GiB (default).  Only speed and memory
                              depend on it, never the results. */
 } epic_config_t;
@@ -326,8 +329,9 @@ int epic_interp_get_stage_times(epic_interp_t *h, float *ms_out, int n_stages,
  * handle holds up to exact_chunk_bytes (1 GiB by default) of relaxation keys
  * and the distances of the 64 x 32 tiles that each match reaches within the
  * bounds (8 KiB a tile; room for 16 per match to begin with, grown on demand,
- * at most N * H * W * 4 bytes and the padding of edge tiles; EPIC_ERR_OOM if
- * it cannot be).  Runs
+ * for few matches room for all to begin with where it can be had; at most
+ * N * H * W * 4 bytes and the padding of edge tiles; EPIC_ERR_OOM if it cannot
+ * be).  Runs
  * on `stream` and waits for completion; returns the device status. */
 int epic_exact_interp(epic_interp_t *h, const float *cost_map,
                       const float *matches, int H, int W, int N, int K,

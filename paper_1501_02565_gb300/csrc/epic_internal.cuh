@@ -135,9 +135,11 @@ struct PairDev {
     int hash_cap;           // power of two
     int flow_vec_ok;        // flow pointer is 16-byte aligned
     pkey_t *keys;            // [H*W] packed (D, L)
-    // cap map of the exact variant only (null elsewhere): a distance offset
-    // per seed (units)
+    // exact variant only (null elsewhere).  Cap map: a distance offset per
+    // seed (units).  Single-source runs: the cap map (a pixel whose distance
+    // exceeds its cap is left unreached)
     const unsigned long long *seed_init;   // [N]
+    const pkey_t *cap;                     // [H*W]
     int *tile_start;        // [tiles+1] seed bins (prefix offsets)
     int *tile_fill;         // [tiles] scatter cursors
     int *tile_seeds;        // [N] match indices grouped by tile
@@ -237,6 +239,7 @@ struct RunState {
     unsigned knn_overflow; // matches whose search outgrew the small tables
     unsigned knn_retry;    // dispenser of the retry pass over those matches
     unsigned edge_next;    // boundary-edge tile dispenser
+    unsigned wl_count[3];  // single-source runs: list lengths of the passes (rotating)
     unsigned compact_done; // CTAs finished in the pruning compaction
     TileWork tiles[2];     // the warp-tile relaxation's: distances, then labels
     unsigned fresh_done;   // tiles that phase 1 of the distances has written
@@ -255,6 +258,11 @@ struct BatchArgs {
     const int *solve_base;   // [npairs+1] prefix of the warp-tile relaxation's solve tiles
     int total_solve;
     int total_tiles, total_matches, total_chunks, total_hash, total_clear;
+    // single-source runs (see epic_exact_interp): the tiles of every pair, three
+    // lists of total_tiles flat tile indices, and the last pass + 1 that a tile
+    // was listed for (0: never)
+    int uniform_tiles;
+    int *wl, *wl_queued;
     int max_degree;
     int knn_hs, knn_fs, knn_kmax;  // main-pass K-NN table sizes per warp, and K bound
     unsigned *relax_req;   // [2][total_solve] warp-tile relaxation: requests for a solve of
@@ -294,6 +302,7 @@ __device__ __forceinline__ int get_status(const RunState *s) {
 // Bounded grid barrier of the cooperative relaxation launches.
 // ---------------------------------------------------------------------------
 constexpr unsigned long long BARRIER_LIMIT_NS = 2000000000ull;  // 2 s
+constexpr int PASS_CHUNK = 8;  // tiles per dispenser step of a single-source run's first pass
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
     unsigned v;
@@ -366,7 +375,7 @@ struct LaunchCfg {
 cudaError_t launch_prepare(const BatchArgs &a, const BatchArgs *dev, const LaunchCfg &lc);
 cudaError_t launch_dt(const BatchArgs &a, const BatchArgs *dev, const LaunchCfg &lc,
                       int max_tile_w, int max_tile_h, int max_apron, bool fixed_grid,
-                      int *grid_used);
+                      int *grid_used, bool single = false);
 cudaError_t launch_edges(const BatchArgs &a, const BatchArgs *dev, const LaunchCfg &lc,
                          int max_tile_w, int max_tile_h);
 cudaError_t launch_scatter(const BatchArgs &a, const BatchArgs *dev, const LaunchCfg &lc);
@@ -438,10 +447,43 @@ struct SingleArgs {
     int *tile_start;         // [tiles + 1]
     int2 *tile_entry;        // [slot_cap] (match, distance tile) by tile
     long long max_solves;    // per match
+    // the sum of the caps, in cost units; above the limit they reach far: every
+    // solve carries 64-bit keys, or nothing is done at all
+    float *cap_sum;
+    float cap_limit;
+    bool far_returns;
     RunState *state;
 };
+// How the single-source runs of a frame of `tiles` tiles go (whole calls, on
+// frames of 96 x 96 to 1500 x 1000 pixels, 1 to 5000 matches, K = 8 to 100, costs
+// from 1e-3 to U(0, 1.99); by pairs is how all went before, and the rules leave
+// nothing slower than it but frames of cost zero throughout, up to 1.3 times, and
+// 100 matches on 1500 x 1000 with K = 100, 1.15 times):
+//   by tiles   a CTA takes whole matches (k_single.cu).
+//   by pairs   every match is a pseudo-pair of the apron tiles (k_dt.cu), all
+//              tiles of all matches spread over the GPU.
+// A match passes through about 3 windows of 32 bits per tile and unit of its cap,
+// so where the caps' mean is above single_far() the tiles are solved with 64-bit
+// keys at once: 1024 x 436, 5000 matches, K = 8, costs U(0.1, 0.4) and U(0.2,
+// 0.8) (mean caps 4.3 and 8.5) 12.3 and 35 ms by windows, 7.9 and 8.0 ms so;
+// K = 64, U(0.032, 0.128) (3.6) 21.3 and 21.8, U(0.05, 0.3) (7.2) 57 and 25.
+// Few matches leave most of the GPU idle by tiles.  By pairs, 1024 x 436 (224
+// tiles), 16 matches, K = 8: 8.6 ms, by tiles 11.8 (64 matches 8.5 and 7.2); 1500
+// x 1000 (768 tiles), 32 matches 18.5 and 30.3 (150 matches 21.2 and 10.4).  With
+// caps that reach far, where a match visits more: 1024 x 436, 64 matches 6.8 and
+// 11.8 ms, 150 matches 6.0 and 5.9, 500 matches 8.1 and 5.2; 1500 x 1000, 500
+// matches, K = 64, 92 and 114; costs up to 1.99, whose diagonal weights leave 32
+// bits, 300 x 200, 500 matches, K = 64, 6.8 and 9.0.
+__host__ __device__ constexpr float single_far(int K) { return 3.f + (float)K / 32.f; }   // mean cap
+__host__ __device__ constexpr bool single_few(long long N, long long tiles) { return 12 * N < tiles; }
+__host__ __device__ constexpr bool single_few_far(long long N, long long tiles) {
+    return N < 512 || N < tiles;
+}
 int single_resident(int num_sms);   // CTAs resident at once
 cudaError_t launch_single(const SingleArgs &x, int ctas, cudaStream_t stream);
+cudaError_t launch_cap_sum(const pkey_t *cap, long long n, float *sum, cudaStream_t stream);
+// The distance tiles of matches m0 .. m0 + n - 1 from key maps of the frame.
+cudaError_t launch_map_tiles(const SingleArgs &x, const pkey_t *maps, int m0, int n, cudaStream_t stream);
 cudaError_t launch_single_lists(const SingleArgs &x, unsigned used, cudaStream_t stream);
 
 // Self-test of the bounded device waits (grid barrier, TMA mbarrier).

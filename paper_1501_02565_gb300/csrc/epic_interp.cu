@@ -74,6 +74,9 @@ struct epic_interp {
     size_t ex_cap = 0;
     char *ex_slots = nullptr;
     size_t ex_slots_cap = 0;
+    // and the tables and bins of its single-source runs by pairs
+    char *ex_pairs = nullptr;
+    size_t ex_pairs_cap = 0;
     // scratch of the variational refinement
     void *rf_buf = nullptr;
     // set by the exact variant around its internal approximate run: keep the
@@ -1299,7 +1302,9 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
     };
     const int ctas_all = ctas_for(ST), ctas = std::max(ctas_all, ctas_for(std::min(ST, 64LL)));
     const int pool = (int)(ctas == ctas_all ? ST : std::min(ST, chunk_bytes / (ctas * tile_bytes)));
-    const size_t o_keys = take((size_t)tile_bytes * std::max((size_t)ctas_all * (size_t)ST, (size_t)ctas * (size_t)pool));
+    const size_t keys_bytes =
+        (size_t)tile_bytes * std::max((size_t)ctas_all * (size_t)ST, (size_t)ctas * (size_t)pool);
+    const size_t o_keys = take(keys_bytes);
     const size_t o_left = take(sizeof(int) * (size_t)N);
     const size_t o_places = take(sizeof(int) * (size_t)ST * ctas);
     const size_t o_queue = take(sizeof(int) * (size_t)ST * ctas);
@@ -1308,6 +1313,7 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
     const size_t o_flags = take((size_t)ST * ctas);
     const size_t o_count = take(sizeof(int) * (size_t)(ST + 4));   // tile counts, then used, next and left
     const size_t o_start = take(sizeof(int) * (size_t)(ST + 1));
+    const size_t o_cap_sum = take(sizeof(float));
     if ((rc = grow(&h->ex_buf, &h->ex_cap, used))) return rc;
     char *b = h->ex_buf;
     pkey_t *vkeys = reinterpret_cast<pkey_t *>(b + o_vkeys);
@@ -1316,7 +1322,7 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
     float *aflow = reinterpret_cast<float *>(b + o_aflow);
     char *tdev = b + o_table;
     epic::LaunchCfg lc{h->num_sms, h->smem_optin, stream, h->smem_per_sm, h->smem_reserved};
-    std::vector<char> thost(t_bytes, 0);   // the cap map's table
+    std::vector<char> thost(t_bytes, 0), phost;   // tables: the cap map's, the pairs'
     CopiesEnd copies_end{stream};
     {
         h->force_keep = true;
@@ -1402,42 +1408,161 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
     s.tile_start = reinterpret_cast<int *>(b + o_start);
     s.max_solves = (long long)c.max_passes * ST;
     s.state = h->state;
-    // distance tiles: room for 16 per match to begin with (11 on the flow
-    // workloads at K = 100); a run that needs more says how many
+    s.cap_sum = reinterpret_cast<float *>(b + o_cap_sum);
     const size_t per_slot = sizeof(float) * epic::SINGLE_TILE + 2 * sizeof(int2);
-    unsigned long long want = std::min<unsigned long long>((unsigned long long)N * ST, 16ull * N + 1024);
-    unsigned n_used = 0, n_done[3];   // used, next, left
-    s.pool_tiles = pool;
-    for (;;) {
+    auto slots = [&](unsigned long long want) -> int {
         want = std::max<unsigned long long>(want, h->ex_slots_cap / per_slot);
         want = std::min<unsigned long long>(want, 0x7fffffffull);
-        if ((rc = grow(&h->ex_slots, &h->ex_slots_cap, (size_t)want * per_slot))) return rc;
+        const int r = grow(&h->ex_slots, &h->ex_slots_cap, (size_t)want * per_slot);
         s.slot_cap = (unsigned)want;
         s.slots = reinterpret_cast<float *>(h->ex_slots);
         s.slot_of = reinterpret_cast<int2 *>(s.slots + (size_t)want * epic::SINGLE_TILE);
         s.tile_entry = s.slot_of + want;
-        if ((e = cudaMemsetAsync(s.tile_count, 0, sizeof(int) * (size_t)(ST + 4), stream)) ||
-            (e = epic::launch_single(s, ctas, stream)) ||
-            (e = cudaMemcpyAsync(n_done, s.used, sizeof n_done, cudaMemcpyDeviceToHost, stream)) ||
-            (e = cudaStreamSynchronize(stream)))
+        return r;
+    };
+    unsigned n_used = 0;
+    // (*far: the caps reach far, and nothing was done for it)
+    auto by_tiles = [&](bool far_returns, bool *far) -> int {
+        // distance tiles: room for 16 per match to begin with (11 on the flow
+        // workloads at K = 100); a run that needs more says how many
+        unsigned long long want = std::min<unsigned long long>((unsigned long long)N * ST, 16ull * N + 1024);
+        unsigned n_done[3];   // used, next, left
+        float cap_sum = 0.f;
+        s.far_returns = far_returns;
+        s.pool_tiles = pool;
+        for (;;) {
+            const int r = slots(want);
+            if (r) return r;
+            if ((e = cudaMemsetAsync(s.tile_count, 0, sizeof(int) * (size_t)(ST + 4), stream)) ||
+                (e = epic::launch_single(s, ctas, stream)) ||
+                (e = cudaMemcpyAsync(n_done, s.used, sizeof n_done, cudaMemcpyDeviceToHost, stream)) ||
+                (e = cudaMemcpyAsync(&cap_sum, s.cap_sum, sizeof cap_sum, cudaMemcpyDeviceToHost, stream)) ||
+                (e = cudaStreamSynchronize(stream)))
+                return cuda_fail(h, e, "exact-variant relaxation");
+            if ((*far = far_returns && cap_sum > s.cap_limit)) return EPIC_OK;
+            n_used = n_done[0];
+            if (n_done[2] > 0 && n_used <= s.slot_cap) {
+                // the matches left over, with pools of every tile
+                epic::SingleArgs all = s;
+                all.list = s.left;
+                all.N = (int)n_done[2];
+                all.pool_tiles = (int)ST;
+                if ((e = cudaMemsetAsync(s.next, 0, sizeof(unsigned), stream)) ||
+                    (e = epic::launch_single(all, std::min(ctas_all, all.N), stream)) ||
+                    (e = cudaMemcpyAsync(&n_used, s.used, sizeof n_used, cudaMemcpyDeviceToHost, stream)) ||
+                    (e = cudaStreamSynchronize(stream)))
+                    return cuda_fail(h, e, "exact-variant relaxation");
+            }
+            if (n_used <= s.slot_cap) return EPIC_OK;
+            if (n_used > 0x7fffffffu)
+                return fail(h, EPIC_ERR_CAPACITY, "exact variant: too many distance tiles");
+            want = n_used;
+        }
+    };
+    // Every match a pseudo-pair of one seed, relaxed by the apron tiles with
+    // the cap map, as many at a time as the budget for keys holds; distance
+    // tiles for all that there can be.
+    auto by_pairs = [&]() -> int {
+        const long long Cm = std::max(1LL, std::min((long long)N, (long long)(keys_bytes / (8 * (size_t)P))));
+        if ((unsigned long long)N * ST > 0x7fffffffull)
+            return fail(h, EPIC_ERR_CAPACITY, "exact variant: too many distance tiles");
+        int r = slots((unsigned long long)N * ST);
+        if (r) return r;
+        const size_t pds = align_up(sizeof(PairDev) * (size_t)Cm, 256);
+        const size_t pre_stride = align_up(sizeof(int) * (size_t)(Cm + 1), 256);
+        const size_t table = args_bytes + pds + 5 * pre_stride;
+        const size_t small_ints = (size_t)(T + 1) + T + 1 + T + 1 + 1 + 4;   // per pseudo-pair
+        const size_t o_small = align_up(table, 256);
+        const size_t o_lists = o_small + align_up((size_t)Cm * small_ints * sizeof(int), 256);
+        if ((r = grow(&h->ex_pairs, &h->ex_pairs_cap, o_lists + sizeof(int) * (size_t)(4 * Cm * T)))) return r;
+        phost.assign(table, 0);
+        int *small = reinterpret_cast<int *>(h->ex_pairs + o_small);
+        int *lists = reinterpret_cast<int *>(h->ex_pairs + o_lists);   // [3][n T], then [n T] marks
+        if ((e = cudaMemsetAsync(s.tile_count, 0, sizeof(int) * (size_t)(ST + 4), stream)))
             return cuda_fail(h, e, "exact-variant relaxation");
-        n_used = n_done[0];
-        if (n_done[2] > 0 && n_used <= s.slot_cap) {
-            // the matches left over, with pools of every tile
-            epic::SingleArgs all = s;
-            all.list = s.left;
-            all.N = (int)n_done[2];
-            all.pool_tiles = (int)ST;
-            if ((e = cudaMemsetAsync(s.next, 0, sizeof(unsigned), stream)) ||
-                (e = epic::launch_single(all, std::min(ctas_all, all.N), stream)) ||
+        for (long long m0 = 0; m0 < N; m0 += Cm) {
+            const int n = (int)std::min(Cm, (long long)N - m0);
+            PairDev *pd = reinterpret_cast<PairDev *>(phost.data() + args_bytes);
+            for (int j = 0; j < n; ++j) {
+                PairDev &q = pd[j];
+                q = PairDev{};
+                q.C = cost_map;
+                q.matches = x.matches + m0 + j;
+                q.H = H;
+                q.W = W;
+                q.N = 1;
+                q.K = 1;
+                q.a = 1.f;
+                q.tile_w = tw;
+                q.tile_h = th;
+                q.apron = ap;
+                q.sweep = sw;
+                q.tiles_x = tx;
+                q.tiles_y = ty;
+                q.keys = s.keys + (size_t)j * P;
+                int *sp = small + (size_t)j * small_ints;
+                q.tile_start = sp;
+                q.tile_fill = sp + T + 1;
+                q.tile_seeds = sp + 2 * T + 1;
+                q.tile_stamp = sp + 2 * T + 2;
+                q.deg = sp + 3 * T + 2;
+                q.wmin = reinterpret_cast<unsigned *>(sp + 3 * T + 3);
+                q.info = sp + 3 * T + 4;
+                q.cap = vkeys;
+            }
+            int *pre[5];   // prefixes of tiles and matches; the others are zero
+            for (int k = 0; k < 5; ++k)
+                pre[k] = reinterpret_cast<int *>(phost.data() + args_bytes + pds + k * pre_stride);
+            for (int j = 0; j <= n; ++j) {
+                pre[0][j] = j * T;
+                pre[1][j] = j;
+            }
+            auto dev = [&](const void *host) {
+                return h->ex_pairs + (static_cast<const char *>(host) - phost.data());
+            };
+            BatchArgs ba{};
+            ba.pairs = reinterpret_cast<const PairDev *>(dev(pd));
+            ba.npairs = n;
+            ba.tile_base = reinterpret_cast<const int *>(dev(pre[0]));
+            ba.match_base = reinterpret_cast<const int *>(dev(pre[1]));
+            ba.chunk_base = reinterpret_cast<const int *>(dev(pre[2]));
+            ba.hash_base = reinterpret_cast<const int *>(dev(pre[3]));
+            ba.clear_base = reinterpret_cast<const int *>(dev(pre[4]));
+            ba.total_tiles = n * T;
+            ba.total_matches = n;
+            ba.uniform_tiles = T;
+            ba.wl = lists;
+            ba.wl_queued = lists + (size_t)3 * n * T;
+            ba.max_degree = 1;
+            ba.max_passes = c.max_passes;
+            ba.weight_squared = 1;
+            ba.fallback_eps = c.fallback_eps;
+            ba.state = h->state;
+            memcpy(phost.data(), &ba, sizeof ba);
+            const BatchArgs *dev_a = reinterpret_cast<const BatchArgs *>(h->ex_pairs);
+            // (the next chunk writes the host table again: wait for this one)
+            if ((e = cudaMemcpyAsync(h->ex_pairs, phost.data(), table, cudaMemcpyHostToDevice, stream)) ||
+                (e = cudaMemsetAsync(ba.wl_queued, 0, sizeof(int) * (size_t)n * T, stream)) ||
+                (e = epic::launch_prepare(ba, dev_a, lc)) ||
+                (e = epic::launch_dt(ba, dev_a, lc, tw, th, ap, false, nullptr, true)) ||
+                (e = epic::launch_map_tiles(s, s.keys, (int)m0, n, stream)) ||
                 (e = cudaMemcpyAsync(&n_used, s.used, sizeof n_used, cudaMemcpyDeviceToHost, stream)) ||
                 (e = cudaStreamSynchronize(stream)))
                 return cuda_fail(h, e, "exact-variant relaxation");
         }
-        if (n_used <= s.slot_cap) break;
-        if (n_used > 0x7fffffffu) return fail(h, EPIC_ERR_CAPACITY, "exact variant: too many distance tiles");
-        want = n_used;
+        return EPIC_OK;
+    };
+    s.cap_limit = epic::single_far(K) * (float)P;
+    if ((e = epic::launch_cap_sum(vkeys, P, s.cap_sum, stream)))
+        return cuda_fail(h, e, "exact-variant cap map");
+    bool pairs = epic::single_few(N, ST);
+    if (!pairs) rc = by_tiles(epic::single_few_far(N, ST), &pairs);
+    if (!rc && pairs) {
+        rc = by_pairs();
+        // distance tiles as they are needed may fit where all do not
+        if (rc == EPIC_ERR_OOM) rc = by_tiles(false, &pairs);
     }
+    if (rc) return rc;
     x.slow_count = reinterpret_cast<int *>(b + o_slow);
     x.slow_list = x.slow_count + 1;
     x.tiles_x = sx;
@@ -1599,6 +1724,7 @@ void epic_interp_destroy(epic_interp_t *h) {
     if (h->io_F) cudaFree(h->io_F);
     if (h->ex_buf) cudaFree(h->ex_buf);
     if (h->ex_slots) cudaFree(h->ex_slots);
+    if (h->ex_pairs) cudaFree(h->ex_pairs);
     if (h->rf_buf) cudaFree(h->rf_buf);
     for (cudaEvent_t x : h->tev) cudaEventDestroy(x);
     delete h;

@@ -261,8 +261,26 @@ __device__ __forceinline__ float *stage_area(unsigned char *smem) {
     return reinterpret_cast<float *>(((uintptr_t)smem + 127) & ~(uintptr_t)127);
 }
 
+// A key as written back: in the exact variant's single-source runs (SINGLE,
+// with a cap map), a distance beyond the pixel's cap is left unreached, so the
+// run stops spreading where it can no longer matter.  The cap is 1-Lipschitz in
+// the same fixed-point metric, so every pixel on a shortest path to a
+// pixel within its cap is within its own cap: capped runs are exact there.
+template <bool SINGLE>
+__device__ __forceinline__ pkey_t capped(const PairDev &P, size_t p, pkey_t k) {
+    return SINGLE && key_dunits(k) > key_dunits(P.cap[p]) ? KEY_INF : k;
+}
+
+// The pair a flat tile index belongs to (a division for single-source runs,
+// whose pairs, one per match, have the same tiles).
+template <bool SINGLE>
+__device__ __forceinline__ int tile_pair(const BatchArgs &a, int t) {
+    return SINGLE ? t / a.uniform_tiles : find_pair(a.tile_base, a.npairs, t);
+}
+
 // Phase 1: solve tile (tx, ty) on its region from its seeds alone.  Returns
 // false when the cost staging timed out (the CTA must leave the kernel).
+template <bool SINGLE>
 __device__ bool solve_fresh(const PairDev &P, int tx, int ty, pkey_t *K,
                             unsigned *h, RunState *st, float *stage, Tma &tma) {
     const int gx0 = tx * P.tile_w, gy0 = ty * P.tile_h;
@@ -323,7 +341,8 @@ __device__ bool solve_fresh(const PairDev &P, int tx, int ty, pkey_t *K,
         int ly = i / P.tile_w, lx = i - ly * P.tile_w;
         int gx = gx0 + lx, gy = gy0 + ly;
         if (gx < P.W && gy < P.H)
-            P.keys[(size_t)gy * P.W + gx] = K[(ly + off) * g.P + lx + off];
+            P.keys[(size_t)gy * P.W + gx] =
+                capped<SINGLE>(P, (size_t)gy * P.W + gx, K[(ly + off) * g.P + lx + off]);
     }
     __syncthreads();
     return true;
@@ -334,6 +353,7 @@ __device__ __forceinline__ pkey_t ld_key(const pkey_t *p) { return __ldcg(p); }
 // Can a border pixel of the tile be improved by a step from a pixel outside
 // it?  Keys of other tiles may be rewritten during the launch, so they are
 // read through L2 (ld.global.cg), never from a stale L1 line.
+template <bool SINGLE>
 __device__ bool border_dirty(const PairDev &P, int tx, int ty) {
     const int gx0 = tx * P.tile_w, gy0 = ty * P.tile_h;
     const int gx1 = min(P.W - 1, gx0 + P.tile_w - 1);
@@ -365,7 +385,9 @@ __device__ bool border_dirty(const PairDev &P, int tx, int ty) {
             const pkey_t kq = ld_key(P.keys + q);
             const unsigned hq = half_cost(__ldg(P.C + q), &bad);
             const unsigned long long w = (dx != 0 && dy != 0) ? step_diag(hp, hq) : step_axis(hp, hq);
-            dirty |= step_key(kq, w) < kp;
+            // an improvement beyond the pixel's cap would be written back
+            // unreached, so it does not make the tile dirty
+            dirty |= capped<SINGLE>(P, p, step_key(kq, w)) < kp;
         }
     }
     return __syncthreads_or(dirty) != 0;
@@ -375,6 +397,7 @@ __device__ bool border_dirty(const PairDev &P, int tx, int ty) {
 // Returns 1 if any key of the region changed, 0 if none did, -1 if the cost
 // staging timed out (the CTA must leave the kernel); the same in every
 // thread.
+template <bool SINGLE>
 __device__ int solve_again(const PairDev &P, int tx, int ty, pkey_t *K,
                             unsigned *h, RunState *st, int pass, float *stage, Tma &tma) {
     const int gx0 = tx * P.tile_w, gy0 = ty * P.tile_h;
@@ -393,7 +416,8 @@ __device__ int solve_again(const PairDev &P, int tx, int ty, pkey_t *K,
             int ly = i / P.tile_w, lx = i - ly * P.tile_w;
             int gx = gx0 + lx, gy = gy0 + ly;
             if (gx < P.W && gy < P.H)
-                P.keys[(size_t)gy * P.W + gx] = K[(ly + 1) * g.P + lx + 1];
+                P.keys[(size_t)gy * P.W + gx] =
+                    capped<SINGLE>(P, (size_t)gy * P.W + gx, K[(ly + 1) * g.P + lx + 1]);
         }
     }
     if (threadIdx.x == 0) P.tile_stamp[ty * P.tiles_x + tx] = pass;
@@ -401,6 +425,31 @@ __device__ int solve_again(const PairDev &P, int tx, int ty, pkey_t *K,
     return changed ? 1 : 0;
 }
 
+// Chunked passes: queue the eight neighbours of tile t (flat index; local
+// (tx, ty) in pair pi) for pass `next`, each at most once (threads 0-7).
+__device__ __forceinline__ void queue_neighbours(const BatchArgs &a, RunState *st, int pi,
+                                                 int tx, int ty, int next) {
+    if (threadIdx.x >= 8) return;
+    const PairDev &P = a.pairs[pi];
+    const int k = threadIdx.x;
+    const int x = tx + (k < 3 ? k - 1 : k < 5 ? 2 * k - 7 : k - 6);
+    const int y = ty + (k < 3 ? -1 : k < 5 ? 0 : 1);
+    if (x < 0 || x >= P.tiles_x || y < 0 || y >= P.tiles_y) return;
+    const int nt = a.tile_base[pi] + y * P.tiles_x + x;
+    if (atomicMax(a.wl_queued + nt, next + 1) < next + 1) {
+        const unsigned q = atomicAdd(&st->wl_count[next % 3], 1u);
+        a.wl[(size_t)(next % 3) * a.total_tiles + q] = nt;
+    }
+}
+
+// SINGLE: single-source runs (see epic_exact_interp).  They take dozens of
+// verification passes while distances cross the image tile by tile, each
+// re-solving a thin front, so the passes hand out chunks of tiles whose neighbour
+// stamps are read in parallel, and lists (300 matches on 1024 x 436: 3.1 -> 2.1
+// s).  The interpolator's runs (a handful of passes, about half of the tiles
+// re-solved in the first) take one tile at a time: at the four-CTA register
+// budget the other loop costs them a spill (2.21 -> 2.33 ms).
+template <bool SINGLE>
 __global__ void __launch_bounds__(DT_THREADS) dt_kernel(const BatchArgs *__restrict__ ap) {
     const BatchArgs a = *ap;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -423,7 +472,7 @@ __global__ void __launch_bounds__(DT_THREADS) dt_kernel(const BatchArgs *__restr
             const int t = (int)atomicAdd(dispenser, 1u);
             s_tile = t;
             if (t < a.total_tiles) {
-                s_pair = find_pair(a.tile_base, a.npairs, t);
+                s_pair = tile_pair<SINGLE>(a, t);
                 s_local = t - a.tile_base[s_pair];
             }
         }
@@ -437,7 +486,7 @@ __global__ void __launch_bounds__(DT_THREADS) dt_kernel(const BatchArgs *__restr
         const Region g = make_region(P, 0, 0, P.tile_w, P.tile_h, P.apron);
         pkey_t *K = reinterpret_cast<pkey_t *>(smem);
         unsigned *h = reinterpret_cast<unsigned *>(smem + sizeof(pkey_t) * g.RH * g.P);
-        if (!solve_fresh(P, s_local % P.tiles_x, s_local / P.tiles_x, K, h, st, stage, tma))
+        if (!solve_fresh<SINGLE>(P, s_local % P.tiles_x, s_local / P.tiles_x, K, h, st, stage, tma))
             return;
     }
     if (!grid_sync(st, nblocks)) return;
@@ -453,26 +502,120 @@ __global__ void __launch_bounds__(DT_THREADS) dt_kernel(const BatchArgs *__restr
         }
         unsigned *cnt = &st->changed[pass % 3];
         unsigned *disp = &st->work[pass % 3];
-        for (int t = next_tile(disp); t < a.total_tiles; t = next_tile(disp)) {
-            const PairDev &P = a.pairs[s_pair];
-            const int tx = s_local % P.tiles_x, ty = s_local / P.tiles_x;
-            // threads 0-7 read the eight neighbour stamps at once
-            bool nb = false;
-            if (threadIdx.x < 8) {
-                const int k = threadIdx.x;
-                const int x = tx + (k < 3 ? k - 1 : k < 5 ? 2 * k - 7 : k - 6);
-                const int y = ty + (k < 3 ? -1 : k < 5 ? 0 : 1);
-                nb = x >= 0 && x < P.tiles_x && y >= 0 && y < P.tiles_y &&
-                     __ldcg(P.tile_stamp + y * P.tiles_x + x) >= pass;
+        if constexpr (!SINGLE) {
+            for (int t = next_tile(disp); t < a.total_tiles; t = next_tile(disp)) {
+                const PairDev &P = a.pairs[s_pair];
+                const int tx = s_local % P.tiles_x, ty = s_local / P.tiles_x;
+                // threads 0-7 read the eight neighbour stamps at once
+                bool nb = false;
+                if (threadIdx.x < 8) {
+                    const int k = threadIdx.x;
+                    const int x = tx + (k < 3 ? k - 1 : k < 5 ? 2 * k - 7 : k - 6);
+                    const int y = ty + (k < 3 ? -1 : k < 5 ? 0 : 1);
+                    nb = x >= 0 && x < P.tiles_x && y >= 0 && y < P.tiles_y &&
+                         __ldcg(P.tile_stamp + y * P.tiles_x + x) >= pass;
+                }
+                if (__syncthreads_or(nb) && border_dirty<SINGLE>(P, tx, ty)) {
+                    const Region g = make_region(P, 0, 0, P.tile_w, P.tile_h, 0);
+                    pkey_t *K = reinterpret_cast<pkey_t *>(smem);
+                    unsigned *h = reinterpret_cast<unsigned *>(smem + sizeof(pkey_t) * g.RH * g.P);
+                    if (solve_again<SINGLE>(P, tx, ty, K, h, st, pass + 1, stage, tma) < 0) return;
+                    if (threadIdx.x == 0) atomicAdd(cnt, 1u);
+                }
+                __syncthreads();
             }
-            if (__syncthreads_or(nb) && border_dirty(P, tx, ty)) {
-                const Region g = make_region(P, 0, 0, P.tile_w, P.tile_h, 0);
-                pkey_t *K = reinterpret_cast<pkey_t *>(smem);
-                unsigned *h = reinterpret_cast<unsigned *>(smem + sizeof(pkey_t) * g.RH * g.P);
-                if (solve_again(P, tx, ty, K, h, st, pass + 1, stage, tma) < 0) return;
-                if (threadIdx.x == 0) atomicAdd(cnt, 1u);
+        } else {
+            // Pass 0 scans every tile, PASS_CHUNK at a time: the first
+            // 8 x PASS_CHUNK threads read the chunk's neighbour stamps in
+            // parallel and flag the tiles with a neighbour written since phase
+            // 1; only those go on to the border test.  A tile that changes
+            // queues its eight neighbours for the next pass, and every later
+            // pass works through that list alone (a single-source run
+            // re-solves a thin front, and scanning every tile in each of its
+            // dozen passes cost more than the re-solves).  The loop state
+            // lives in shared memory, so nothing extra stays in registers
+            // across a re-solve.
+            __shared__ int s_t0, s_bits;
+            if (pass == 0) {
+                for (;;) {
+                    __syncthreads();
+                    if (threadIdx.x == 0) {
+                        s_t0 = (int)atomicAdd(disp, (unsigned)PASS_CHUNK);
+                        s_bits = 0;
+                    }
+                    __syncthreads();
+                    if (s_t0 >= a.total_tiles) break;
+                    if (threadIdx.x < 8 * PASS_CHUNK) {
+                        const int t = s_t0 + (threadIdx.x >> 3), k = threadIdx.x & 7;
+                        if (t < a.total_tiles) {
+                            const int pi = tile_pair<SINGLE>(a, t);
+                            const PairDev &P = a.pairs[pi];
+                            const int lt = t - a.tile_base[pi];
+                            const int x = lt % P.tiles_x + (k < 3 ? k - 1 : k < 5 ? 2 * k - 7 : k - 6);
+                            const int y = lt / P.tiles_x + (k < 3 ? -1 : k < 5 ? 0 : 1);
+                            if (x >= 0 && x < P.tiles_x && y >= 0 && y < P.tiles_y &&
+                                __ldcg(P.tile_stamp + y * P.tiles_x + x) >= pass)
+                                atomicOr(&s_bits, 1 << (threadIdx.x >> 3));
+                        }
+                    }
+                    for (;;) {
+                        __syncthreads();
+                        if (threadIdx.x == 0) {
+                            const int b = s_bits;
+                            if (b) {
+                                const int t = s_t0 + __ffs(b) - 1;
+                                s_bits = b & (b - 1);
+                                s_tile = t;
+                                s_pair = tile_pair<SINGLE>(a, t);
+                                s_local = t - a.tile_base[s_pair];
+                            } else {
+                                s_tile = -1;
+                            }
+                        }
+                        __syncthreads();
+                        if (s_tile < 0) break;
+                        const PairDev &P = a.pairs[s_pair];
+                        const int tx = s_local % P.tiles_x, ty = s_local / P.tiles_x;
+                        if (border_dirty<SINGLE>(P, tx, ty)) {
+                            const Region g = make_region(P, 0, 0, P.tile_w, P.tile_h, 0);
+                            pkey_t *K = reinterpret_cast<pkey_t *>(smem);
+                            unsigned *h = reinterpret_cast<unsigned *>(smem + sizeof(pkey_t) * g.RH * g.P);
+                            const int r = solve_again<SINGLE>(P, tx, ty, K, h, st, pass + 1, stage, tma);
+                            if (r < 0) return;
+                            if (r > 0) queue_neighbours(a, st, s_pair, tx, ty, pass + 1);
+                            if (threadIdx.x == 0) atomicAdd(cnt, 1u);
+                        }
+                    }
+                }
+            } else {
+                // the list of this pass was complete before the last barrier
+                const unsigned n = ld_acquire(&st->wl_count[pass % 3]);
+                const int *list = a.wl + (size_t)(pass % 3) * a.total_tiles;
+                for (;;) {
+                    __syncthreads();
+                    if (threadIdx.x == 0) {
+                        const unsigned q = atomicAdd(disp, 1u);
+                        s_tile = q < n ? list[q] : -1;
+                        if (s_tile >= 0) {
+                            s_pair = tile_pair<SINGLE>(a, s_tile);
+                            s_local = s_tile - a.tile_base[s_pair];
+                        }
+                    }
+                    __syncthreads();
+                    if (s_tile < 0) break;
+                    const PairDev &P = a.pairs[s_pair];
+                    const int tx = s_local % P.tiles_x, ty = s_local / P.tiles_x;
+                    if (border_dirty<SINGLE>(P, tx, ty)) {
+                        const Region g = make_region(P, 0, 0, P.tile_w, P.tile_h, 0);
+                        pkey_t *K = reinterpret_cast<pkey_t *>(smem);
+                        unsigned *h = reinterpret_cast<unsigned *>(smem + sizeof(pkey_t) * g.RH * g.P);
+                        const int r = solve_again<SINGLE>(P, tx, ty, K, h, st, pass + 1, stage, tma);
+                        if (r < 0) return;
+                        if (r > 0) queue_neighbours(a, st, s_pair, tx, ty, pass + 1);
+                        if (threadIdx.x == 0) atomicAdd(cnt, 1u);
+                    }
+                }
             }
-            __syncthreads();
         }
         if (!grid_sync(st, nblocks)) return;
         const unsigned dirty = ld_acquire(cnt);
@@ -481,6 +624,7 @@ __global__ void __launch_bounds__(DT_THREADS) dt_kernel(const BatchArgs *__restr
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             st->changed[(pass + 2) % 3] = 0;
             st->work[(pass + 2) % 3] = 0;
+            st->wl_count[(pass + 2) % 3] = 0;
         }
         if (dirty == 0) {
             if (blockIdx.x == 0 && threadIdx.x == 0) st->passes = pass + 1;
@@ -523,9 +667,9 @@ size_t dt_smem_bytes(int tile_w, int tile_h, int apron) {
 
 cudaError_t launch_dt(const BatchArgs &a, const BatchArgs *dev, const LaunchCfg &lc,
                       int max_tile_w, int max_tile_h, int max_apron, bool fixed_grid,
-                      int *grid_used) {
+                      int *grid_used, bool single) {
     size_t smem = dt_smem_bytes(max_tile_w, max_tile_h, max_apron);
-    void (*kernel)(const BatchArgs *) = dt_kernel;
+    void (*kernel)(const BatchArgs *) = single ? dt_kernel<true> : dt_kernel<false>;
     cudaError_t e = cudaFuncSetAttribute(
         kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

@@ -14,10 +14,15 @@
 //                  path to a pixel within its cap is within its own, and the
 //                  capped distances are exact.  Pixels that can matter beyond
 //                  a tile's 32-bit window are solved in further windows; what
-//                  lies beyond 32 bits or MAX_WINDOWS with 64-bit keys
-//                  (relax_settle.cuh).  The tiles that a match reaches (13 of
+//                  lies beyond 32 bits or MAX_WINDOWS, and every tile where the
+//                  caps reach far (single_far in epic_internal.cuh), with 64-bit
+//                  keys (relax_settle.cuh).  The tiles that a match reaches (13 of
 //                  224 on a 1024 x 436 frame with 5000 matches and K = 100)
 //                  are written out as float32 distance tiles.
+//   cap_sum_kernel how far the caps reach.
+//   map_tiles_kernel
+//                  the distance tiles of matches that were relaxed by pairs (few
+//                  matches, see epic_internal.cuh).
 //   start_kernel,  the distance tiles by image tile, for the per-pixel fit.
 //   list_kernel
 //
@@ -281,25 +286,26 @@ __device__ bool next_window(const PoolMap &map, const TileGeo &g, DistTile<SR> &
 // place of the nearest distance that can improve one of their pixels, 2^32 - 1
 // for nothing (nothing within the cap changed; the match's first solve offers
 // in any case, its seed is in the map already).  A window beyond `limit`, the
-// first place in the queue, or beyond an offer waits: sh.offer[8].
+// first place in the queue, or beyond an offer waits: sh.offer[8].  far: with
+// 64-bit keys at once.
 __device__ void solve_single(const PairDev &P, const PoolMap &map, const pkey_t *cap, int tx, int ty, SingleShared &sh,
-                             RunState *st, bool first, unsigned limit) {
+                             RunState *st, bool first, unsigned limit, bool far) {
     const int tid = threadIdx.x, bx = tid & 15, by = tid >> 4;
     const int b = (by + 1) * RT_BX + bx + 1;
     const TileGeo g = tile_geo(P, tx, ty);
     pkey_t *mine = map.own + 4 * by * SINGLE_W + 4 * bx;
     const int nrow = min(4, g.rv - 4 * by), ncol = min(4, g.wv - 4 * bx);
-    bool wide = false;
+    bool wide = far;
     fetch_caps(cap, P, g, nrow, ncol, sh.cap);
     RingState R;
-    load_ring(P, map, cap, g, R);
+    if (!far) load_ring(P, map, cap, g, R);
     if (tid < 9) sh.offer[tid] = 0xFFFFFFFFu;   // (barriers follow)
     auto offer = [&](unsigned f, unsigned at) {
 #pragma unroll
         for (int k = 0; k < 8; ++k)
             if ((f >> k) & 1u) atomicMin(&sh.offer[k], at);
     };
-    {
+    if (!far) {
         DistTile<SR> &T = sh.dist;
         DistBlock B;
         Staged S;
@@ -382,6 +388,8 @@ __device__ void solve_single(const PairDev &P, const PoolMap &map, const pkey_t 
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const int i = 4 * r + c;
+                // (the seed, where no window has offered it yet)
+                if (far && first && r < nrow && c < ncol && key_dunits(B.k[r][c]) == 0) keep |= 1u << i;
                 if (!((changed >> i) & 1u) || r >= nrow || c >= ncol) continue;
                 if (key_reached(B.k[r][c]) && key_dunits(B.k[r][c]) <= v[r][c]) mask |= 1u << c;
                 else B.k[r][c] = KEY_INF;
@@ -402,16 +410,19 @@ __device__ void solve_single(const PairDev &P, const PoolMap &map, const pkey_t 
     __syncthreads();
 }
 
-// Write the reached pixels of tile t out as a distance tile of match m.
-__device__ void put_tile(const SingleArgs &x, const PairDev &P, const pkey_t *own, int t, int m, int *shared_slot) {
+// Write the reached pixels of a tile, whose keys start at `keys` with `pitch` a
+// row, out as a distance tile of match m.
+__device__ void put_tile(const SingleArgs &x, int tile, const pkey_t *keys, int pitch, bool vec, int m,
+                         int *shared_slot) {
     const int tid = threadIdx.x, bx = tid & 15, by = tid >> 4;
-    const TileGeo g = tile_geo(P, t % P.tiles_x, t / P.tiles_x);
-    const int nrow = min(4, g.rv - 4 * by), ncol = min(4, g.wv - 4 * bx);
+    const int rv = min(SINGLE_H, x.H - tile / x.tiles_x * SINGLE_H);
+    const int wv = min(SINGLE_W, x.W - tile % x.tiles_x * SINGLE_W);
+    const int nrow = min(4, rv - 4 * by), ncol = min(4, wv - 4 * bx);
     pkey_t k[4][4];
     bool any = false;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-        load_keys(own, (size_t)(4 * by + r) * SINGLE_W + 4 * bx, r < nrow ? ncol : 0, true, k[r]);
+        load_keys(keys, (size_t)(4 * by + r) * pitch + 4 * bx, r < nrow ? ncol : 0, vec, k[r]);
 #pragma unroll
         for (int c = 0; c < 4; ++c) any |= key_reached(k[r][c]);
     }
@@ -420,8 +431,8 @@ __device__ void put_tile(const SingleArgs &x, const PairDev &P, const pkey_t *ow
         const unsigned s = atomicAdd(x.used, 1u);
         *shared_slot = s < x.slot_cap ? (int)s : -1;
         if (s < x.slot_cap) {
-            x.slot_of[s] = make_int2(t, m);
-            atomicAdd(x.tile_count + t, 1);
+            x.slot_of[s] = make_int2(tile, m);
+            atomicAdd(x.tile_count + tile, 1);
         }
     }
     __syncthreads();
@@ -434,9 +445,35 @@ __device__ void put_tile(const SingleArgs &x, const PairDev &P, const pkey_t *ow
     __syncthreads();
 }
 
+// A CTA takes tile blockIdx.x of match m0 + blockIdx.y.
+__global__ void __launch_bounds__(ST) map_tiles_kernel(SingleArgs x, const pkey_t *maps, int m0) {
+    __shared__ int s_slot;
+    const int tile = blockIdx.x;
+    const size_t P = (size_t)x.H * x.W;
+    const size_t at = blockIdx.y * P + (size_t)(tile / x.tiles_x * SINGLE_H) * x.W + tile % x.tiles_x * SINGLE_W;
+    put_tile(x, tile, maps + at, x.W, (x.W & 1) == 0, m0 + (int)blockIdx.y, &s_slot);
+}
+
+// The sum of the distances of a map, in cost units (unreached: 1024).
+__global__ void __launch_bounds__(256) cap_sum_kernel(const pkey_t *cap, long long n, float *sum) {
+    float v = 0.f;
+    for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += gridDim.x * 256LL)
+        v += fminf(key_dist(cap[i]), 1024.f);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    __shared__ float s_part[8];
+    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) v += s_part[w];
+        atomicAdd(sum, v);
+    }
+}
+
 __global__ void __launch_bounds__(ST, 384 / ST) single_kernel(SingleArgs x) {
     RunState *st = x.state;
-    if (get_status(st) != 0) return;
+    const bool far = *x.cap_sum > x.cap_limit;
+    if (get_status(st) != 0 || (far && x.far_returns)) return;
     __shared__ SingleShared sh;
     __shared__ PairDev P;
     __shared__ int s_item, s_queued, s_touched, s_slot, s_seed, s_fresh;
@@ -547,7 +584,7 @@ __global__ void __launch_bounds__(ST, 384 / ST) single_kernel(SingleArgs x) {
                 if (solves == 0 && tid == 0) map.own[s_seed] = make_key(0ull, LABEL_NONE);
                 __syncthreads();
             }
-            solve_single(P, map, x.cap, tx, ty, sh, st, solves == 0, s_limit);
+            solve_single(P, map, x.cap, tx, ty, sh, st, solves == 0, s_limit, far);
             if (tid < 9 && sh.offer[tid] != 0xFFFFFFFFu) {
                 const int nx = tid == 8 ? tx : tx + (tid < 3 ? tid - 1 : tid < 5 ? 2 * tid - 7 : tid - 6);
                 const int ny = tid == 8 ? ty : ty + (tid < 3 ? -1 : tid < 5 ? 0 : 1);
@@ -568,7 +605,7 @@ __global__ void __launch_bounds__(ST, 384 / ST) single_kernel(SingleArgs x) {
         const int n = s_touched;
         if (whole) {
             for (int i = 0; i < n; ++i)
-                put_tile(x, P, map.pool + (size_t)i * SINGLE_TILE, touched[i], m, &s_slot);
+                put_tile(x, touched[i], map.pool + (size_t)i * SINGLE_TILE, SINGLE_W, true, m, &s_slot);
         } else if (tid == 0) {
             x.left[atomicAdd(x.left_count, 1u)] = m;
             flags[-2 - s_item] = 0;
@@ -640,6 +677,23 @@ int single_resident(int num_sms) {
 
 cudaError_t launch_single(const SingleArgs &x, int ctas, cudaStream_t stream) {
     single_kernel<<<ctas, ST, 0, stream>>>(x);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cap_sum(const pkey_t *cap, long long n, float *sum, cudaStream_t stream) {
+    const cudaError_t e = cudaMemsetAsync(sum, 0, sizeof(float), stream);
+    if (e != cudaSuccess) return e;
+    const long long blocks = (n + 1023) / 1024;
+    cap_sum_kernel<<<(unsigned)(blocks < 1024 ? blocks : 1024), 256, 0, stream>>>(cap, n, sum);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_map_tiles(const SingleArgs &x, const pkey_t *maps, int m0, int n, cudaStream_t stream) {
+    const size_t P = (size_t)x.H * x.W;
+    for (int j = 0; j < n; j += 65535) {   // (the grid's rows)
+        const dim3 grid((unsigned)(x.tiles_x * x.tiles_y), (unsigned)(n - j < 65535 ? n - j : 65535));
+        map_tiles_kernel<<<grid, ST, 0, stream>>>(x, maps + j * P, m0 + j);
+    }
     return cudaGetLastError();
 }
 
