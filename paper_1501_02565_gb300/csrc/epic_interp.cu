@@ -1261,8 +1261,7 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
         x.cell_start = start;
         x.cell_match = match;
         x.weights = weights;
-        if ((e = cudaMemsetAsync(x.slow_count, 0, sizeof(int), stream)) ||
-            (e = epic::launch_exact_euclidean(x, start, match, weights, cells, h->num_sms, stream)))
+        if ((e = epic::launch_exact_euclidean(x, start, match, weights, cells, h->num_sms, stream)))
             return cuda_fail(h, e, "exact-variant fit");
         h->last_stream = stream;
         return epic_interp_sync(h);
@@ -1570,7 +1569,6 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
     x.tile_entry = s.tile_entry;
     x.slots = s.slots;
     if ((e = epic::launch_single_lists(s, n_used, stream)) ||
-        (e = cudaMemsetAsync(x.slow_count, 0, sizeof(int), stream)) ||
         (e = epic::launch_exact_geodesic(x, h->num_sms, stream)))
         return cuda_fail(h, e, "exact-variant fit");
     h->last_stream = stream;

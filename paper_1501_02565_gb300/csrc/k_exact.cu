@@ -19,8 +19,8 @@
 //                      degenerate or requested) and writes the model's value
 //                      at the pixel.
 //   scan_kernel        groups with more candidates than fit in shared memory
-//                      (rare: dense clusters): every candidate in index
-//                      order, into 64-bit keys.
+//                      (dense clusters), or all groups (scan_all): every
+//                      candidate in index order, into 64-bit keys.
 //
 // 1024 x 436 pixels, 5000 matches, K = 100: 1.83 ms (Euclidean) and 4.9 + 1.3
 // ms (geodesic; the second for the groups left to scan_kernel), against 28.0
@@ -202,6 +202,25 @@ __device__ void sort_keys(unsigned long long *key, int n) {
         }
 }
 
+// Euclidean: the radius around a group's centre in which candidates are first
+// looked for: the K-th distance at the mean density, and some.
+__host__ __device__ __forceinline__ float first_radius(const ExactArgs &x) {
+    return 1.25f * sqrtf((float)x.K * (float)x.W * (float)x.H / (3.1416f * (float)x.N)) + 2.f * GROUP_RADIUS + 4.f;
+}
+// Whether all groups are scanned: so few matches that gathering and sorting them
+// costs more (1024 x 436: one match 105 us scanned and 138 by groups, 33 of K = 10
+// 451 and 488, 48 of K = 10 449 and 452, 64 of K = 64 2.5 and 3.1 ms, 100 of K =
+// 100 4.7 and 4.6 ms), or so many that at the mean density a group needs more
+// than shared memory holds (128 x 128, a match per pixel, K = 32: 4.5 ms, and 4.6
+// with the look at the groups before it).
+constexpr int SCAN_FEW = 24, SCAN_MOST = 80;
+bool scan_all(const ExactArgs &x) {
+    if (x.N <= SCAN_MOST && x.N <= SCAN_FEW + x.K) return true;
+    const float per = (float)x.N / ((float)x.W * (float)x.H);
+    const float need = sqrtf((float)x.K / (3.1416f * per)) + 2.f * GROUP_RADIUS;
+    return x.N > CAND && 3.1416f * need * need * per > 1.1f * (float)CAND;
+}
+
 template <bool GEO>
 __global__ void __launch_bounds__(EXACT_THREADS) fit_kernel(ExactArgs x, int groups_x) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -225,9 +244,8 @@ __global__ void __launch_bounds__(EXACT_THREADS) fit_kernel(ExactArgs x, int gro
     // ---- candidates, by their distance from the centre
     if constexpr (!GEO) {
         const float all = (float)(W + H);   // from here on every cell is looked at
-        // the K-th distance at the mean density, and some
-        float S = fminf(all, 1.25f * sqrtf((float)K * (float)W * (float)H / (3.1416f * (float)x.N)) +
-                                 2.f * GROUP_RADIUS + 4.f);
+        float S = fminf(all, first_radius(x));
+        bool narrowed = false;
         for (int round = 0; round < 64; ++round) {
             if (t == 0) s_n = 0;
             __syncthreads();
@@ -255,8 +273,16 @@ __global__ void __launch_bounds__(EXACT_THREADS) fit_kernel(ExactArgs x, int gro
             n = s_n;
             __syncthreads();
             if (n > CAND) {
-                fits = false;
-                break;
+                // the first look may take in more than is needed: once, look
+                // at a part of it (1024 x 436, a match for four pixels, K =
+                // 100: 3.8 ms; 326 ms when such groups were left to the scan)
+                if (narrowed) {
+                    fits = false;
+                    break;
+                }
+                narrowed = true;
+                S *= sqrtf(0.9f * (float)CAND / (float)n);
+                continue;
             }
             if (n < K && !every) {   // (K <= N; fewer may be at a finite distance)
                 S = fminf(all, 1.5f * S);
@@ -453,41 +479,54 @@ __global__ void __launch_bounds__(EXACT_THREADS) fit_kernel(ExactArgs x, int gro
         }
 }
 
-// The groups that fit_kernel left: every candidate in index order, a thread a
-// pixel, sorted insertion of 64-bit keys (distance, index).
+// The groups that fit_kernel left, or all of them: every candidate in index
+// order, a thread a pixel, sorted insertion of 64-bit keys (distance, index).
 template <bool GEO>
-__global__ void __launch_bounds__(EXACT_THREADS) scan_kernel(ExactArgs x, int groups_x) {
+__global__ void __launch_bounds__(EXACT_THREADS) scan_kernel(ExactArgs x, int groups_x, int all) {
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned long long *list = reinterpret_cast<unsigned long long *>(smem);
     const int T = EXACT_THREADS, t = threadIdx.x, K = x.K;
-    const int count = *(volatile const int *)x.slow_count;
+    const int count = all ? all : *(volatile const int *)x.slow_count;
     for (int g = blockIdx.x; g < count; g += gridDim.x) {
-        const int grp = x.slow_list[g];
+        const int grp = all ? g : x.slow_list[g];
         const int gx = grp % groups_x * GROUP, gy = grp / groups_x * GROUP;
         const int px = gx + (t & 7), py = gy + (t >> 3);
         if (px >= x.W || py >= x.H) continue;
         const int tile = GEO ? (gy / 32) * x.tiles_x + gx / 64 : 0;
         const int e0 = GEO ? x.tile_start[tile] : 0, e1 = GEO ? x.tile_start[tile + 1] : x.N;
         int cnt = 0;
-        for (int e = e0; e < e1; ++e) {
-            int m = e;
-            float d;
-            if (GEO) {
-                const int2 ent = __ldg(x.tile_entry + e);
-                m = ent.x;
-                d = __ldg(x.slots + (size_t)ent.y * SINGLE_TILE + (py & 31) * 64 + (px & 63));
-            } else {
-                const float4 q = __ldg(x.matches + m);
-                d = __fsqrt_rn(dist2((float)px, (float)py, source(q.x), source(q.y)));
+        // (SCAN distances at a time, for their loads to overlap)
+        constexpr int SCAN = 8;
+        for (int b = e0; b < e1; b += SCAN) {
+            float dg[SCAN];
+            int mg[SCAN];
+#pragma unroll
+            for (int u = 0; u < SCAN; ++u) {
+                const int e = b + u;
+                dg[u] = inf();
+                mg[u] = e;
+                if (e >= e1) continue;
+                if (GEO) {
+                    const int2 ent = __ldg(x.tile_entry + e);
+                    mg[u] = ent.x;
+                    dg[u] = __ldg(x.slots + (size_t)ent.y * SINGLE_TILE + (py & 31) * 64 + (px & 63));
+                } else {
+                    const float4 q = __ldg(x.matches + e);
+                    dg[u] = __fsqrt_rn(dist2((float)px, (float)py, source(q.x), source(q.y)));
+                }
             }
-            if (!(d < inf())) continue;
-            const unsigned long long key = ((unsigned long long)__float_as_uint(d) << 32) | (unsigned)m;
-            int j;
-            if (cnt < K) j = cnt++;
-            else if (key < list[(K - 1) * T + t]) j = K - 1;
-            else continue;
-            for (; j > 0 && list[(j - 1) * T + t] > key; --j) list[j * T + t] = list[(j - 1) * T + t];
-            list[j * T + t] = key;
+#pragma unroll
+            for (int u = 0; u < SCAN; ++u) {
+                const float d = dg[u];
+                if (!(d < inf())) continue;
+                const unsigned long long key = ((unsigned long long)__float_as_uint(d) << 32) | (unsigned)mg[u];
+                int j;
+                if (cnt < K) j = cnt++;
+                else if (key < list[(K - 1) * T + t]) j = K - 1;
+                else continue;
+                for (; j > 0 && list[(j - 1) * T + t] > key; --j) list[j * T + t] = list[(j - 1) * T + t];
+                list[j * T + t] = key;
+            }
         }
         const long long p = (long long)py * x.W + px;
         Sums s;
@@ -553,10 +592,15 @@ cudaError_t fit_launch(const ExactArgs &x, int num_sms, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     const int groups_x = (x.W + GROUP - 1) / GROUP;
     const long long groups = exact_groups(x.H, x.W);
+    if (!GEO && scan_all(x)) {
+        scan_kernel<GEO><<<(unsigned)groups, EXACT_THREADS, slow, stream>>>(x, groups_x, (int)groups);
+        return cudaGetLastError();
+    }
+    if ((e = cudaMemsetAsync(x.slow_count, 0, sizeof(int), stream)) != cudaSuccess) return e;
     fit_kernel<GEO><<<(unsigned)groups, EXACT_THREADS, smem, stream>>>(x, groups_x);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int blocks = (int)(groups < 4LL * num_sms ? groups : 4LL * num_sms);
-    scan_kernel<GEO><<<blocks, EXACT_THREADS, slow, stream>>>(x, groups_x);
+    scan_kernel<GEO><<<blocks, EXACT_THREADS, slow, stream>>>(x, groups_x, 0);
     return cudaGetLastError();
 }
 
@@ -588,9 +632,11 @@ cudaError_t launch_cap_seed(const float *knn_dist, const int *knn_count, int N, 
 
 cudaError_t launch_exact_euclidean(const ExactArgs &x, int *cell_start, int *cell_match, double *weights,
                                    int cells, int num_sms, cudaStream_t stream) {
-    bin_kernel<<<1, BIN_THREADS, 0, stream>>>(x.matches, x.N, x.W, x.H, x.cell_shift, x.cells_x, cells,
-                                              cell_start, cell_match);
-    weight_kernel<<<(EXACT_WEIGHTS + 255) / 256, 256, 0, stream>>>(x.a, weights);
+    if (!scan_all(x)) {
+        bin_kernel<<<1, BIN_THREADS, 0, stream>>>(x.matches, x.N, x.W, x.H, x.cell_shift, x.cells_x, cells,
+                                                  cell_start, cell_match);
+        weight_kernel<<<(EXACT_WEIGHTS + 255) / 256, 256, 0, stream>>>(x.a, weights);
+    }
     const cudaError_t e = cudaGetLastError();
     return e ? e : fit_launch<false>(x, num_sms, stream);
 }
