@@ -51,6 +51,10 @@
 // twice in the last steps and the owner searched by shuffles 5.74 ms and 314
 // us.  Rows held beside the settled list instead of in it cost 128 bytes a warp
 // and with them table space: 5.57 ms and a quarter more for the second launch.
+// A batch of one is found and settled in one look at the frontier, which is not
+// compacted for it: with the second launch 5.57 -> 5.20 ms for the batch (a
+// batch cut to one key ends many searches), 1024 x 436 with half its costs zero,
+// 1200 matches, K = 100, 11.0 -> 7.5 ms and less.
 //
 // The fit uses centred coordinates x~ = p_n - p_m and fits the flow
 // u = p' - p (the same least-squares problem as fitting p', Eq. 2, with
@@ -248,38 +252,26 @@ __global__ void __launch_bounds__(KNN_WARPS * 32, 4)
             if (kd == EMPTY32) break;  // component exhausted
             rk = EMPTY32;
             rb = __int_as_float(0x7f800000);
-            // the smallest key's node, where it counts: when no entry is below
-            // the bound, and for a batch cut to one key
-            auto smallest_node = [&]() {
-                unsigned n = EMPTY32;
-                for (int i = lane; i < fn; i += 32) {
-                    const FEnt f = fe[i];
-                    if (f.t == kd && hv[f.sl] == dist_word(kd)) n = min(n, hk[f.sl]);
-                }
-                return __reduce_min_sync(0xffffffffu, n);
-            };
-            const bool below = __uint_as_float(kd) < bound;
-            unsigned kn = below ? EMPTY32 : smallest_node();
-            // (2) the batch: current entries below the bound (and the
-            //     smallest).  A batch that reaches K is finished by sorting it
-            //     in lanes; one reaching K with more than a warp of entries is
-            //     cut to the smallest key alone.
-            // (fn counts every frontier entry, an upper bound on the batch:
-            // while cnt + fn < K the batch cannot reach K and is not counted)
             auto load = [&](int i, FEnt &f) {   // whether entry i is current
                 f = FEnt{EMPTY32, 0u, 0.f, 0u};
                 if (i < fn) f = fe[i];
                 return i < fn && hv[f.sl] == dist_word(f.t);
             };
-            auto in_batch = [&](const FEnt &f) {
-                return __uint_as_float(f.t) < bound || (!below && f.t == kd && hk[f.sl] == kn);
-            };
             // (the frontier is 35 entries on average: up to 64 stay in registers
-            // for both passes)
+            // for all looks at them)
             FEnt f0, f1;
             const bool v0 = load(lane, f0), v1 = fn > 32 && load(lane + 32, f1);
-            int nwin = 0;
-            if (cnt + fn >= K) {
+            // (2) the batch: current entries below the bound.  A batch that reaches
+            //     K is finished by sorting it in lanes.  One reaching K with more
+            //     than a warp of entries is cut to the smallest key alone, and
+            //     where no entry is below the bound (every step, among edges of
+            //     weight zero) the smallest key is the batch.
+            // (fn counts every frontier entry, an upper bound on the batch:
+            // while cnt + fn < K the batch cannot reach K and is not counted)
+            auto in_batch = [&](const FEnt &f) { return __uint_as_float(f.t) < bound; };
+            bool one = !(__uint_as_float(kd) < bound);
+            int nwin = 1;
+            if (!one && cnt + fn >= K) {
                 nwin = __popc(__ballot_sync(0xffffffffu, v0 && in_batch(f0)));
                 if (fn > 32) nwin += __popc(__ballot_sync(0xffffffffu, v1 && in_batch(f1)));
                 for (int b0 = 64; b0 < fn; b0 += 32) {
@@ -287,24 +279,66 @@ __global__ void __launch_bounds__(KNN_WARPS * 32, 4)
                     const bool v = load(b0 + lane, f);
                     nwin += __popc(__ballot_sync(0xffffffffu, v && in_batch(f)));
                 }
+                one = cnt + nwin >= K && nwin > 32;
             }
-            const bool final_batch = cnt + nwin >= K && nwin <= 32;
-            const bool single = cnt + nwin >= K && nwin > 32;
-            if (single && below) kn = smallest_node();
-            // (3) partition: kept entries are compacted to the front (writes
-            //     never pass reads); batch entries are settled into the list
-            //     or, for the final batch, handed to lanes
+            const bool final_batch = !one && cnt + nwin >= K;
+            // (3) batch entries are settled into the list or, for the final
+            //     batch, handed to lanes.  The others are compacted to the front
+            //     (writes never pass reads); a batch of one leaves them where
+            //     they are, the last in place of its own.
             int wpos = 0, nb = 0;
             pkey_t bk = EMPTY64;
+            auto keep_on = [&](unsigned t, float tw) {
+                rk = min(rk, t);
+                rb = fminf(rb, tw);
+            };
+            auto smallest = [&]() {
+                unsigned n = EMPTY32, sl = 0u, row = 0u;   // this lane's smallest key
+                float tw = 0.f;
+                int at = 0;
+                auto look = [&](const FEnt &f, bool valid, int i) {
+                    if (!valid) return;
+                    const unsigned node = f.t == kd ? hk[f.sl] : EMPTY32;
+                    if (node >= n) {
+                        keep_on(f.t, f.tw);
+                        return;
+                    }
+                    if (n != EMPTY32) keep_on(kd, tw);
+                    n = node;
+                    sl = f.sl;
+                    row = f.row;
+                    tw = f.tw;
+                    at = i;
+                };
+                look(f0, v0, lane);
+                look(f1, v1, lane + 32);
+                for (int i = lane + 64; i < fn; i += 32) {
+                    FEnt f;
+                    const bool v = load(i, f);
+                    look(f, v, i);
+                }
+                const unsigned kn = __reduce_min_sync(0xffffffffu, n);
+                --fn;
+                if (n == kn && n != EMPTY32) {   // (a node has one current entry)
+                    fe[at] = fe[fn];
+                    hv[sl] = SETTLED;
+                    rn[cnt] = row;   // (node and batch start follow)
+                    rd[cnt] = __uint_as_float(kd);
+                    bs[cnt] = (unsigned short)sl;
+                } else if (n != EMPTY32) {
+                    keep_on(kd, tw);
+                }
+                nb = 1;
+                __syncwarp();
+            };
             auto part = [&](const FEnt &f, bool valid) {
-                const bool inb = valid && (single ? f.t == kd && hk[f.sl] == kn : in_batch(f));
+                const bool inb = valid && in_batch(f);
                 const bool keep = valid && !inb;
                 const unsigned kb = __ballot_sync(0xffffffffu, keep);
                 const unsigned bb = __ballot_sync(0xffffffffu, inb);
                 if (keep) {
                     fe[wpos + __popc(kb & lt_mask)] = f;
-                    rk = min(rk, f.t);
-                    rb = fminf(rb, f.tw);
+                    keep_on(f.t, f.tw);
                 }
                 if (final_batch) {
                     const pkey_t k = inb ? ((pkey_t)f.t << 32) | hk[f.sl] : EMPTY64;
@@ -330,15 +364,19 @@ __global__ void __launch_bounds__(KNN_WARPS * 32, 4)
                 __syncwarp();
             };
             __syncwarp();
-            part(f0, v0);
-            if (fn > 32) part(f1, v1);
-            for (int b0 = 64; b0 < fn; b0 += 32) {
-                FEnt f;
-                const bool v = load(b0 + lane, f);
-                __syncwarp();
-                part(f, v);
+            if (one) {
+                smallest();
+            } else {
+                part(f0, v0);
+                if (fn > 32) part(f1, v1);
+                for (int b0 = 64; b0 < fn; b0 += 32) {
+                    FEnt f;
+                    const bool v = load(b0 + lane, f);
+                    __syncwarp();
+                    part(f, v);
+                }
+                fn = wpos;
             }
-            fn = wpos;
             if (final_batch) {
                 // sort the final batch by key across lanes (bitonic) and keep
                 // the smallest K - cnt
