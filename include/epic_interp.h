@@ -381,19 +381,26 @@ void epic_refine_params_default(epic_refine_params_t *p);
  * handle holds about H*W*56 bytes of scratch (grown on demand, EPIC_ERR_OOM
  * if it cannot be).  Enqueued on `stream` without waiting; one
  * refinement in flight per handle (the scratch is shared).  params NULL =
- * defaults. */
+ * defaults.  Frames that fit on the chip are refined by thread blocks that wait
+ * for one another (bounded, see epic_selftest_wait_timeout): where such a wait
+ * gives up, the refinement ends with the flow partly updated and
+ * EPIC_ERR_TIMEOUT recorded as by a run, so that epic_interp_sync returns it and
+ * runs queued on the handle before that do nothing. */
 int epic_refine(epic_interp_t *h, const float *I1, const float *I2, int H,
                 int W, int channels, float *flow,
                 const epic_refine_params_t *params, void *stream);
 
 /* Self-test of failure detection without a GPU fault.  Every device wait
- * of the library is bounded: the relaxation's grid barrier (2 s), its waits
- * for other tiles and the refinement's (1 s) and the TMA staging's mbarrier
- * wait (1 s) give up, record EPIC_ERR_TIMEOUT and let the
+ * of the library is bounded: the relaxation's grid barrier and its wait for
+ * requests (2 s), its waits for other tiles and the refinement's (1 s) and the
+ * TMA staging's mbarrier wait (1 s) give up, record EPIC_ERR_TIMEOUT and let the
  * kernel return.  This runs one of those waits with a limit of limit_ms
  * (1..10000) where the awaited event never happens: which = 0, a grid
- * barrier that expects a second CTA which does not exist; which = 1, an
- * mbarrier whose transaction is never issued.  Returns the status the wait
+ * barrier that expects a second CTA which does not exist; 1, an mbarrier whose
+ * transaction is never issued; 2, 3, the stamps of a tile's edge neighbours, of
+ * the tile and its neighbours, which nobody sets; 4, an open request that nobody
+ * answers; 5, 6, the refinement's wait for its neighbours' progress, for their
+ * updates.  Returns the status the wait
  * recorded (EPIC_ERR_TIMEOUT when the bound works) and leaves the handle and
  * the context usable.  Waits for completion. */
 int epic_selftest_wait_timeout(epic_interp_t *h, int which, int limit_ms);
@@ -401,9 +408,9 @@ int epic_selftest_wait_timeout(epic_interp_t *h, int which, int limit_ms);
 /* Device scratch one pair of H x W pixels, N matches and neighbourhood size
  * K takes in the handle's arena when it runs in a batch (its packed keys,
  * seed bins, edge table, CSR rows, models, optional K-NN lists and pruning
- * buffers, its K-NN retry-list slots and its relaxation tiles' work-queue
- * slots), in *bytes; a batch needs the sum over its pairs plus 512 bytes.  The caller's own buffers (cost map,
- * matches, flow) are not included.  Uses the configuration and tile rules of
+ * buffers, its K-NN retry-list slots and its relaxation tiles' request
+ * counts), in *bytes; a batch needs the sum over its pairs plus 512 bytes.  The
+ * caller's own buffers (cost map, matches, flow) are not included.  Uses the configuration and tile rules of
  * `h`; with h = NULL, those of *cfg and no tile rules (cfg = NULL: the
  * defaults).  A host computation: needs no device and enqueues nothing.
  * EPIC_ERR_INVALID for sizes that epic_interp_run would refuse. */

@@ -486,7 +486,10 @@ cudaError_t launch_cap_sum(const pkey_t *cap, long long n, float *sum, cudaStrea
 cudaError_t launch_map_tiles(const SingleArgs &x, const pkey_t *maps, int m0, int n, cudaStream_t stream);
 cudaError_t launch_single_lists(const SingleArgs &x, unsigned used, cudaStream_t stream);
 
-// Self-test of the bounded device waits (grid barrier, TMA mbarrier).
+// Self-test of the bounded device waits: grid barrier (which = 0), TMA mbarrier
+// (1); the relaxation's (2 to 4); the refinement's (5, 6).
+cudaError_t launch_relax_wait_selftest(RunState *st, int which, unsigned long long limit_ns, cudaStream_t stream);
+cudaError_t launch_refine_wait_selftest(RunState *st, int which, unsigned long long limit_ns, cudaStream_t stream);
 cudaError_t launch_wait_selftest(RunState *st, int which, unsigned long long limit_ns,
                                  cudaStream_t stream);
 

@@ -217,13 +217,14 @@ struct SorCell {
     float du, dv;
 };
 
-// Whether a wait is to end: after SOR_WAIT_NS from its first call (*t0 = 0), or
-// when another CTA has given up.
-__device__ __noinline__ bool sor_gives_up(unsigned long long *t0, unsigned *error, RunState *st) {
+// Whether a wait is to end: `limit` ns after its first call (*t0 = 0), or when
+// another CTA has given up.
+__device__ __noinline__ bool sor_gives_up(unsigned long long *t0, unsigned *error, RunState *st,
+                                          unsigned long long limit) {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     if (*t0 == 0) *t0 = t;
-    if (t - *t0 <= SOR_WAIT_NS && *(volatile unsigned *)error == 0u) return false;
+    if (t - *t0 <= limit && *(volatile unsigned *)error == 0u) return false;
     atomicExch(error, 1u);
     set_status(st, EPIC_ERR_TIMEOUT);
     return true;
@@ -231,7 +232,8 @@ __device__ __noinline__ bool sor_gives_up(unsigned long long *t0, unsigned *erro
 
 // Waits until the neighbouring tiles' progress is `want` at least (false in
 // every thread: gave up).
-__device__ bool sor_wait(const SorGrid &g, unsigned *progress, unsigned want, RunState *st) {
+__device__ bool sor_wait(const SorGrid &g, unsigned *progress, unsigned want, RunState *st,
+                         unsigned long long limit = SOR_WAIT_NS) {
     const int k = threadIdx.x;
     bool failed = false;
     if (k < 8) {
@@ -240,7 +242,7 @@ __device__ bool sor_wait(const SorGrid &g, unsigned *progress, unsigned want, Ru
         if (x >= 0 && x < g.tiles_x && y >= 0 && y < g.tiles_y) {
             unsigned long long t0 = 0;
             for (int n = 1; ld_acquire(progress + y * g.tiles_x + x) < want; ++n)
-                if ((n & 63) == 0 && sor_gives_up(&t0, progress + g.tiles_x * g.tiles_y, st)) {
+                if ((n & 63) == 0 && sor_gives_up(&t0, progress + g.tiles_x * g.tiles_y, st, limit)) {
                     failed = true;
                     break;
                 }
@@ -259,6 +261,16 @@ __device__ __forceinline__ void put_tagged(ulonglong2 *p, float du, float dv, un
 }
 __device__ __forceinline__ void get_tagged(const ulonglong2 *p, ulonglong2 *v) {
     asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v->x), "=l"(v->y) : "l"(p) : "memory");
+}
+// Reads *p into *v until it carries the tag (false: gave up).
+__device__ __forceinline__ bool await_tagged(const ulonglong2 *p, unsigned tag, ulonglong2 *v, unsigned *error,
+                                             RunState *st, unsigned long long limit = SOR_WAIT_NS) {
+    unsigned long long t0 = 0;
+    for (int m = 1; (unsigned)(v->x >> 32) != tag || (unsigned)(v->y >> 32) != tag; ++m) {
+        if ((m & 63) == 0 && sor_gives_up(&t0, error, st, limit)) return false;
+        get_tagged(p, v);
+    }
+    return true;
 }
 
 // This CTA's writes, by every thread, are done up to step `step`.
@@ -462,14 +474,7 @@ __global__ void __launch_bounds__(SOR_THREADS, SOR_PER_SM)
 #pragma unroll
             for (int k = 0; k < BATCH; ++k) {
                 if (to[k] < 0) continue;
-                unsigned long long t0 = 0;
-                for (int m = 1; (unsigned)(v[k].x >> 32) != tag || (unsigned)(v[k].y >> 32) != tag; ++m) {
-                    if ((m & 63) == 0 && sor_gives_up(&t0, x.progress + g.tiles_x * g.tiles_y, st)) {
-                        failed = true;
-                        break;
-                    }
-                    get_tagged(buf + from[k], &v[k]);
-                }
+                if (!await_tagged(buf + from[k], tag, &v[k], x.progress + g.tiles_x * g.tiles_y, st)) failed = true;
                 const float2 d = make_float2(__uint_as_float((unsigned)v[k].x), __uint_as_float((unsigned)v[k].y));
                 const int q = to[k] & 1, e = to[k] >> 1;
                 const float4 o = sh.own[q][e];
@@ -496,6 +501,23 @@ __global__ void __launch_bounds__(SOR_THREADS, SOR_PER_SM)
             else dout[p] = make_float2(cell[q][j].du, cell[q][j].dv);
         });
         if (ROUNDS && it + 1 < iterations) sor_post(x.progress, 3u * it + 3u);
+    }
+}
+
+// Self-test of this kernel's waits (see epic_selftest_wait_timeout): nobody makes
+// progress and nobody sends an update.
+__device__ unsigned selftest_progress[3];
+__device__ ulonglong2 selftest_update;
+__global__ void refine_wait_selftest_kernel(RunState *st, int which, unsigned long long limit_ns) {
+    if (threadIdx.x < 3) selftest_progress[threadIdx.x] = 0;
+    __threadfence();
+    __syncthreads();
+    if (which == 5) {
+        sor_wait(SorGrid{8, 8, 2, 1, 10, 20}, selftest_progress, 1u, st, limit_ns);
+    } else if (threadIdx.x == 0) {
+        ulonglong2 v;
+        get_tagged(&selftest_update, &v);
+        await_tagged(&selftest_update, 1u, &v, selftest_progress + 2, st, limit_ns);
     }
 }
 
@@ -551,6 +573,11 @@ void launch_coeff(const float *I1, const float *I2, int H, int W, const float *f
 }
 
 }  // namespace
+
+cudaError_t launch_refine_wait_selftest(RunState *st, int which, unsigned long long limit_ns, cudaStream_t stream) {
+    refine_wait_selftest_kernel<<<1, 32, 0, stream>>>(st, which, limit_ns);
+    return cudaGetLastError();
+}
 
 size_t refine_scratch_bytes(int H, int W) {
     const size_t P = (size_t)H * W;

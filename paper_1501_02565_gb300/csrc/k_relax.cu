@@ -407,8 +407,40 @@ __global__ void __launch_bounds__(Dim<MAXR>::NT, 384 / Dim<MAXR>::NT)
     }
 }
 
+// Self-test of this kernel's waits (see epic_selftest_wait_timeout): nothing
+// stamps the tiles and nobody answers the request.
+__device__ int selftest_words[4];
+__global__ void relax_wait_selftest_kernel(RunState *st, int which, unsigned long long limit_ns) {
+    __shared__ PairDev P;
+    __shared__ OwnShared own;
+    if (threadIdx.x == 0) {
+        P.tiles_x = 2;   // two tiles side by side
+        P.tiles_y = P.stack = 1;
+        P.tile_stamp = selftest_words;
+        selftest_words[0] = selftest_words[1] = STAMP_PENDING;
+        selftest_words[2] = 0;   // requests of the one tile below
+        st->tiles[0].open = 1;
+    }
+    __threadfence();
+    __syncthreads();
+    if (which == 2) {
+        wait_edge_neighbours(P, 0, 0, st, limit_ns);
+    } else if (which == 3) {
+        wait_tile_and_ring(P, 0, 0, st, limit_ns);
+    } else {
+        BatchArgs a{};
+        a.npairs = a.total_solve = a.total_tiles = a.max_passes = 1;
+        own_tiles(a, st, &st->tiles[0], reinterpret_cast<unsigned *>(selftest_words + 2), own, 1u,
+                  [](const PairDev &, int, int, int) { return 0u; }, limit_ns);
+    }
+}
 
 }  // namespace
+
+cudaError_t launch_relax_wait_selftest(RunState *st, int which, unsigned long long limit_ns, cudaStream_t stream) {
+    relax_wait_selftest_kernel<<<1, 32, 0, stream>>>(st, which, limit_ns);
+    return cudaGetLastError();
+}
 
 size_t relax_smem_bytes(int max_rows) {
     return max_rows <= 8    ? sizeof(RelaxShared<8>)

@@ -154,9 +154,10 @@ __device__ __forceinline__ unsigned long long wait_ns() {
 
 // Waits until the four edge neighbours of tile (tx, ty) (those inside the
 // tile grid) carry a stamp of this run, i.e. are written; thread k < 4
-// watches one.  Gives up after WAIT_LIMIT_NS with EPIC_ERR_TIMEOUT (false in
-// every thread).
-__device__ bool wait_edge_neighbours(const PairDev &P, int tx, int ty, RunState *st) {
+// watches one.  Gives up after `limit` ns with EPIC_ERR_TIMEOUT (false in every
+// thread).
+__device__ bool wait_edge_neighbours(const PairDev &P, int tx, int ty, RunState *st,
+                                     unsigned long long limit = WAIT_LIMIT_NS) {
     bool gave_up = false;
     const int k = threadIdx.x;
     if (k < 4) {
@@ -166,7 +167,7 @@ __device__ bool wait_edge_neighbours(const PairDev &P, int tx, int ty, RunState 
             const unsigned *sp = reinterpret_cast<const unsigned *>(P.tile_stamp + y * P.tiles_x + x);
             const unsigned long long t0 = wait_ns();
             while (ld_acquire(sp) == (unsigned)STAMP_PENDING) {
-                if (wait_ns() - t0 > WAIT_LIMIT_NS) {
+                if (wait_ns() - t0 > limit) {
                     set_status(st, EPIC_ERR_TIMEOUT);
                     gave_up = true;
                     break;
@@ -180,9 +181,10 @@ __device__ bool wait_edge_neighbours(const PairDev &P, int tx, int ty, RunState 
 
 // Waits until tile (tx, ty) and its eight neighbours (those inside the tile
 // grid) carry a stamp of this run (phase 1 has written them); thread k < 8
-// watches neighbour k, thread 8 the tile.  Gives up after WAIT_LIMIT_NS with
+// watches neighbour k, thread 8 the tile.  Gives up after `limit` ns with
 // EPIC_ERR_TIMEOUT (false in every thread).
-__device__ bool wait_tile_and_ring(const PairDev &P, int tx, int ty, RunState *st) {
+__device__ bool wait_tile_and_ring(const PairDev &P, int tx, int ty, RunState *st,
+                                   unsigned long long limit = WAIT_LIMIT_NS) {
     bool gave_up = false;
     const int k = threadIdx.x;
     if (k < 9) {
@@ -192,7 +194,7 @@ __device__ bool wait_tile_and_ring(const PairDev &P, int tx, int ty, RunState *s
             const unsigned *sp = reinterpret_cast<const unsigned *>(P.tile_stamp + y * P.tiles_x + x);
             const unsigned long long t0 = wait_ns();
             while (ld_acquire(sp) == (unsigned)STAMP_PENDING) {
-                if (wait_ns() - t0 > WAIT_LIMIT_NS) {
+                if (wait_ns() - t0 > limit) {
                     set_status(st, EPIC_ERR_TIMEOUT);
                     gave_up = true;
                     break;
@@ -224,8 +226,8 @@ constexpr unsigned long long IDLE_LIMIT_NS = 2000000000ull;  // 2 s
 // where turns take ~3.7 on a batch.)
 //
 // solve(P, lt, tx, ty) stages and solves a tile, writes its changed keys and
-// returns what it did (TB_*; 0: nothing changed), the same in every thread.  Returns false if the run has an error or nothing moved for
-// IDLE_LIMIT_NS.
+// returns what it did (TB_*; 0: nothing changed), the same in every thread.
+// Returns false if the run has an error or nothing moved for `limit` ns.
 struct OwnShared {
     unsigned count[32];   // requests of 32 owned tiles
     unsigned dirty;       // those that have any
@@ -234,7 +236,8 @@ struct OwnShared {
 
 template <typename Solve>
 __device__ bool own_tiles(const BatchArgs &a, RunState *st, TileWork *q, unsigned *req,
-                          OwnShared &S, unsigned nblocks, Solve solve) {
+                          OwnShared &S, unsigned nblocks, Solve solve,
+                          unsigned long long limit = IDLE_LIMIT_NS) {
     const unsigned Tt = (unsigned)a.total_solve;
     const unsigned mine = (Tt - blockIdx.x + nblocks - 1) / nblocks;   // tiles owned
     // solves of the whole run: a pass is two for each of its tiles (a stack
@@ -268,7 +271,7 @@ __device__ bool own_tiles(const BatchArgs &a, RunState *st, TileWork *q, unsigne
                         } else if (now != seen) {
                             seen = now;
                             t0 = wait_ns();
-                        } else if (wait_ns() - t0 > IDLE_LIMIT_NS) {
+                        } else if (wait_ns() - t0 > limit) {
                             set_status(st, EPIC_ERR_TIMEOUT);
                             S.state = -2;
                         }

@@ -401,7 +401,8 @@ class EpicInterp:
 
     def selftest_wait_timeout(self, which, limit_ms=50):
         """Status recorded by a bounded device wait that never completes
-        (0: grid barrier, 1: TMA mbarrier); EPIC_ERR_TIMEOUT expected."""
+        (0: grid barrier, 1: TMA mbarrier, 2 to 4: the relaxation's, 5 and 6:
+        the refinement's); EPIC_ERR_TIMEOUT expected."""
         return self.lib.epic_selftest_wait_timeout(self.h, int(which), int(limit_ms))
 
     def get_pruning(self, pair, N):
