@@ -21,6 +21,7 @@
 #include <type_traits>
 
 #include "epic_internal.cuh"
+#include "quotient.cuh"
 
 namespace epic {
 
@@ -199,13 +200,6 @@ struct SorShared {
     float right[2][SOR_CELLS];   // weight of the edge to the right (first: phi)
     float down[2][SOR_CELLS];    // and downwards
 };
-
-// n / det from the correctly rounded inverse of det: the quotient corrected by
-// its residual (Markstein 1990).
-__device__ __forceinline__ float quotient(float n, float det, float inv) {
-    const float q = n * inv;
-    return __fmaf_rn(__fmaf_rn(-q, det, n), inv, q);
-}
 
 struct SorGrid {
     int cw, ch, tiles_x, tiles_y;   // cores
