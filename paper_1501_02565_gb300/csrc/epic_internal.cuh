@@ -129,7 +129,7 @@ struct PairDev {
     float a;
     int tile_w, tile_h, apron;
     int sweep;              // relaxation schedule: 0 segmented lines, 1 whole lines
-                            // (k_dt.cu); 2 row-closure passes on warp tiles (k_relax.cu)
+                            // (k_dt.cu); 2 tiles solved in registers (k_relax.cu), the "warp tiles"
     int tiles_x, tiles_y;
     int stack;              // warp tiles: tiles of a column solved as one (1 or 2)
     int hash_cap;           // power of two
@@ -518,9 +518,9 @@ size_t dt_smem_bytes(int tile_w, int tile_h, int apron);
 // max_rows = the rows of the batch's largest solve tile (<= 32).
 constexpr int RELAX_TILE_W = 64;
 constexpr int RELAX_MAX_ROWS = 32;
-// Tiles are solved in stacks of two (see solve_stack in epic_interp.cu) from
-// this many on.
-constexpr int RELAX_STACK_TILES = 1400;
+// Tiles are solved in stacks of two (see solve_stack in epic_interp.cu) from so
+// many per four SMs on (1406 on 152).
+constexpr int RELAX_STACK_TILES = 37;
 size_t relax_smem_bytes(int max_rows);
 cudaError_t launch_relax(const BatchArgs &a, const BatchArgs *dev, const LaunchCfg &lc,
                          int max_rows, bool fixed_grid, int *grid_used);

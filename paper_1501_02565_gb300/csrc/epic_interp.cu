@@ -136,8 +136,10 @@ int next_pow2(long long x) {
 constexpr int SWEEP_WARP_TILES = 2;
 
 // Tile height when neither the configuration nor a rule gives one: 16 rows
-// for warp tiles (what the tile autotuner picks for frames above 64 K
-// pixels), 32 for the apron tiles.
+// for warp tiles (what the tile autotuner picked for frames above 64 K pixels
+// with the row-closure kernel; with this one it takes 32, by little on large
+// frames: relaxation of a 1024 x 436 pair 130 and 147 us), 32 for the apron
+// tiles.
 int default_tile_h(int sweep) { return sweep == SWEEP_WARP_TILES ? 16 : 32; }
 
 void choose_tiles(const epic_config_t &c, const std::vector<epic_tile_rule_t> &rules, int H,
@@ -194,9 +196,9 @@ bool uses_warp_tiles(const epic_config_t &c, const std::vector<epic_tile_rule_t>
 // two 64 x 16 tiles at a time are faster (distances and settling of a
 // 2048 x 1024 pair, 2048 tiles: 249 -> 181 us; of 8 pruned 1024 x 436 pairs,
 // 3584 tiles: 1114 -> 860 us); with fewer, one at a time spreads over more SMs
-// (912 tiles are resident at once).
-int solve_stack(long long tiles, int max_th) {
-    return tiles >= epic::RELAX_STACK_TILES && 2 * max_th <= epic::RELAX_MAX_ROWS ? 2 : 1;
+// (six tiles are resident on each).
+int solve_stack(long long tiles, int max_th, int num_sms) {
+    return 4 * tiles >= (long long)epic::RELAX_STACK_TILES * num_sms && 2 * max_th <= epic::RELAX_MAX_ROWS ? 2 : 1;
 }
 
 // Waits, on every way out of a call, for the copies from the call's own memory
@@ -644,7 +646,7 @@ int epic_interp_run_batch(epic_interp_t *h, const epic_pair_desc_t *descs, int n
         const long long cfg_tiles = (long long)std::max(1, c.max_pairs) *
                                     ((std::max(1, c.max_W) + epic::RELAX_TILE_W - 1) / epic::RELAX_TILE_W) *
                                     ((std::max(1, c.max_H) + cfg_th - 1) / cfg_th);
-        stack = graph ? solve_stack(cfg_tiles, cfg_th) : solve_stack((long long)total_T, max_th);
+        stack = graph ? solve_stack(cfg_tiles, cfg_th, h->num_sms) : solve_stack((long long)total_T, max_th, h->num_sms);
     }
 
     // batch table: BatchArgs, PairDev[n], then 6 prefix arrays of n+1 ints

@@ -94,12 +94,13 @@ __device__ __forceinline__ int find_pair_in(const int *base, int n, int i) {   /
     }
     return lo;
 }
-// Runs of fewer tiles than this take an item per tile, or parts of a tile, so
-// that every SM has items: 2048 x 1024 (2048 tiles) takes 41 us by the tile, 48
-// stacked; 1024 x 436 (448 tiles) 22 us in halves, 23.5 in quarters, 41 stacked.
-constexpr int EDGE_STACK_TILES = 2432;
-__device__ __forceinline__ int edge_split(int total_tiles) {
-    return total_tiles < 304 ? 4 : total_tiles < 1216 ? 2 : 1;
+// Runs of fewer tiles than so many per SM take an item per tile, or parts of a
+// tile, so that every SM has items: 2048 x 1024 (2048 tiles on 152 SMs) takes 41
+// us by the tile, 48 stacked; 1024 x 436 (448 tiles) 22 us in halves, 23.5 in
+// quarters, 41 stacked.
+constexpr int EDGE_STACK_TILES = 16;
+__device__ __forceinline__ int edge_split(int total_tiles, int num_sms) {
+    return total_tiles < 2 * num_sms ? 4 : total_tiles < 8 * num_sms ? 2 : 1;
 }
 
 // Lower the weight of pair k in the shared table (straight in the global table
@@ -127,7 +128,8 @@ __device__ __forceinline__ void smem_insert(const PairDev &P, pkey_t k, unsigned
     table_insert(P, k, wbits, st);
 }
 
-__global__ void __launch_bounds__(EDGE_THREADS) edges_kernel(const BatchArgs *__restrict__ ap, int parts) {
+__global__ void __launch_bounds__(EDGE_THREADS) edges_kernel(const BatchArgs *__restrict__ ap, int parts,
+                                                             int num_sms) {
     const BatchArgs a = *ap;
     RunState *st = a.state;
     if (get_status(st) != 0) return;
@@ -169,8 +171,8 @@ __global__ void __launch_bounds__(EDGE_THREADS) edges_kernel(const BatchArgs *__
         for (int i = threadIdx.x; i < a.npairs; i += EDGE_THREADS) s_base[i] = a.tile_base[i];
     __syncthreads();
     int next = threadIdx.x == 0 ? (int)atomicAdd(&st->edge_next, 1u) : 0;   // thread 0: the next item
-    const int split = max(edge_split(a.total_tiles), parts);   // (parts of tall tiles)
-    const bool stacked = parts == 1 && a.total_tiles >= EDGE_STACK_TILES;
+    const int split = max(edge_split(a.total_tiles, num_sms), parts);   // (parts of tall tiles)
+    const bool stacked = parts == 1 && a.total_tiles >= EDGE_STACK_TILES * num_sms;
     // items are handed out from a counter: their cost varies with the number
     // of cell boundaries they hold
     for (;;) {
@@ -516,7 +518,7 @@ cudaError_t launch_edges(const BatchArgs &a, const BatchArgs *dev, const LaunchC
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     edges_kernel<<<lc.num_sms * per_sm, EDGE_THREADS, smem, lc.stream>>>(
-        dev, max_tile_h > EDGE_ROWS ? (max_tile_h + EDGE_ROWS - 1) / EDGE_ROWS : 1);
+        dev, max_tile_h > EDGE_ROWS ? (max_tile_h + EDGE_ROWS - 1) / EDGE_ROWS : 1, lc.num_sms);
     return cudaGetLastError();
 }
 
