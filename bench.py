@@ -688,10 +688,7 @@ def run_ours(args, rank, world, local_rank):
                  "mean_before": float(e0.mean()), "mean_after": float(e1.mean()),
                  "median_before": float(e0.median()), "median_after": float(e1.median())}
         sor_ms = times[30] - times[0]
-        sor_bytes = 48.0 * p0.P * 5 * 30   # per SOR iteration and pixel: flow, update, coefficients
         refine = {"pair": f"{p0.W}x{p0.H}", "ms": times[30], "sor_ms": sor_ms,
-                  "sor_algorithmic_bytes": sor_bytes,
-                  "sor_achieved_gbs": sor_bytes / (sor_ms / 1e3) / 1e9 if sor_ms > 0 else None,
                   "launches": 1, "aee_interpolated": aee0, "aee_refined": aee1,
                   "from_perturbed_gt": basin}
         reng.close()

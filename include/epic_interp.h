@@ -164,9 +164,9 @@ typedef struct {
  *   0: a CTA solves a tile with its apron by directional sweeps, lines cut
  *      into segments so every thread of the CTA has one;
  *   1: the same, a thread sweeping whole lines;
- *   2: a warp solves a tile of 64 x tile_h (tile_h 1..32, apron 0) by down
- *      and up passes over its rows, each row taking the three candidates of
- *      the row before it and then closed along itself (the default). */
+ *   2: a CTA solves a tile of 64 x tile_h (tile_h 1..32, apron 0), or two of
+ *      a column as one where there are many, with 4 x 4 pixels a thread in
+ *      registers: distances, then labels (the default; "warp tiles" here). */
 typedef struct {
     long long max_pixels;
     int tile_w, tile_h, apron;

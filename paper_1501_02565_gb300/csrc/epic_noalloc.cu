@@ -29,8 +29,7 @@ using epic::pkey_t;
 constexpr int NA_MAX_PIXELS = 1 << 19;   // e.g. 1024 x 512
 constexpr int NA_MAX_MATCHES = 1 << 15;
 constexpr int NA_MAX_TILES = 1 << 14;    // of 64 x 32 pixels
-// Tiles of 64 x 16 pixels, what the tile autotuner picks for frames above
-// 64 K pixels: a call for 1024 x 436 takes 366 us by 64 x 32 apron tiles and
+// Tiles of 64 x 16 pixels, the interpolator's default: a call for 1024 x 436 takes 366 us by 64 x 32 apron tiles and
 // three argument copies, 219 us by these and one (timed in turn; k_relax.cu,
 // its distance unit held at 2^-31, so that what this entry point refuses and
 // how it rounds do not depend on the frame).

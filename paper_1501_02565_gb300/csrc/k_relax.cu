@@ -42,15 +42,17 @@
 // -> 328 us, the call 880 -> 802).
 // Carrying labels through every round of the first two phases instead makes
 // each of their steps five times as expensive (see relax_dist.cuh): that form
-// took 5.8 ms for the 64-pair mixed batch, this one 4.07 ms.  The form before,
+// took 5.8 ms for the 64-pair mixed batch, this one 4.17 ms.  The form before,
 // one warp stepping through the rows of a 64 x 16 tile and closing each along
-// itself, ran ~118 dependent row steps per fresh tile and took 4.28 ms for the
+// itself, ran ~118 dependent row steps per fresh tile and took 4.35 ms for the
 // batch; on single frames, where the chain of solves from tile to tile counts,
-// it took 503 us on a 1024 x 436 pair, 366 us on 1242 x 375 and 618 us on
-// 2048 x 1024 against 230, 123 and 218 us now.  What bounds it now: latency
-// (12 warps per SM at 168 registers, 26 % of the issue slots: barriers in the
-// CTA 31 % of the stalls, L2 loads 14 %, instruction fetch 14 %, dependent
-// integer steps 13 %).
+// it took 199 us on a 256 x 128 pair, 308 us on 1024 x 436, 365 us on 1242 x 375
+// and 549 us on 2048 x 1024 against 90, 147, 137 and 214 us now (the stage's
+// events in turn).  What bounds it now: latency (12 warps per SM at 168
+// registers, 26 % of the issue slots: barriers in the CTA 31 % of the stalls, L2
+// loads 14 %, instruction fetch 14 %, dependent integer steps 13 %).  The
+// settling sets the registers and spills ~200 bytes of stores and ~300 of loads
+// at them; the distances alone need no spill.
 //
 // Within a phase, and from fresh to spread, nothing waits for the whole grid:
 // a second-half tile waits for its four edge neighbours' stamps, and a spread

@@ -8,7 +8,7 @@ run (20 with --prune).
 --what gradcost: the image-gradient cost map of `--batch` synthetic frames,
 one launch per run.
 --what refine: the variational refinement of the first pair's interpolated
-flow (one interpolation run first), 5 x (3 + 10) launches per run.
+flow (one interpolation run first), one launch per run.
 
 Nothing else launches kernels of the library, so a profiler can skip the
 warm-up launches by count and capture the runs that follow.
@@ -94,7 +94,7 @@ def _other(args):
         eng.refine(I1, I2, f)
     torch.cuda.synchronize()
     eng.close()
-    print("1 pair, 7 interpolation launches, then 5 x (3 + 10) refinement launches per run")
+    print("1 pair, 10 interpolation launches, then 1 refinement launch per run")
     return 0
 
 

@@ -17,8 +17,8 @@ from __future__ import annotations
 import json
 import os
 
-# (tile_w, tile_h, apron, sweep).  sweep 2: the row-closure passes on warp
-# tiles of 64 x tile_h (the interpolator's default relaxation); the library
+# (tile_w, tile_h, apron, sweep).  sweep 2: tiles of 64 x tile_h solved in
+# registers (the interpolator's default relaxation); the library
 # uses them only when every rule asks for them, so a rule set is tuned from
 # one family at a time.
 CANDIDATES = ((64, 32, 0, 2), (64, 16, 0, 2), (64, 12, 0, 2), (64, 8, 0, 2))
