@@ -44,17 +44,18 @@
 // only where it decides.  Lanes find the batch node that owns their edge from
 // the ranges' starts as a bit mask and a popcount.
 //
-// What bounds it: instruction issue (73 % of the slots, 11 K warp
+// What bounds it: instruction issue (73 % of the slots, 10 K warp
 // instructions per search of K = 100: 15 steps, 23 groups of 32 edges).  The
-// 64-pair mixed batch takes 5.38 ms, 2048 x 1024 299 us; with the rows loaded
-// when a batch is settled, keys of 64 bits in the frontier, the frontier read
-// twice in the last steps and the owner searched by shuffles 5.74 ms and 314
-// us.  Rows held beside the settled list instead of in it cost 128 bytes a warp
-// and with them table space: 5.57 ms and a quarter more for the second launch.
-// A batch of one is found and settled in one look at the frontier, which is not
-// compacted for it: with the second launch 5.57 -> 5.20 ms for the batch (a
-// batch cut to one key ends many searches), 1024 x 436 with half its costs zero,
-// 1200 matches, K = 100, 11.0 -> 7.5 ms and less.
+// two launches take 5.20 ms for the 64-pair mixed batch and 384 us for a 2048 x
+// 1024 pair.  With the rows loaded when a batch is settled, keys of 64 bits in
+// the frontier, the frontier read twice in the last steps and the owner searched
+// by shuffles they took 5.95 ms and 438 us; with a batch of one cut out of the
+// frontier like any other 5.57 ms and 420 us (a batch cut to one key ends many
+// searches), and 1024 x 436 with half its costs zero, 1200 matches, K = 100, 11.0
+// instead of 7.5 ms: it is found and settled in one look at the frontier, which
+// is not compacted for it.  Rows held beside the settled list instead of in it
+// cost 128 bytes a warp and with them table space: the main launch 0.2 ms, the
+// second a quarter more.
 //
 // The fit uses centred coordinates x~ = p_n - p_m and fits the flow
 // u = p' - p (the same least-squares problem as fitting p', Eq. 2, with

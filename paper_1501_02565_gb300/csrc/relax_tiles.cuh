@@ -223,7 +223,8 @@ constexpr unsigned long long IDLE_LIMIT_NS = 2000000000ull;  // 2 s
 // a write, a fence, an add and the owner's next look.  (A shared queue of
 // tiles cost three more round trips to the L2 per solve, and, serving tiles
 // in the order of their requests rather than in turns, 6.7 solves per tile
-// where turns take ~3.7 on a batch.)
+// where turns and that test take 3.6 on the 64-pair mixed batch, after the
+// first.)
 //
 // solve(P, lt, tx, ty) stages and solves a tile, writes its changed keys and
 // returns what it did (TB_*; 0: nothing changed), the same in every thread.
