@@ -35,7 +35,9 @@ namespace {
 
 constexpr int GROUP = 8;               // a CTA's pixels: GROUP x GROUP
 constexpr float GROUP_RADIUS = 5.66f;  // farthest pixel from its centre pixel
-constexpr int CAND = 512;              // candidates of a group in shared memory
+constexpr int CAND_BITS = 9;
+constexpr int CAND = 1 << CAND_BITS;   // candidates of a group in shared memory
+static_assert(LABEL_BITS + CAND_BITS <= 32, "a match and a place in a word");
 constexpr int BIN_CELLS = 8192;
 constexpr int BIN_THREADS = 1024;
 constexpr float FAR = 2040.f;          // beyond: squared distances leave a packed key
@@ -163,8 +165,13 @@ __device__ __forceinline__ Cand cand_of(float4 q) {
 // at j * EXACT_THREADS + t), then the candidates, first as they are selected,
 // then as they are fitted.
 struct Select {
-    unsigned long long key[CAND];   // distance from the centre << 32 | match (or list position)
-    float2 xy[CAND];                // Euclidean: source pixels, in key order
+    // distance from the centre << 32 | match (geodesic: match << 9 | place as
+    // gathered): equal distances (frames of cost zero, matches on one pixel) come
+    // in the order that the insertions below want (as gathered, which is any
+    // order, 1024 x 436 of cost zero, 300 matches, K = 200: 59 ms; so: 21)
+    unsigned long long key[CAND];
+    float2 xy[CAND];                // Euclidean: source pixels, in key order; geodesic: the distance
+                                    // tiles in y, as gathered
     int slot[CAND];                 // geodesic: distance tiles, in key order
     unsigned short id[CAND];        // rank of the match index among the candidates, in key order
 };
@@ -337,7 +344,9 @@ __global__ void __launch_bounds__(EXACT_THREADS) fit_kernel(ExactArgs x, int gro
                 const int at = atomicAdd(&s_n, 1);
                 if (at < CAND) {
                     const float d = __ldg(x.slots + (size_t)ent.y * SINGLE_TILE + coff);
-                    w.s.key[at] = ((unsigned long long)__float_as_uint(d) << 32) | (unsigned)(e - e0);
+                    w.s.key[at] = ((unsigned long long)__float_as_uint(d) << 32) |
+                                  ((unsigned)ent.x << CAND_BITS) | (unsigned)at;
+                    w.s.xy[at].y = __int_as_float(ent.y);
                 }
             }
         }
@@ -353,12 +362,8 @@ __global__ void __launch_bounds__(EXACT_THREADS) fit_kernel(ExactArgs x, int gro
     __syncthreads();
     // ---- ranks of the match indices (ties go to the smaller index)
     if constexpr (GEO) {
-        const int2 *ent = x.tile_entry + __ldg(x.tile_start + (gy / 32) * x.tiles_x + gx / 64);
-        for (int i = t; i < n; i += EXACT_THREADS) {
-            const int2 e = __ldg(ent + (unsigned)w.s.key[i]);
-            w.s.slot[i] = e.y;
-            w.s.xy[i].x = __int_as_float(e.x);   // (the match, for the ranks)
-        }
+        for (int i = t; i < n; i += EXACT_THREADS)
+            w.s.slot[i] = __float_as_int(w.s.xy[(unsigned)w.s.key[i] & (CAND - 1)].y);
     } else {
         for (int i = t; i < n; i += EXACT_THREADS) {
             const float4 q = __ldg(x.matches + (unsigned)w.s.key[i]);
@@ -367,7 +372,7 @@ __global__ void __launch_bounds__(EXACT_THREADS) fit_kernel(ExactArgs x, int gro
     }
     __syncthreads();
     for (int i = t; i < n; i += EXACT_THREADS) {
-        auto index = [&](int j) { return GEO ? __float_as_int(w.s.xy[j].x) : (int)(unsigned)w.s.key[j]; };
+        auto index = [&](int j) { return (int)((unsigned)w.s.key[j] >> (GEO ? CAND_BITS : 0)); };
         const int m = index(i);
         int r = 0;
         for (int j = 0; j < n; ++j) r += index(j) < m;

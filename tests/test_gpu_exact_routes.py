@@ -49,6 +49,45 @@ def test_lists_hold_the_single_match_maps(kind, H, W, N, K, budget):
     assert torch.equal(idx.reshape(-1, K).long(), order[:, :K])
 
 
+@pytest.mark.parametrize("H,W,N,K,pixels", [
+    (45, 70, 60, 20, 60),
+    (45, 70, 60, 60, 7),       # several matches on a pixel
+    (45, 70, 600, 30, 600),    # more candidates than shared memory holds
+    (301, 701, 300, 40, 300),
+])
+def test_equal_distances_go_by_index(H, W, N, K, pixels):
+    import torch
+    rng = np.random.Generator(np.random.PCG64(H + N + pixels))
+    xy = _spread(rng, H, W, pixels)[np.arange(N) % pixels]
+    C = torch.zeros(H, W, device="cuda")
+    eng = native.EpicInterp(0)
+    _, idx, dist = eng.exact(C, torch.from_numpy(_matches(rng, xy)).cuda(), K, 1.0, with_knn=True)
+    eng.close()
+    assert not dist.any()
+    assert torch.equal(idx.reshape(-1, K).long(), torch.arange(K, device="cuda").expand(H * W, K))
+
+
+def test_costs_of_zero_do_not_take_many_times_as_long():
+    # (59 ms against 17 when the candidates of a group came in any order)
+    import torch
+    rng = np.random.Generator(np.random.PCG64(9))
+    H, W, N, K = 436, 1024, 300, 200
+    M = torch.from_numpy(_matches(rng, _spread(rng, H, W, N))).cuda()
+    times = []
+    for c in (1e-3, 0.0):
+        C = torch.full((H, W), c, device="cuda")
+        eng = native.EpicInterp(0)
+        best = float("inf")
+        for _ in range(4):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            eng.exact(C, M, K, 1.0)
+            best = min(best, time.perf_counter() - t0)
+        eng.close()
+        times.append(best)
+    assert times[1] < 2 * times[0], times
+
+
 @pytest.mark.parametrize("N,K", [(10, 10), (100, 10), (600, 10)])
 def test_high_costs_do_not_take_many_times_as_long(N, K):
     # (by windows 85 ms against 2 ms for N = 100)
