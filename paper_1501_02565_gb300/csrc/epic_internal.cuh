@@ -450,15 +450,15 @@ struct SingleArgs {
     // the sum of the caps, in cost units; above the limit they reach far: every
     // solve carries 64-bit keys, or nothing is done at all
     float *cap_sum;
-    float cap_limit;
+    float cap_limit, cap_floor;
     bool far_returns;
     RunState *state;
 };
 // How the single-source runs of a frame of `tiles` tiles go (whole calls, on
 // frames of 96 x 96 to 1500 x 1000 pixels, 1 to 5000 matches, K = 8 to 100, costs
 // from 1e-3 to U(0, 1.99); by pairs is how all went before, and the rules leave
-// nothing slower than it but frames of cost zero throughout, up to 1.3 times, and
-// 100 matches on 1500 x 1000 with K = 100, 1.15 times):
+// nothing slower than it but large frames of cost zero throughout with many
+// matches, 1500 x 1000 and 700 matches 1.1 times):
 //   by tiles   a CTA takes whole matches (k_single.cu).
 //   by pairs   every match is a pseudo-pair of the apron tiles (k_dt.cu), all
 //              tiles of all matches spread over the GPU.
@@ -474,11 +474,24 @@ struct SingleArgs {
 // 11.8 ms, 150 matches 6.0 and 5.9, 500 matches 8.1 and 5.2; 1500 x 1000, 500
 // matches, K = 64, 92 and 114; costs up to 1.99, whose diagonal weights leave 32
 // bits, 300 x 200, 500 matches, K = 64, 6.8 and 9.0.
+// Where the budget for keys is short of a pool of every tile per CTA, matches that
+// touch more than their pools run a second time.  With single_outgrow() most do:
+// by pairs 1500 x 1000, constant cost 1e-3, 100 matches, K = 100, 34 ms, by tiles
+// 45 (K = 50, 22 and 28; K = 25, whose matches touch less, 15 and 11); 2048 x 1024
+// (1024 tiles), 130 matches, K = 60, 35 and 42, 200 matches, K = 100, 55 and 62, K
+// = 60, 37 and 37.  So do nearly all where every cost is zero, and the caps with
+// them (a mean below SINGLE_ZERO: they keep nothing out): 1500 x 1000, 300 matches,
+// K = 100, 52 and 70 ms; 1024 x 436 16 and 16; and, where few, with pools of every
+// tile too: 64 matches, K = 64, 17 and 22 ms; 1024 x 436, 32, K = 32, 4.6 and 5.7.
 __host__ __device__ constexpr float single_far(int K) { return 3.f + (float)K / 32.f; }   // mean cap
 __host__ __device__ constexpr bool single_few(long long N, long long tiles) { return 12 * N < tiles; }
 __host__ __device__ constexpr bool single_few_far(long long N, long long tiles) {
     return N < 512 || N < tiles;
 }
+__host__ __device__ constexpr bool single_outgrow(long long N, int K, long long tiles, long long pool) {
+    return pool < tiles && 4 * N < tiles && 5ll * K >= 2 * N;
+}
+constexpr float SINGLE_ZERO = 1.f / (1 << 20);
 int single_resident(int num_sms);   // CTAs resident at once
 cudaError_t launch_single(const SingleArgs &x, int ctas, cudaStream_t stream);
 cudaError_t launch_cap_sum(const pkey_t *cap, long long n, float *sum, cudaStream_t stream);

@@ -1422,8 +1422,8 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
         return r;
     };
     unsigned n_used = 0;
-    // (*far: the caps reach far, and nothing was done for it)
-    auto by_tiles = [&](bool far_returns, bool *far) -> int {
+    // (*away: the caps are a case for pairs, and nothing was done)
+    auto by_tiles = [&](bool far_returns, bool *away) -> int {
         // distance tiles: room for 16 per match to begin with (11 on the flow
         // workloads at K = 100); a run that needs more says how many
         unsigned long long want = std::min<unsigned long long>((unsigned long long)N * ST, 16ull * N + 1024);
@@ -1440,7 +1440,7 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
                 (e = cudaMemcpyAsync(&cap_sum, s.cap_sum, sizeof cap_sum, cudaMemcpyDeviceToHost, stream)) ||
                 (e = cudaStreamSynchronize(stream)))
                 return cuda_fail(h, e, "exact-variant relaxation");
-            if ((*far = far_returns && cap_sum > s.cap_limit)) return EPIC_OK;
+            if ((*away = far_returns && (cap_sum > s.cap_limit || cap_sum < s.cap_floor))) return EPIC_OK;
             n_used = n_done[0];
             if (n_done[2] > 0 && n_used <= s.slot_cap) {
                 // the matches left over, with pools of every tile
@@ -1554,9 +1554,10 @@ int epic_exact_interp(epic_interp_t *h, const float *cost_map, const float *matc
         return EPIC_OK;
     };
     s.cap_limit = epic::single_far(K) * (float)P;
+    s.cap_floor = pool < ST || 4LL * N < ST ? epic::SINGLE_ZERO * (float)P : 0.f;
     if ((e = epic::launch_cap_sum(vkeys, P, s.cap_sum, stream)))
         return cuda_fail(h, e, "exact-variant cap map");
-    bool pairs = epic::single_few(N, ST);
+    bool pairs = epic::single_few(N, ST) || epic::single_outgrow(N, K, ST, pool);
     if (!pairs) rc = by_tiles(epic::single_few_far(N, ST), &pairs);
     if (!rc && pairs) {
         rc = by_pairs();

@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(256) cap_sum_kernel(const pkey_t *cap, long lo
 __global__ void __launch_bounds__(ST, 384 / ST) single_kernel(SingleArgs x) {
     RunState *st = x.state;
     const bool far = *x.cap_sum > x.cap_limit;
-    if (get_status(st) != 0 || (far && x.far_returns)) return;
+    if (get_status(st) != 0 || (x.far_returns && (far || *x.cap_sum < x.cap_floor))) return;
     __shared__ SingleShared sh;
     __shared__ PairDev P;
     __shared__ int s_item, s_queued, s_touched, s_slot, s_seed, s_fresh;

@@ -26,12 +26,18 @@ pytestmark = pytest.mark.gpu
     ("wide", 97, 131, 520, 30, 0),
     ("high", 301, 700, 530, 60, 2 * 110 * 16384),   # pools that do not hold a match's tiles
     ("edges", 40, 70, 1, 1, 0),
+    # 17 pools of 64 of the 110 tiles, which most matches outgrow
+    ("edges", 301, 701, 20, 20, 10 * 110 * 16384),   # by pairs
+    ("edges", 301, 701, 20, 7, 10 * 110 * 16384),    # by tiles
+    ("zero", 301, 701, 60, 9, 10 * 110 * 16384),     # by pairs
+    ("zero", 301, 701, 24, 9, 0),
 ])
 def test_lists_hold_the_single_match_maps(kind, H, W, N, K, budget):
     import torch
     rng = np.random.Generator(np.random.PCG64(H + W + N))
     M = _matches(rng, _spread(rng, H, W, N))
-    C = torch.from_numpy(_cost(kind, rng, H, W)).cuda()
+    C = np.zeros((H, W), np.float32) if kind == "zero" else _cost(kind, rng, H, W)
+    C = torch.from_numpy(C).cuda()
     eng = native.EpicInterp(0, exact_chunk_bytes=budget)
     for _ in range(2):   # the second call finds the first one's buffers
         _, idx, dist = eng.exact(C, torch.from_numpy(M).cuda(), K, 1.0, with_knn=True)
@@ -86,6 +92,29 @@ def test_costs_of_zero_do_not_take_many_times_as_long():
         eng.close()
         times.append(best)
     assert times[1] < 2 * times[0], times
+
+
+@pytest.mark.parametrize("c", [0.0, 1e-3])
+def test_a_few_matches_more_than_there_are_full_pools(c):
+    # 85 pools of every tile fit the budget.  By tiles most of 100 matches outgrow
+    # theirs and run twice.
+    import torch
+    rng = np.random.Generator(np.random.PCG64(10))
+    H, W, K = 1000, 1500, 50
+    C = torch.full((H, W), c, device="cuda")
+    times = []
+    for N in (85, 100):
+        M = torch.from_numpy(_matches(rng, _spread(rng, H, W, N))).cuda()
+        eng = native.EpicInterp(0)
+        best = float("inf")
+        for _ in range(4):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            eng.exact(C, M, K, 1.0)
+            best = min(best, time.perf_counter() - t0)
+        eng.close()
+        times.append(best)
+    assert times[1] < 1.45 * times[0], times
 
 
 @pytest.mark.parametrize("N,K", [(10, 10), (100, 10), (600, 10)])
