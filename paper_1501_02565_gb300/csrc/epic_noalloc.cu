@@ -29,10 +29,10 @@ using epic::pkey_t;
 constexpr int NA_MAX_PIXELS = 1 << 19;   // e.g. 1024 x 512
 constexpr int NA_MAX_MATCHES = 1 << 15;
 constexpr int NA_MAX_TILES = 1 << 14;    // of 64 x 32 pixels
-// Tiles of 64 x 16 pixels, the interpolator's default: a call for 1024 x 436 takes 366 us by 64 x 32 apron tiles and
-// three argument copies, 219 us by these and one (timed in turn; k_relax.cu,
-// its distance unit held at 2^-31, so that what this entry point refuses and
-// how it rounds do not depend on the frame).
+// Tiles of 64 x 16 pixels, the interpolator's default: a call for 1024 x 436
+// takes 366 us by 64 x 32 apron tiles and three argument copies, 219 us by these
+// and one (timed in turn; k_relax.cu, its distance unit held at 2^-31, so that
+// what this entry point refuses and how it rounds do not depend on the frame).
 constexpr int NA_TILE_W = 64, NA_TILE_H = 16, NA_TILES = 2 * NA_MAX_TILES;
 
 // byte offsets inside the scratch array (each 256-byte aligned)
